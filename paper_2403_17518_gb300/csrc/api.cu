@@ -48,7 +48,8 @@ struct Plan {
     int pitch = 0;                     // row pitch of every window in a pool
     long long n_data = 0;
     long long cells_per_step_all = 0;  // padded cells of all shots
-    DevBuf d_shots, d_tiles, d_recs, d_slot_of, d_wav, d_infos, d_rtiles, d_xrecs, d_xrec_off;
+    DevBuf d_shots, d_tiles, d_recs, d_slot_of, d_wav, d_infos, d_rtiles, d_xrecs, d_xrec_off, d_sponge;
+    int nwz = 0;                       // row factors at the head of d_sponge, then the slots' column factors
 };
 
 }  // namespace
@@ -413,6 +414,14 @@ int get_plan(dhfwi_ctx *ctx, const dhfwi_geom *G) {
     if ((rc = upload(ctx, P.d_rtiles, P.rtiles, "receiver tile list"))) return rc;
     if ((rc = upload(ctx, P.d_xrecs, P.xrecs, "grown-region receiver table"))) return rc;
     if ((rc = upload(ctx, P.d_xrec_off, P.xrec_off, "grown-region receiver offsets"))) return rc;
+    // Sponge factors of the rows and of each slot's columns.
+    P.nwz = round_up(NZ, TZ) + 2 * HALO;
+    const size_t nwx = (size_t)ns * (pitch + 2 * HALO);
+    if ((rc = ensure(ctx, P.d_sponge, sizeof(float) * (P.nwz + nwx), "sponge tables"))) return rc;
+    launch_sponge_tables((const ShotDesc *)P.d_shots.p, ns, NZ, nb, pitch, (float *)P.d_sponge.p, P.nwz,
+                         (float *)P.d_sponge.p + P.nwz, 0);
+    CK(cudaGetLastError());
+    CK(cudaDeviceSynchronize());  // the call's stream may not wait for the default one
     P.hash = h;
     return DHFWI_OK;
 }
@@ -459,6 +468,8 @@ StepCommon common(dhfwi_ctx *ctx) {
     c.NZ = ctx->NZ;
     c.nb = ctx->g.nb;
     c.tflag = (unsigned *)ctx->status.p + TFLAG_WORD;
+    c.wz = (const float *)ctx->plan.d_sponge.p;
+    c.wx = c.wz + ctx->plan.nwz;
     if (ctx->plan.xinj) {
         c.xrecs = (const TileRec *)ctx->plan.d_xrecs.p;
         c.xrec_off = (const int *)ctx->plan.d_xrec_off.p;
@@ -468,7 +479,7 @@ StepCommon common(dhfwi_ctx *ctx) {
 
 // Tensor-map shape kinds: field pool with halo box, field pool cell box,
 // model array (4 copies) cell box.
-enum { MAP_POOL_HALO = 0, MAP_POOL_CELL = 1, MAP_MODEL = 2, MAP_POOL_HALO2 = 3, MAP_MODEL_HALO = 4 };
+enum { MAP_POOL_HALO = 0, MAP_POOL_CELL = 1, MAP_MODEL = 2, MAP_POOL_HALO2 = 3 };
 
 // The tensor map of one array for the TMA-staged kernels (cached).
 int tensor_map(dhfwi_ctx *ctx, const float *base, int kind, CUtensorMap *out) {
@@ -483,14 +494,14 @@ int tensor_map(dhfwi_ctx *ctx, const float *base, int kind, CUtensorMap *out) {
     const Plan &P = ctx->plan;
     cuuint64_t dims[3], strides[2];
     cuuint32_t box[3] = {TX, TZ, 1}, estr[3] = {1, 1, 1};
-    if (kind == MAP_POOL_HALO || kind == MAP_MODEL_HALO) {
+    if (kind == MAP_POOL_HALO) {
         box[0] = TX + 2 * HALO;
         box[1] = TZ + 2 * HALO;
     } else if (kind == MAP_POOL_HALO2) {
-        box[0] = TX + 2 * HALO2;
+        box[0] = U2PITCH;
         box[1] = TZ + 2 * HALO2;
     }
-    if (kind == MAP_MODEL || kind == MAP_MODEL_HALO) {
+    if (kind == MAP_MODEL) {
         dims[0] = ctx->pf;
         dims[1] = ctx->NZ;
         dims[2] = 4;
@@ -822,16 +833,15 @@ bool time_blocking(const dhfwi_ctx *ctx, int which) {
 }
 
 // Maps of a two-step forward launch (u^n with the doubled halo, D^n with
-// its ring, kappa with its ring).
+// its ring).
 int pair_maps(dhfwi_ctx *ctx, const FwdArgs &a, TileMaps *M) {
     int rc;
     if ((rc = tensor_map(ctx, a.u, MAP_POOL_HALO2, &M->m[0]))) return rc;
-    if ((rc = tensor_map(ctx, a.dd, MAP_POOL_HALO, &M->m[1]))) return rc;
-    return tensor_map(ctx, a.c.kap, MAP_MODEL_HALO, &M->m[2]);
+    return tensor_map(ctx, a.dd, MAP_POOL_HALO, &M->m[1]);
 }
 
 // Maps of a two-step adjoint launch (nu^{k+1} with the doubled halo, D_nu
-// with its ring, kappa with its ring; the image, a^{k-1} and a^{k-2}, which
+// with its ring; the image, a^{k-1} and a^{k-2}, which
 // the kernel only prefetches into L2).  A history step's map spans all
 // slots from its base: the spare pool at the history's end keeps it inside
 // the allocation.
@@ -839,7 +849,6 @@ int adj_pair_maps(dhfwi_ctx *ctx, const AdjArgs &b, TileMaps *M) {
     int rc;
     if ((rc = tensor_map(ctx, b.nu, MAP_POOL_HALO2, &M->m[0]))) return rc;
     if ((rc = tensor_map(ctx, b.dd, MAP_POOL_HALO, &M->m[1]))) return rc;
-    if ((rc = tensor_map(ctx, b.c.kap, MAP_MODEL_HALO, &M->m[2]))) return rc;
     if ((rc = tensor_map(ctx, b.g, MAP_POOL_CELL, &M->m[3]))) return rc;
     if ((rc = tensor_map(ctx, b.a, MAP_POOL_CELL, &M->m[4]))) return rc;
     return tensor_map(ctx, b.a2, MAP_POOL_CELL, &M->m[5]);
@@ -1276,7 +1285,7 @@ void dhfwi_destroy(dhfwi_ctx *ctx) {
     DevBuf *bufs[] = {&ctx->kap, &ctx->dkap, &ctx->status, &ctx->partial, &ctx->fields,
                       &ctx->ck, &ctx->abuf, &ctx->hist, &ctx->dtmp, &ctx->rtmp, &ctx->plan.d_shots, &ctx->plan.d_tiles,
                       &ctx->plan.d_recs, &ctx->plan.d_slot_of, &ctx->plan.d_wav, &ctx->plan.d_infos,
-                      &ctx->plan.d_rtiles, &ctx->plan.d_xrecs, &ctx->plan.d_xrec_off};
+                      &ctx->plan.d_rtiles, &ctx->plan.d_xrecs, &ctx->plan.d_xrec_off, &ctx->plan.d_sponge};
     for (DevBuf *b : bufs) release(*b);
     if (ctx->h_status) cudaFreeHost(ctx->h_status);
     if (ctx->h_partial) cudaFreeHost(ctx->h_partial);

@@ -79,6 +79,62 @@ __device__ __forceinline__ f2 lap8x2(const STile &s, const float2 *zc, int lzr, 
     return lap8x2_seg(reinterpret_cast<const float2 *>(&s[lzr + HALO][lxp]), zc);
 }
 
+// ---------------------------------------------------------------------------
+// Four adjacent columns of one row (16-byte shared and global accesses).
+// ---------------------------------------------------------------------------
+struct q4 {
+    f2 lo, hi;
+};
+__device__ __forceinline__ q4 ld4(const float *p) {
+    const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(p);
+    return q4{v.x, v.y};
+}
+__device__ __forceinline__ void st4(float *p, q4 v) { *reinterpret_cast<ulonglong2 *>(p) = make_ulonglong2(v.lo, v.hi); }
+__device__ __forceinline__ q4 add4(q4 a, q4 b) { return q4{add2(a.lo, b.lo), add2(a.hi, b.hi)}; }
+__device__ __forceinline__ q4 mul4(q4 a, q4 b) { return q4{mul2(a.lo, b.lo), mul2(a.hi, b.hi)}; }
+__device__ __forceinline__ q4 fma4(q4 a, q4 b, q4 c) { return q4{fma2(a.lo, b.lo, c.lo), fma2(a.hi, b.hi, c.hi)}; }
+
+// One ring of the difference-form D u (see lap8x2_seg): right, left, lower
+// and upper neighbours of two cells.
+__device__ __forceinline__ f2 lap_ring(f2 p, f2 m, f2 zp, f2 zm, f2 u) {
+    return add2(add2(sub2(p, u), sub2(m, u)), add2(sub2(zp, u), sub2(zm, u)));
+}
+
+// D u down a column of quads in a shared-memory tile of row pitch P, with
+// lap8x2_seg's operations in its order.  p points at the quad, four rows above
+// the first row; rows are taken in order, each row of the column read once.
+template <int P>
+struct LapColumn {
+    const float *p;
+    q4 c[9];  // the rows around the current one, as a ring
+    __device__ __forceinline__ explicit LapColumn(const float *p_) : p(p_) {
+#pragma unroll
+        for (int r = 0; r < 8; r++) c[r] = ld4(p + r * P);
+    }
+    // Row rr (a compile-time constant after unrolling): D u and u itself.
+    __device__ __forceinline__ q4 row(int rr, q4 &u) {
+        c[(rr + 8) % 9] = ld4(p + (rr + 8) * P);
+        auto z = [&](int k) { return c[(rr + 4 + k) % 9]; };
+        const float *r = p + (rr + 4) * P;
+        const q4 L = ld4(r - 4), R = ld4(r + 4), C = z(0);
+        u = C;
+        const float2 l0 = upk(L.lo), l1 = upk(L.hi), c0 = upk(C.lo), c1 = upk(C.hi), r0 = upk(R.lo), r1 = upk(R.hi);
+        // Pairs that start at odd columns: x-3, x-1, x+1, x+3, x+5.
+        const f2 b0 = pk2(l0.y, l1.x), b1 = pk2(l1.y, c0.x), b2 = pk2(c0.y, c1.x), b3 = pk2(c1.y, r0.x),
+                 b4 = pk2(r0.y, r1.x);
+        const f2 w1 = pk2(FD_C1, FD_C1), w2 = pk2(FD_C2, FD_C2), w3 = pk2(FD_C3, FD_C3), w4 = pk2(FD_C4, FD_C4);
+        f2 a = mul2(w4, lap_ring(R.lo, L.lo, z(4).lo, z(-4).lo, C.lo));
+        a = fma2(w3, lap_ring(b3, b0, z(3).lo, z(-3).lo, C.lo), a);
+        a = fma2(w2, lap_ring(C.hi, L.hi, z(2).lo, z(-2).lo, C.lo), a);
+        a = fma2(w1, lap_ring(b2, b1, z(1).lo, z(-1).lo, C.lo), a);
+        f2 e = mul2(w4, lap_ring(R.hi, L.hi, z(4).hi, z(-4).hi, C.hi));
+        e = fma2(w3, lap_ring(b4, b1, z(3).hi, z(-3).hi, C.hi), e);
+        e = fma2(w2, lap_ring(R.lo, C.lo, z(2).hi, z(-2).hi, C.hi), e);
+        e = fma2(w1, lap_ring(b3, b2, z(1).hi, z(-1).hi, C.hi), e);
+        return q4{a, e};
+    }
+};
+
 // Source injection into lane 0 / 1 of a when the cell is the source node.
 __device__ __forceinline__ f2 inject(f2 a, int i, int j, int sz, int sx, float q) {
     if (i == sz && (j == sx || j + 1 == sx)) {

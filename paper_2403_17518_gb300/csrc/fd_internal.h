@@ -90,6 +90,13 @@ struct StepCommon {
     // staged D_nu from them (nullable: no such lists, separate injection).
     const TileRec *xrecs = nullptr;
     const int *xrec_off = nullptr;
+    // Sponge factors by row and by window column (the factor of a cell is
+    // their product), zero outside the padded domain and from a window's
+    // width on: wz[i + HALO] for rows i from -HALO to the last tile's last
+    // row + HALO, wx[slot * (pitch + 2 HALO) + j + HALO] for columns j from
+    // -HALO to pitch + HALO - 1.
+    const float *wz = nullptr;
+    const float *wx = nullptr;
 };
 // Most grown-region receiver entries the two-step adjoint's shared-memory
 // list holds; plans with more use the separate injection pass.
@@ -185,14 +192,14 @@ int step_variants(int kind);
 int step_occupancy(int kind, int variant, int store_a);
 
 // Two-step (time-blocked) TMA forward kernel (fd_tma2.cu): steps n and n+1
-// of the tiles active at step n.  maps: 0 u^n (HALO2 box), 1 D^n (halo box),
-// 2 kappa (model halo box).
+// of the tiles active at step n.  maps: 0 u^n (HALO2 box), 1 D^n (halo box).
 constexpr int HALO2 = 2 * HALO;
+constexpr int U2PITCH = TX + 2 * HALO2 + 4;  // columns of its u^n box (shared-memory row pitch)
 void launch_fwd_pair(const FwdArgs &a, int ntiles, const TileMaps &maps, cudaStream_t s);
 int fwd_pair_occupancy();
 // Two-step adjoint (fd_tma2.cu): steps k and k-1 of the tiles active at step
-// k-1; maps: 0 nu^{k+1} (HALO2 box), 1 D_nu (halo box), 2 kappa (model halo
-// box).  Before it, launch_adj_inject adds kappa r^{k-1} (the data of step k,
+// k-1; maps: 0 nu^{k+1} (HALO2 box), 1 D_nu (halo box), 3 image, 4 a^{k-1}, 5
+// a^{k-2} (cell boxes).  Before it, launch_adj_inject adds kappa r^{k-1} (the data of step k,
 // receivers sharing a cell summed in order) to D_nu at the receiver cells of
 // the first nrtiles tiles listed in rtiles (tiles with receivers, by slot).
 void launch_adj_pair(const AdjArgs &a, int ntiles, const TileMaps &maps, cudaStream_t s);
@@ -242,6 +249,10 @@ void launch_bb_partials(const float *xk, const float *xp, const float *gk, const
                         double *partial, int nblocks, unsigned *mxbits, cudaStream_t s);
 void launch_update_model(const float *v, const float *dir, int nz, int nx, int mute_rows, float alpha, float vmin,
                          float vmax, unsigned *mxbits, float *vout, cudaStream_t s);
+
+// Sponge tables of a plan (StepCommon::wz, wx): the factors of sponge1.
+void launch_sponge_tables(const ShotDesc *shots, int n_shots, int NZ, int nb, int pitch, float *wz, int nwz,
+                          float *wx, cudaStream_t s);
 
 // One kernel whose bounded wait runs out (on a barrier nothing arrives at)
 // and sets *tflag, as a step kernel's timed-out wait does.

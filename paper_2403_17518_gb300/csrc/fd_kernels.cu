@@ -497,6 +497,28 @@ void launch_prep_model(const float *v, const float *dv, int rel, int nz, int nx,
 }
 
 // ---------------------------------------------------------------------------
+// Sponge tables of a plan (blockIdx.y = 0: rows, 1 + slot: that slot's columns)
+// ---------------------------------------------------------------------------
+__global__ void sponge_tables_kernel(const ShotDesc *__restrict__ shots, int NZ, int nb, int pitch,
+                                     float *__restrict__ wz, int nwz, float *__restrict__ wx) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool rows = blockIdx.y == 0;
+    const int len = rows ? nwz : pitch + 2 * HALO;
+    if (t >= len) return;
+    const int slot = (int)blockIdx.y - 1;
+    const int N = rows ? NZ : shots[slot].nxw;
+    const int i = t - HALO;
+    const float w = i >= 0 && i < N ? sponge1(i, N, nb) : 0.f;
+    (rows ? wz : wx + (long long)slot * len)[t] = w;
+}
+
+void launch_sponge_tables(const ShotDesc *shots, int n_shots, int NZ, int nb, int pitch, float *wz, int nwz,
+                          float *wx, cudaStream_t s) {
+    const int len = nwz > pitch + 2 * HALO ? nwz : pitch + 2 * HALO;
+    sponge_tables_kernel<<<dim3((len + 127) / 128, 1 + n_shots), 128, 0, s>>>(shots, NZ, nb, pitch, wz, nwz, wx);
+}
+
+// ---------------------------------------------------------------------------
 // Residual and misfit partial sums
 // ---------------------------------------------------------------------------
 __global__ void residual_kernel(const float *__restrict__ ds, const float *__restrict__ dobs,

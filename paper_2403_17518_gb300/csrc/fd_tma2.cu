@@ -1,24 +1,39 @@
-// Two-step (time-blocked) forward kernel for sm_103a: one launch advances
-// every active tile by the steps n and n+1 of the recurrence of Section 2.1
-// (Eq. 1, summed form, difference-form Laplacian; see fd_kernels.cu), so
-// u and D cross HBM once per two updates.
+// Two-step (time-blocked) forward and adjoint kernels for sm_103a: one launch
+// advances every active tile by two steps of the recurrence of Section 2.1
+// (Eq. 1, summed form; see fd_kernels.cu), so u and D cross HBM once per two
+// updates.
 //
-// Per 64 x 64 tile the TMA stages u^n with an 8-cell halo (80 x 80) and D^n
-// and kappa with a 4-cell ring (72 x 72).  Step n is computed on the tile
-// grown by the ring (36 column pairs x 72 rows, 9 rows per thread), giving
-// u^{n+1} and D^{n+1} on 72 x 72 in shared memory (zero outside the window:
-// the Dirichlet boundary); step n+1 is then computed on the core from them.
-// The ring cells are recomputed by each tile that needs them, so tiles
-// never exchange data within the launch; since they read D^n on their
-// neighbours' cells, D^{n+2} goes to a second pool.  Every cell goes through
-// the same floating-point operations in the same order as in the one-step
-// kernels, so the results are bit-identical.
+// Per 64 x 64 tile the TMA stages u^n with an 8-cell halo and D^n with a
+// 4-cell ring.  Step n is computed on the tile and its ring, giving
+// u^{n+1} in shared memory (zero outside the window: the Dirichlet boundary);
+// step n+1 is then computed on the core from it.  The ring cells are
+// recomputed by each tile that needs them (1024 per 4096, the corners, which
+// no stencil reaches, left out), so tiles never exchange data within the
+// launch; since they read D^n on their neighbours' cells, D^{n+2} goes to a
+// second pool.  Every cell goes through the same floating-point operations in
+// the same order as in the one-step kernels, so the results are bit-identical.
+//
+// Work split: an item is 4 columns x 4 rows.  The 256 items of the core
+// belong to warps 0-7, the 32 left and right ring items to warp 8, the 32 top
+// and bottom ones to warp 9: ten full warps in step n, and a core thread
+// advances the same 16 cells in both steps, so D^{n+1} only passes through the
+// thread's own 64 bytes of shared memory.  16-byte accesses take 1.9 shared
+// loads per update where two columns per thread took 5.7, and the tile takes
+// 41 instead of 57 instructions per update.  What bounds it: latency at 20
+// warps per SM (FMA pipe 42 % busy, DRAM 34 %).
+// Forward, 64 shots of 400 x 1200: 64.4 -> 58.8 us per launch (two columns x
+// 9 rows per thread, sponge factors and bounds tests computed per row -> this).
+//
+// Sponge: the factor is separable and depends on the distances to the padded
+// domain's edges only, so the plan holds it per row and per slot's column
+// (zero outside the domain, which also masks the cells out there); a tile that
+// the sponge reaches reads 4 + 4 factors per item and needs no bounds tests.
 //
 // Sources: injected at both steps (q^n, q^{n+1}), also on ring cells.
 // Receivers: sample n from u^{n+1} in shared memory, sample n+1 from the
-// pool after the tile's stores.  Checkpoints (u^n, D^n) at even n, segment
-// stores of a^n and a^{n+1} for the backward recompute.  Tiles of a shot
-// whose record ends at n+1 take step n only.
+// pool after the tile's stores.  Checkpoints (u^n, D^n) at even n, history or
+// segment stores of a^n and a^{n+1}.  Tiles of a shot whose record ends at n+1
+// take step n only.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -27,19 +42,31 @@
 namespace dhfwi {
 namespace {
 
-constexpr int E = TX + 2 * HALO;    // 72: core + ring
-constexpr int U2 = TX + 2 * HALO2;  // 80: u^n box
-static_assert(TX == TZ, "square tiles");
-typedef float UTile2[U2][U2];  // u^n: rows z0-8 .., cols x0-8 ..
-typedef float ETile[E][E];     // rows z0-4 .., cols x0-4 ..
-
-struct Fwd2Stage {
-    UTile2 u;
-    ETile d, k;
+constexpr int E = TX + 2 * HALO;     // 72: core + ring
+constexpr int U2R = TZ + 2 * HALO2;  // 80 rows of the u^n box
+static_assert(TX == TZ && TX == 64 && HALO == 4, "the item layout below");
+// Row pitches with 4 rows off a multiple of the 32 banks, so that the ring
+// items of one column of quads spread over them (u: box of 84 columns).
+constexpr int VP = 76;
+struct Pair2Stage {
+    float u[U2R][U2PITCH];  // u^n: rows z0-8 .., cols x0-8 ..
+    float d[E][E];          // D^n: rows z0-4 .., cols x0-4 ..
 };
-constexpr unsigned kFwd2StageBytes = sizeof(UTile2) + 2 * sizeof(ETile);
-static_assert(sizeof(Fwd2Stage) == kFwd2StageBytes && sizeof(Fwd2Stage) % 128 == 0, "stage layout");
-constexpr size_t kFwd2Smem = sizeof(Fwd2Stage) + 2 * sizeof(ETile) + sizeof(PipeTail);
+constexpr unsigned kPair2StageBytes = sizeof(float) * (U2R * U2PITCH + E * E);
+static_assert(sizeof(Pair2Stage) == kPair2StageBytes, "stage layout");
+static_assert(U2R * U2PITCH * 4 % 128 == 0 && E * E * 4 % 128 == 0, "TMA destinations stay 128-byte aligned");
+typedef float VTile[E][VP];  // u^{n+1}: rows z0-4 .., cols x0-4 ..
+// The stage's barrier and the descriptors of this tile, the next one (whose
+// loads the leader issues in the middle of this one) and the one after.
+struct PairTail {
+    unsigned long long bar[2];
+    TileInfo desc[3];
+};
+static_assert(sizeof(PairTail) % 16 == 0, "tail layout");
+// D^{n+1} of the core threads' cells between the steps (each thread its own
+// 4 x 16 bytes).
+typedef float4 DStash[4][256];
+constexpr size_t kPair2Smem = sizeof(Pair2Stage) + sizeof(VTile) + sizeof(DStash) + sizeof(PairTail);
 // The two-step adjoint's list of its next tile's data injection (grown
 // region, step k): offset of the cell in the staged D_nu (-1: a further
 // receiver of the cell before, already summed), kappa there, summed data.
@@ -51,146 +78,166 @@ struct InjBuf {
     int n, pad[3];
     InjEntry e[kInjCap];
 };
-constexpr size_t kAdj2Smem = kFwd2Smem + sizeof(InjBuf);
-static_assert(kFwd2Smem % 16 == 0, "injection list alignment");
-// Thread layout: 288 threads.  Step n covers the 72 x 72 grown tile with
-// 36 column pairs x 8 blocks of R1 = 9 rows; step n+1 covers the 64 x 64
-// core with the first 256 threads, 32 column pairs x 8 blocks of R2 = 8 rows.
-constexpr int NT2 = 288, R1 = 9, R2 = 8, PAIRS1 = E / 2;
-static_assert(PAIRS1 * (E / R1) == NT2 && (TX / 2) * (TZ / R2) == 256, "thread layout");
+constexpr size_t kAdj2Smem = kPair2Smem + sizeof(InjBuf);
+static_assert(kPair2Smem % 16 == 0, "injection list alignment");
+
+constexpr int NT2 = 320, NCORE = 256, R4 = 4;
+constexpr int LEADER = 288;  // first thread of warp 9, which is free during step n+1
+
+// Core-relative column and row of a thread's item.
+__device__ __forceinline__ void item_of(int tid, int &lx, int &lz) {
+    if (tid < NCORE) {
+        lx = 4 * (tid & 15);
+        lz = R4 * (tid >> 4);
+    } else if (tid < 288) {  // left and right alternately
+        lx = (tid & 1) ? TX : -HALO;
+        lz = R4 * ((tid & 31) >> 1);
+    } else {
+        lx = 4 * (tid & 15);
+        lz = (tid & 16) ? TZ : -HALO;
+    }
+}
+
+// Sponge factors of an item's rows, read from the plan's tables (L1 and L2
+// hits), and its source cell.
+struct ItemEdge {
+    const float *wz, *wx;
+    int src;  // 4 * row + column of the source inside the item, -1 without one
+    __device__ __forceinline__ ItemEdge(const StepCommon &c, const TileInfo &T, int lx, int lz) {
+        wz = c.wz + (T.z0 + lz + HALO);
+        wx = c.wx + ((long long)T.slot * (T.pitch + 2 * HALO) + T.x0 + lx + HALO);
+        const unsigned x = T.sx - (T.x0 + lx), z = T.sz - (T.z0 + lz);
+        src = x < 4u && z < (unsigned)R4 ? (int)(4 * z + x) : -1;
+    }
+    __device__ __forceinline__ q4 w(int rr) const {
+        const float z = __ldg(wz + rr);
+        const float4 x = __ldg(reinterpret_cast<const float4 *>(wx));
+        return q4{mul2(pk2(z, z), pk2(x.x, x.y)), mul2(pk2(z, z), pk2(x.z, x.w))};
+    }
+};
+// kappa of an item's row rr, from the L2-resident model array (both steps read
+// it there: staging it would cost 20 KB of shared memory).  Quads outside the
+// padded domain, whose sponge factor is zero, take some cell's inside it.
+template <bool FULL>
+struct ItemKappa {
+    const float *p;
+    int pf, i0, NZ;
+    __device__ __forceinline__ ItemKappa(const StepCommon &c, const TileInfo &T, int lx, int lz) {
+        pf = c.pf;
+        i0 = T.z0 + lz;
+        NZ = c.NZ;
+        const float *m = c.kap + (long long)T.mc * c.mstride;
+        if constexpr (FULL) p = m + (i0 * pf + T.mx + lx);
+        else p = m + min(max(T.mx + lx, 0), pf - 4);
+    }
+    __device__ __forceinline__ q4 row(int rr) const {
+        const float4 v = __ldg(reinterpret_cast<const float4 *>(
+            FULL ? p + rr * pf : p + min(max(i0 + rr, 0), NZ - 1) * pf));
+        return q4{pk2(v.x, v.y), pk2(v.z, v.w)};
+    }
+};
+__device__ __forceinline__ void add_source(q4 &a, int scol, float q) {
+    float2 l = upk(a.lo), h = upk(a.hi);
+    if (scol == 0) l.x += q;
+    if (scol == 1) l.y += q;
+    if (scol == 2) h.x += q;
+    if (scol == 3) h.y += q;
+    a = q4{pk(l), pk(h)};
+}
 
 // mid(): called by every thread after the barrier that ends step n (the
-// stage is no longer read; kappa of the core is in registers): the leader
-// refills the stage.
+// stage is no longer read): the leader refills the stage.
 template <bool STORE_A, bool FULL, class MidFn>
-__device__ __forceinline__ void pair_tile(const FwdArgs &A, const Fwd2Stage &S, ETile &V, ETile &Dn, const TileInfo &T,
-                                          int tid, bool two, MidFn mid) {
-    const int NZ = A.c.NZ, nb = A.c.nb, nxw = T.nxw, pitch = T.pitch, n = A.n;
-    float q0 = 0.f, q1 = 0.f;
-    if constexpr (!FULL) {
-        q0 = A.c.wav[T.wav_off + n];
-        q1 = two ? A.c.wav[T.wav_off + n + 1] : 0.f;
-    }
+__device__ __forceinline__ void pair_tile(const FwdArgs &A, const Pair2Stage &S, VTile &V, DStash &DS,
+                                          const TileInfo &T, int tid, bool two, MidFn mid) {
+    int lx, lz;
+    item_of(tid, lx, lz);
+    const bool core = tid < NCORE;
+    const int n = A.n, pitch = T.pitch;
+    const int j = T.x0 + lx, i0 = T.z0 + lz;
+    const int nrow = FULL ? R4 : A.c.NZ - i0;
+    const bool ok = core && (FULL || j < T.nxw);
+    const long long cbase = T.foff + (long long)i0 * pitch + j;
+    const ItemEdge ed(A.c, T, lx, lz);  // (unused where FULL)
+    const ItemKappa<FULL> kap(A.c, T, lx, lz);
 
-    // ---- step n on the grown tile -----------------------------------------
+    // ---- step n on the item ------------------------------------------------
     {
-        const int ex = 2 * (tid % PAIRS1), ez0 = R1 * (tid / PAIRS1);
-        const int jj = T.x0 - HALO + ex;  // window column of lane 0
-        const bool core_x = ex >= HALO && ex < TX + HALO;
-        float wx0 = 1.f, wx1 = 1.f;
-        bool c0ok = true, c1ok = true;
-        if constexpr (!FULL) {
-            c0ok = jj >= 0 && jj < nxw;
-            c1ok = jj + 1 >= 0 && jj + 1 < nxw;
-            wx0 = sponge1(jj, nxw, nb);
-            wx1 = sponge1(jj + 1, nxw, nb);
-        }
-        float2 zc[R1 + 2 * HALO];
+        LapColumn<U2PITCH> col(&S.u[lz + HALO][lx + HALO2]);
 #pragma unroll
-        for (int r = 0; r < R1 + 2 * HALO; r++) zc[r] = *reinterpret_cast<const float2 *>(&S.u[ez0 + r][ex + HALO]);
-#pragma unroll
-        for (int rr = 0; rr < R1; rr++) {
-            const int ez = ez0 + rr;
-            const int i = T.z0 - HALO + ez;
-            f2 a = lap8x2_seg(reinterpret_cast<const float2 *>(&S.u[ez + HALO][ex]), zc + rr);
-            const f2 u = pk(zc[rr + HALO]);
-            const f2 dv = pk(*reinterpret_cast<const float2 *>(&S.d[ez][ex]));
-            const f2 kv = pk(*reinterpret_cast<const float2 *>(&S.k[ez][ex]));
-            f2 dn, un;
-            bool v0 = true, v1 = true;
+        for (int rr = 0; rr < R4; rr++) {
+            q4 u;
+            q4 a = col.row(rr, u);
+            const q4 dv = ld4(&S.d[lz + rr + HALO][lx + HALO]);
+            const q4 kv = kap.row(rr);
+            q4 un, dn;
             if constexpr (FULL) {
-                dn = fma2(kv, a, dv);
-                un = add2(u, dn);
+                dn = fma4(kv, a, dv);
+                un = add4(u, dn);
             } else {
-                const bool rok = i >= 0 && i < NZ;
-                v0 = rok && c0ok;
-                v1 = rok && c1ok;
-                a = inject(a, i, jj, T.sz, T.sx, q0);
-                const float wz = sponge1(i, NZ, nb);
-                const f2 w = pk2(wz * wx0, wz * wx1);
-                dn = keep_lo(mul2(w, fma2(kv, a, dv)), v1);
-                un = keep_lo(fma2(w, u, dn), v1);
-                if (!v0) dn = un = 0ull;
+                if (rr == ed.src >> 2) add_source(a, ed.src & 3, A.c.wav[T.wav_off + n]);
+                const q4 w = ed.w(rr);
+                dn = mul4(w, fma4(kv, a, dv));
+                un = fma4(w, u, dn);
             }
-            *reinterpret_cast<f2 *>(&V[ez][ex]) = un;
-            *reinterpret_cast<f2 *>(&Dn[ez][ex]) = dn;
-            if (core_x && ez >= HALO && ez < TZ + HALO && v0) {
-                const long long c = T.foff + (long long)i * pitch + jj;
+            st4(&V[lz + rr + HALO][lx + HALO], un);
+            if (core) st4(&DS[rr][tid].x, dn);
+            if (ok && rr < nrow) {
+                const long long c = cbase + (long long)rr * pitch;
                 if (!STORE_A && A.ck_u) {
-                    *reinterpret_cast<f2 *>(A.ck_u + c) = keep_lo(u, v1);
-                    *reinterpret_cast<f2 *>(A.ck_d + c) = keep_lo(dv, v1);
+                    st4(A.ck_u + c, u);
+                    st4(A.ck_d + c, dv);
                 }
-                if constexpr (STORE_A) *reinterpret_cast<f2 *>(A.a_out + c) = keep_lo(a, v1);
+                if constexpr (STORE_A) st4(A.a_out + c, a);
             }
         }
     }
-    // kappa of this thread's core cells for step n+1; after the barrier the
-    // stage is no longer read and u^{n+1}, D^{n+1} are complete.
-    const int lxp = 2 * (tid % 32), lz0 = R2 * (tid / 32);
-    const bool worker = tid < 256;
-    f2 kv2[R2];
-#pragma unroll
-    for (int rr = 0; rr < R2; rr++)
-        kv2[rr] = worker ? *reinterpret_cast<const f2 *>(&S.k[lz0 + rr + HALO][lxp + HALO]) : 0ull;
-    __syncthreads();
+    __syncthreads();  // u^{n+1} complete; the stage is no longer read
     mid();
 
-    // Receivers: sample n is u^{n+1}.
-    if (A.d) {
-        for (int e = T.rec_begin + tid; e < T.rec_end; e += NT2) {
+    // Receivers: sample n is u^{n+1} (the ring warps, free from here on).
+    if (A.d && !core) {
+        for (int e = T.rec_begin + tid - NCORE; e < T.rec_end; e += NT2 - NCORE) {
             const TileRec tr = A.c.recs[e];
             A.d[T.doff + (long long)n * T.nrec + tr.r] = V[tr.cell / TX + HALO][tr.cell % TX + HALO];
         }
     }
 
-    // ---- step n+1 on the core (threads 0..255) ---------------------------------
-    const int j = T.x0 + lxp;
-    const int i0 = T.z0 + lz0;
-    const long long cbase = T.foff + (long long)i0 * pitch + j;
-    const int nrow = FULL ? R2 : min(R2, NZ - i0);
-    const bool ok = worker && (FULL || j < nxw), hi = FULL || j + 1 < nxw;
+    // ---- step n+1 on the core ----------------------------------------------
     if (!two) {  // the record ends at n+1: store u^{n+1}, D^{n+1}
 #pragma unroll
-        for (int rr = 0; rr < R2; rr++) {
+        for (int rr = 0; rr < R4; rr++) {
             if (ok && rr < nrow) {
                 const long long c = cbase + (long long)rr * pitch;
-                *reinterpret_cast<f2 *>(A.un + c) = *reinterpret_cast<const f2 *>(&V[lz0 + rr + HALO][lxp + HALO]);
-                *reinterpret_cast<f2 *>(A.dd_out + c) = *reinterpret_cast<const f2 *>(&Dn[lz0 + rr + HALO][lxp + HALO]);
+                st4(A.un + c, ld4(&V[lz + rr + HALO][lx + HALO]));
+                st4(A.dd_out + c, ld4(&DS[rr][tid].x));
             }
         }
         return;
     }
-    if (worker) {
-        float wx0 = 1.f, wx1 = 1.f;
-        if constexpr (!FULL) {
-            wx0 = sponge1(j, nxw, nb);
-            wx1 = sponge1(j + 1, nxw, nb);
-        }
-        float2 zc[R2 + 2 * HALO];
+    if (ok) {
+        LapColumn<VP> col(&V[lz][lx + HALO]);
 #pragma unroll
-        for (int r = 0; r < R2 + 2 * HALO; r++) zc[r] = *reinterpret_cast<const float2 *>(&V[lz0 + r][lxp + HALO]);
-#pragma unroll
-        for (int rr = 0; rr < R2; rr++) {
-            if (!(ok && rr < nrow)) continue;
-            f2 a = lap8x2_seg(reinterpret_cast<const float2 *>(&V[lz0 + rr + HALO][lxp]), zc + rr);
-            if constexpr (!FULL) a = inject(a, i0 + rr, j, T.sz, T.sx, q1);
-            const f2 u = pk(zc[rr + HALO]);
-            const f2 kv = kv2[rr];
-            const f2 d1 = *reinterpret_cast<const f2 *>(&Dn[lz0 + rr + HALO][lxp + HALO]);
-            f2 dn, un;
+        for (int rr = 0; rr < R4; rr++) {
+            q4 u;
+            q4 a = col.row(rr, u);
+            const q4 kv = kap.row(rr), dn = ld4(&DS[rr][tid].x);
+            q4 d2, un;
             if constexpr (FULL) {
-                dn = fma2(kv, a, d1);
-                un = add2(u, dn);
+                d2 = fma4(kv, a, dn);
+                un = add4(u, d2);
             } else {
-                const float wz = sponge1(i0 + rr, NZ, nb);
-                const f2 w = pk2(wz * wx0, wz * wx1);
-                dn = keep_lo(mul2(w, fma2(kv, a, d1)), hi);
-                un = keep_lo(fma2(w, u, dn), hi);
+                if (rr == ed.src >> 2) add_source(a, ed.src & 3, A.c.wav[T.wav_off + n + 1]);
+                const q4 w = ed.w(rr);
+                d2 = mul4(w, fma4(kv, a, dn));
+                un = fma4(w, u, d2);
             }
-            const long long c = cbase + (long long)rr * pitch;
-            *reinterpret_cast<f2 *>(A.dd_out + c) = dn;
-            *reinterpret_cast<f2 *>(A.un + c) = un;
-            if constexpr (STORE_A) *reinterpret_cast<f2 *>(A.a_out2 + c) = keep_lo(a, hi);
+            if (rr < nrow) {
+                const long long c = cbase + (long long)rr * pitch;
+                st4(A.dd_out + c, d2);
+                st4(A.un + c, un);
+                if constexpr (STORE_A) st4(A.a_out2 + c, a);
+            }
         }
     }
     // Receivers: sample n+1 is u^{n+2}, read back from the pool.
@@ -198,21 +245,21 @@ __device__ __forceinline__ void pair_tile(const FwdArgs &A, const Fwd2Stage &S, 
 }
 
 // Tile loop: one stage, refilled in the middle of a tile (see mid() in
-// pair_tile) so that the next tile's loads overlap step n+1; the descriptor
-// slot is refilled at the end of the tile.  Waits bounded as in run_tiles.
+// pair_tile) so that the next tile's loads overlap step n+1; the barrier that
+// opens a tile also certifies that every thread is done with the tile before
+// (V, and the descriptor slot, which alternates).  Waits bounded as in
+// run_tiles.
 template <bool STORE_A>
 __global__ void __launch_bounds__(NT2, 2) fwd_pair_kernel(FwdArgs A, const __grid_constant__ TileMaps M, int ntiles) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    Fwd2Stage &S = *reinterpret_cast<Fwd2Stage *>(smem_raw);
-    ETile &V = *reinterpret_cast<ETile *>(smem_raw + sizeof(Fwd2Stage));
-    ETile &Dn = *reinterpret_cast<ETile *>(smem_raw + sizeof(Fwd2Stage) + sizeof(ETile));
-    PipeTail *tail = reinterpret_cast<PipeTail *>(smem_raw + sizeof(Fwd2Stage) + 2 * sizeof(ETile));
+    Pair2Stage &S = *reinterpret_cast<Pair2Stage *>(smem_raw);
+    VTile &V = *reinterpret_cast<VTile *>(smem_raw + sizeof(Pair2Stage));
+    DStash &DS = *reinterpret_cast<DStash *>(smem_raw + sizeof(Pair2Stage) + sizeof(VTile));
+    PairTail *tail = reinterpret_cast<PairTail *>(smem_raw + sizeof(Pair2Stage) + sizeof(VTile) + sizeof(DStash));
     const int tid = threadIdx.x + threadIdx.y * 32;
-    const bool leader = tid == 0;
+    const bool leader = tid == LEADER;
     const unsigned bar = smem_u32(&tail->bar[0]);
     const int b = blockIdx.x, g = gridDim.x;
-    int4 co = make_int4(0, 0, 0, 0);
-    int mc = 0;
     if (smem_u32(&S) & 127u) {
         if (leader) atomicExch(A.c.tflag, 2u);
         return;
@@ -220,24 +267,22 @@ __global__ void __launch_bounds__(NT2, 2) fwd_pair_kernel(FwdArgs A, const __gri
     if (leader) {
         mbar_init(bar, 1);
         fence_mbar_init();
-        fetch_coords(A.c.infos, b, co, mc);
         copy_desc(&tail->desc[0], &A.c.infos[b]);
+        if (b + g < ntiles) copy_desc(&tail->desc[1], &A.c.infos[b + g]);
+        cp_async_wait_all();
     }
     griddep_wait();
     griddep_launch_dependents();
-    auto issue = [&]() {
+    auto issue = [&](const TileInfo &N) {
         fence_proxy_async();
-        mbar_expect_tx(bar, kFwd2StageBytes);
-        tma_load_3d(smem_u32(&S.u), &M.m[0], co.z - HALO2, co.y - HALO2, co.x, bar);
-        tma_load_3d(smem_u32(&S.d), &M.m[1], co.z - HALO, co.y - HALO, co.x, bar);
-        tma_load_3d(smem_u32(&S.k), &M.m[2], co.w - HALO, co.y - HALO, mc, bar);
+        mbar_expect_tx(bar, kPair2StageBytes);
+        tma_load_3d(smem_u32(&S.u), &M.m[0], N.x0 - HALO2, N.z0 - HALO2, N.slot, bar);
+        tma_load_3d(smem_u32(&S.d), &M.m[1], N.x0 - HALO, N.z0 - HALO, N.slot, bar);
     };
-    if (leader) {
-        issue();
-        if (b + g < ntiles) fetch_coords(A.c.infos, b + g, co, mc);
-    }
+    if (leader) issue(tail->desc[0]);
     __syncthreads();
     unsigned phase = 0;
+    int slot = 0, next = 1;
     for (int tix = b; tix < ntiles; tix += g) {
         const bool landed = mbar_wait(bar, phase);
         phase ^= 1u;
@@ -249,168 +294,139 @@ __global__ void __launch_bounds__(NT2, 2) fwd_pair_kernel(FwdArgs A, const __gri
             }
             return;
         }
-        const bool more = tix + g < ntiles;
         auto mid = [&]() {  // after a barrier: every thread is done with the stage
-            if (leader && more) issue();
+            if (leader && tix + g < ntiles) {
+                issue(tail->desc[next]);
+                if (tix + 2 * g < ntiles) copy_desc(&tail->desc[3 - slot - next], &A.c.infos[tix + 2 * g]);
+            }
         };
-        const TileInfo &T = tail->desc[0];
+        const TileInfo &T = tail->desc[slot];
         const bool two = T.nt > A.n + 1;
-        if ((T.flags & TI_FULL2) && two) pair_tile<STORE_A, true>(A, S, V, Dn, T, tid, true, mid);
-        else pair_tile<STORE_A, false>(A, S, V, Dn, T, tid, two, mid);
-        __syncthreads();  // the descriptor, V and Dn are free
-        if (leader && more) {
-            copy_desc(&tail->desc[0], &A.c.infos[tix + g]);
-            if (tix + 2 * g < ntiles) fetch_coords(A.c.infos, tix + 2 * g, co, mc);
-        }
+        if (T.flags & TI_FULL2) pair_tile<STORE_A, true>(A, S, V, DS, T, tid, two, mid);
+        else pair_tile<STORE_A, false>(A, S, V, DS, T, tid, two, mid);
+        const int after = 3 - slot - next;
+        slot = next;
+        next = after;
     }
 }
 
 // ---------------------------------------------------------------------------
 // Two-step adjoint: steps k (nu^{k+1} -> nu^k) and k-1 in one launch, the
 // same layout and stage refill as fwd_pair_kernel.  The data of step k are
-// already in the staged D_nu (D' = D + kappa r^{k-1}, launch_adj_inject, so
-// ring cells need no injection tile); the data of step k-1 are added to the
-// core's D_nu^k in shared memory after step k.  The image accumulator takes
-// a^{k-1} nu^k (tiles whose record reaches step k) and then a^{k-2} nu^{k-1},
-// in that order, as two one-step launches would.
+// added to the staged D_nu (inject_here) or already in it (D' = D + kappa
+// r^{k-1}, launch_adj_inject); the data of step k-1 are added to the core's
+// D_nu^k after step k.  The image accumulator
+// takes a^{k-1} nu^k (tiles whose record reaches step k) and then a^{k-2}
+// nu^{k-1}, in that order, as two one-step launches would.
 // ---------------------------------------------------------------------------
 template <bool FULL, class MidFn>
-__device__ __forceinline__ void adj_pair_tile(const AdjArgs &A, const Fwd2Stage &S, ETile &V, ETile &Dn,
+__device__ __forceinline__ void adj_pair_tile(const AdjArgs &A, Pair2Stage &S, VTile &V, DStash &DS,
                                               const TileInfo &T, int tid, MidFn mid) {
-    const int NZ = A.c.NZ, nb = A.c.nb, nxw = T.nxw, pitch = T.pitch, k = A.k;
+    int lx, lz;
+    item_of(tid, lx, lz);
+    const bool core = tid < NCORE;
+    const int k = A.k, pitch = T.pitch;
+    const int j = T.x0 + lx, i0 = T.z0 + lz;
+    const int nrow = FULL ? R4 : A.c.NZ - i0;
+    const bool ok = core && (FULL || j < T.nxw);
+    const long long cbase = T.foff + (long long)i0 * pitch + j;
+    const ItemEdge ed(A.c, T, lx, lz);  // (unused where FULL)
+    const ItemKappa<FULL> kap(A.c, T, lx, lz);
 
-    // ---- step k on the grown tile -------------------------------------------
+    // ---- step k on the item --------------------------------------------------
     {
-        const int ex = 2 * (tid % PAIRS1), ez0 = R1 * (tid / PAIRS1);
-        const int jj = T.x0 - HALO + ex;
-        float wx0 = 1.f, wx1 = 1.f;
-        bool c0ok = true, c1ok = true;
-        if constexpr (!FULL) {
-            c0ok = jj >= 0 && jj < nxw;
-            c1ok = jj + 1 >= 0 && jj + 1 < nxw;
-            wx0 = sponge1(jj, nxw, nb);
-            wx1 = sponge1(jj + 1, nxw, nb);
-        }
-        float2 zc[R1 + 2 * HALO];
+        LapColumn<U2PITCH> col(&S.u[lz + HALO][lx + HALO2]);
 #pragma unroll
-        for (int r = 0; r < R1 + 2 * HALO; r++) zc[r] = *reinterpret_cast<const float2 *>(&S.u[ez0 + r][ex + HALO]);
-#pragma unroll
-        for (int rr = 0; rr < R1; rr++) {
-            const int ez = ez0 + rr;
-            const int i = T.z0 - HALO + ez;
-            const f2 a = lap8x2_seg(reinterpret_cast<const float2 *>(&S.u[ez + HALO][ex]), zc + rr);
-            const f2 nu = pk(zc[rr + HALO]);
-            const f2 dv = pk(*reinterpret_cast<const float2 *>(&S.d[ez][ex]));
-            const f2 kv = pk(*reinterpret_cast<const float2 *>(&S.k[ez][ex]));
-            f2 dn, nn;
+        for (int rr = 0; rr < R4; rr++) {
+            q4 nu;
+            const q4 a = col.row(rr, nu);
+            const q4 dv = ld4(&S.d[lz + rr + HALO][lx + HALO]);
+            const q4 kv = kap.row(rr);
+            q4 nn, dn;
             if constexpr (FULL) {
-                dn = fma2(kv, a, dv);
-                nn = add2(nu, dn);
+                dn = fma4(kv, a, dv);
+                nn = add4(nu, dn);
             } else {
-                const bool rok = i >= 0 && i < NZ;
-                const bool v0 = rok && c0ok, v1 = rok && c1ok;
-                const float wz = sponge1(i, NZ, nb);
-                const f2 w = pk2(wz * wx0, wz * wx1);
-                dn = keep_lo(mul2(w, fma2(kv, a, dv)), v1);
-                nn = keep_lo(fma2(w, nu, dn), v1);
-                if (!v0) dn = nn = 0ull;
+                const q4 w = ed.w(rr);
+                dn = mul4(w, fma4(kv, a, dv));
+                nn = fma4(w, nu, dn);
             }
-            *reinterpret_cast<f2 *>(&V[ez][ex]) = nn;
-            *reinterpret_cast<f2 *>(&Dn[ez][ex]) = dn;
+            st4(&V[lz + rr + HALO][lx + HALO], nn);
+            if (core) st4(&DS[rr][tid].x, dn);
         }
     }
-    const int lxp = 2 * (tid % 32), lz0 = R2 * (tid / 32);
-    const bool worker = tid < 256;
-    const int j = T.x0 + lxp;
-    const int i0 = T.z0 + lz0;
-    const long long cbase = T.foff + (long long)i0 * pitch + j;
-    const int nrow = FULL ? R2 : min(R2, NZ - i0);
-    const bool ok = worker && (FULL || j < nxw), hi = FULL || j + 1 < nxw;
-    // Global operands of the second step (image accumulator, a^{k-1},
-    // a^{k-2}; prefetched into L2 a tile ahead) kept PF rows ahead of the
-    // arithmetic, the first rows requested before the barrier.  a^{k-1}
-    // exists only where the record reaches step k (a stored history holds
-    // the shots active at each step only).
+    // The image and the background terms of the second step (prefetched into
+    // L2 a tile ahead), a row ahead of the arithmetic, the first requested
+    // before the barrier.  a^{k-1} exists only where the record reaches step
+    // k (a stored history holds the shots active at each step only).
     const bool image_k = T.nt > k - 1;
-    constexpr int PF = 2;
-    f2 gq[PF], a1q[PF], a2q[PF];
-    auto fetch = [&](int rr, int q) {
-        const bool v = ok && rr < nrow;
-        const long long c = cbase + (long long)rr * pitch;
-        gq[q] = v ? *reinterpret_cast<const f2 *>(A.g + c) : 0ull;
-        a1q[q] = v && image_k ? *reinterpret_cast<const f2 *>(A.a + c) : 0ull;
-        a2q[q] = v ? *reinterpret_cast<const f2 *>(A.a2 + c) : 0ull;
+    q4 gq{}, a1q{}, a2q{};
+    auto fetch = [&](int rr) {
+        if (ok && rr < nrow) {
+            const long long c = cbase + (long long)rr * pitch;
+            gq = ld4(A.g + c);
+            if (image_k) a1q = ld4(A.a + c);
+            a2q = ld4(A.a2 + c);
+        }
     };
-#pragma unroll
-    for (int q = 0; q < PF; q++) fetch(q, q);
-    __syncthreads();  // nu^k, D_nu^k complete on the grown tile
-
+    fetch(0);
+    __syncthreads();  // nu^k and D_nu^k complete; the stage is no longer read
     // Data of step k-1 at the tile's receivers: D' = D_nu^k + kappa r^{k-2}.
     if (T.rec_end > T.rec_begin) {
         const float *rk = A.r + T.doff + (long long)(k - 2) * T.nrec;
         for (int e = T.rec_begin + tid; e < T.rec_end; e += NT2)
             if (e == T.rec_begin || A.c.recs[e - 1].cell != A.c.recs[e].cell) {
-                const int cell = A.c.recs[e].cell;
-                const int lz = cell / TX + HALO, lx = cell % TX + HALO;
-                Dn[lz][lx] = fmaf(S.k[lz][lx], receiver_sum(A.c.recs, e, T.rec_end, rk), Dn[lz][lx]);
+                const int z = A.c.recs[e].cell / TX, x = A.c.recs[e].cell % TX;
+                const float kc = A.c.kap[T.mc * A.c.mstride + (long long)(T.z0 + z) * A.c.pf + T.mx + x];
+                float &d = (&DS[z % R4][(z / R4) * 16 + x / 4].x)[x % 4];
+                d = fmaf(kc, receiver_sum(A.c.recs, e, T.rec_end, rk), d);
             }
         __syncthreads();
     }
-    mid();  // u and D_nu of the stage are no longer read (kappa is: it is refilled at the tile's end)
+    mid();
 
-    // ---- step k-1 on the core (threads 0..255), imaging of both steps -----
-    if (!worker) return;
-    float wx0 = 1.f, wx1 = 1.f;
-    if constexpr (!FULL) {
-        wx0 = sponge1(j, nxw, nb);
-        wx1 = sponge1(j + 1, nxw, nb);
-    }
-    float2 zc[R2 + 2 * HALO];
+    // ---- step k-1 on the core, imaging of both steps --------------------------
+    if (!ok) return;
+    LapColumn<VP> col(&V[lz][lx + HALO]);
 #pragma unroll
-    for (int r = 0; r < R2 + 2 * HALO; r++) zc[r] = *reinterpret_cast<const float2 *>(&V[lz0 + r][lxp + HALO]);
-#pragma unroll
-    for (int rr = 0; rr < R2; rr++) {
-        const int q = rr % PF;
-        f2 g = gq[q];
-        const f2 a1 = a1q[q], a2 = a2q[q];
-        if (rr + PF < R2) fetch(rr + PF, q);
-        if (!(ok && rr < nrow)) continue;
-        const long long c = cbase + (long long)rr * pitch;
-        const f2 kv = *reinterpret_cast<const f2 *>(&S.k[lz0 + rr + HALO][lxp + HALO]);
-        const f2 a = lap8x2_seg(reinterpret_cast<const float2 *>(&V[lz0 + rr + HALO][lxp]), zc + rr);
-        const f2 nu = pk(zc[rr + HALO]);  // nu^k
-        const f2 d1 = *reinterpret_cast<const f2 *>(&Dn[lz0 + rr + HALO][lxp + HALO]);
-        f2 dn, nn;
+    for (int rr = 0; rr < R4; rr++) {
+        q4 nu;  // nu^k
+        const q4 a = col.row(rr, nu);
+        q4 g = gq;
+        const q4 a1 = a1q, a2 = a2q;
+        if (rr + 1 < R4) fetch(rr + 1);
+        const q4 kv = kap.row(rr), dn = ld4(&DS[rr][tid].x);
+        q4 d2, nn;
         if constexpr (FULL) {
-            dn = fma2(kv, a, d1);
-            nn = add2(nu, dn);
+            d2 = fma4(kv, a, dn);
+            nn = add4(nu, d2);
         } else {
-            const float wz = sponge1(i0 + rr, NZ, nb);
-            const f2 w = pk2(wz * wx0, wz * wx1);
-            dn = keep_lo(mul2(w, fma2(kv, a, d1)), hi);
-            nn = keep_lo(fma2(w, nu, dn), hi);
+            const q4 w = ed.w(rr);
+            d2 = mul4(w, fma4(kv, a, dn));
+            nn = fma4(w, nu, d2);
         }
-        if (image_k) g = keep_lo(fma2(a1, nu, g), hi);
-        g = keep_lo(fma2(a2, nn, g), hi);
-        *reinterpret_cast<f2 *>(A.dd_out + c) = dn;
-        *reinterpret_cast<f2 *>(A.nun + c) = nn;
-        *reinterpret_cast<f2 *>(A.g + c) = g;
+        if (image_k) g = fma4(a1, nu, g);
+        g = fma4(a2, nn, g);
+        if (rr < nrow) {
+            const long long c = cbase + (long long)rr * pitch;
+            st4(A.dd_out + c, d2);
+            st4(A.nun + c, nn);
+            st4(A.g + c, g);
+        }
     }
 }
 
 __global__ void __launch_bounds__(NT2, 2) adj_pair_kernel(AdjArgs A, const __grid_constant__ TileMaps M, int ntiles) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    Fwd2Stage &S = *reinterpret_cast<Fwd2Stage *>(smem_raw);
-    ETile &V = *reinterpret_cast<ETile *>(smem_raw + sizeof(Fwd2Stage));
-    ETile &Dn = *reinterpret_cast<ETile *>(smem_raw + sizeof(Fwd2Stage) + sizeof(ETile));
-    PipeTail *tail = reinterpret_cast<PipeTail *>(smem_raw + sizeof(Fwd2Stage) + 2 * sizeof(ETile));
-    InjBuf &IB = *reinterpret_cast<InjBuf *>(smem_raw + kFwd2Smem);
+    Pair2Stage &S = *reinterpret_cast<Pair2Stage *>(smem_raw);
+    VTile &V = *reinterpret_cast<VTile *>(smem_raw + sizeof(Pair2Stage));
+    DStash &DS = *reinterpret_cast<DStash *>(smem_raw + sizeof(Pair2Stage) + sizeof(VTile));
+    PairTail *tail = reinterpret_cast<PairTail *>(smem_raw + sizeof(Pair2Stage) + sizeof(VTile) + sizeof(DStash));
+    InjBuf &IB = *reinterpret_cast<InjBuf *>(smem_raw + kPair2Smem);
     const int tid = threadIdx.x + threadIdx.y * 32;
-    const bool leader = tid == 0;
+    const bool leader = tid == LEADER;
     const unsigned bar = smem_u32(&tail->bar[0]);
     const int b = blockIdx.x, g = gridDim.x;
-    int4 co = make_int4(0, 0, 0, 0);
-    int mc = 0;
     if (smem_u32(&S) & 127u) {
         if (leader) atomicExch(A.c.tflag, 2u);
         return;
@@ -418,39 +434,33 @@ __global__ void __launch_bounds__(NT2, 2) adj_pair_kernel(AdjArgs A, const __gri
     if (leader) {
         mbar_init(bar, 1);
         fence_mbar_init();
-        fetch_coords(A.c.infos, b, co, mc);
         copy_desc(&tail->desc[0], &A.c.infos[b]);
+        if (b + g < ntiles) copy_desc(&tail->desc[1], &A.c.infos[b + g]);
+        cp_async_wait_all();
     }
     griddep_wait();
     griddep_launch_dependents();
-    // The stage is refilled in two parts on one mbarrier phase: u and D_nu
-    // once the first step is done, kappa (read by the second step too) at
-    // the end of the tile.  The same tile's image, a^{k-1} and a^{k-2},
-    // which the second step loads from global memory, are prefetched into L2
-    // then, a tile ahead of their use.
-    auto issue_ud = [&]() {
+    // The same tile's image, a^{k-1} and a^{k-2}, which the second step loads
+    // from global memory, are prefetched into L2 with the stage.
+    auto issue = [&](const TileInfo &N) {
         fence_proxy_async();
-        mbar_expect_tx(bar, kFwd2StageBytes);
-        tma_load_3d(smem_u32(&S.u), &M.m[0], co.z - HALO2, co.y - HALO2, co.x, bar);
-        tma_load_3d(smem_u32(&S.d), &M.m[1], co.z - HALO, co.y - HALO, co.x, bar);
-        tma_prefetch_l2_3d(&M.m[3], co.z, co.y, co.x);
-        tma_prefetch_l2_3d(&M.m[4], co.z, co.y, co.x);
-        tma_prefetch_l2_3d(&M.m[5], co.z, co.y, co.x);
+        mbar_expect_tx(bar, kPair2StageBytes);
+        tma_load_3d(smem_u32(&S.u), &M.m[0], N.x0 - HALO2, N.z0 - HALO2, N.slot, bar);
+        tma_load_3d(smem_u32(&S.d), &M.m[1], N.x0 - HALO, N.z0 - HALO, N.slot, bar);
+        tma_prefetch_l2_3d(&M.m[3], N.x0, N.z0, N.slot);
+        tma_prefetch_l2_3d(&M.m[4], N.x0, N.z0, N.slot);
+        tma_prefetch_l2_3d(&M.m[5], N.x0, N.z0, N.slot);
     };
-    auto issue_k = [&]() {
-        fence_proxy_async();
-        tma_load_3d(smem_u32(&S.k), &M.m[2], co.w - HALO, co.y - HALO, mc, bar);
-    };
-    // Data of step k injected here (inject_here): warp 8, which has no cells
-    // in the second step, lists the next tile's grown-region injection
-    // (kappa and the receivers' summed data, from global memory) while the
-    // other warps run that step; after the tile's stage lands every thread
-    // adds the list to the staged D_nu, D' = fmaf(kappa, sum, D) as the
-    // separate pass computes it.  Shots whose record ends before step k take
-    // none.
+    // Data of step k injected here (inject_here): warp 8, free in the second
+    // step, lists the next tile's grown-region injection (kappa and the
+    // receivers' summed data, from global memory) while the core warps run
+    // that step; after the tile's stage lands every thread adds the list to
+    // the staged D_nu, D' = fmaf(kappa, sum, D) as the separate pass computes
+    // it.  Shots whose record ends before step k take none.
     const bool inj = A.inject_here && A.c.xrec_off != nullptr;
+    const bool lister = tid >= NCORE && tid < NCORE + 32;
     auto build = [&](int t) {
-        const int lane = tid - 256;
+        const int lane = tid - NCORE;
         const int xb = A.c.xrec_off[t], xe = A.c.xrec_off[t + 1];
         const TileInfo &Tg = A.c.infos[t];
         const bool has = Tg.nt > A.k - 1;
@@ -468,14 +478,11 @@ __global__ void __launch_bounds__(NT2, 2) adj_pair_kernel(AdjArgs A, const __gri
         }
         if (lane == 0) IB.n = has ? xe - xb : 0;
     };
-    if (leader) {
-        issue_ud();
-        issue_k();
-        if (b + g < ntiles) fetch_coords(A.c.infos, b + g, co, mc);
-    }
-    if (inj && tid >= 256) build(b);
+    if (leader) issue(tail->desc[0]);
+    if (inj && lister) build(b);
     __syncthreads();
     unsigned phase = 0;
+    int slot = 0, next = 1;
     for (int tix = b; tix < ntiles; tix += g) {
         const bool landed = mbar_wait(bar, phase);
         phase ^= 1u;
@@ -497,19 +504,19 @@ __global__ void __launch_bounds__(NT2, 2) adj_pair_kernel(AdjArgs A, const __gri
             if (n > 0) __syncthreads();
         }
         const bool more = tix + g < ntiles;
-        auto mid = [&]() {  // after a barrier: every thread is done with u and D_nu
-            if (leader && more) issue_ud();
+        auto mid = [&]() {  // after a barrier: every thread is done with the stage
+            if (leader && more) {
+                issue(tail->desc[next]);
+                if (tix + 2 * g < ntiles) copy_desc(&tail->desc[3 - slot - next], &A.c.infos[tix + 2 * g]);
+            }
         };
-        const TileInfo &T = tail->desc[0];
-        if (T.flags & TI_INTERIOR2) adj_pair_tile<true>(A, S, V, Dn, T, tid, mid);
-        else adj_pair_tile<false>(A, S, V, Dn, T, tid, mid);
-        if (inj && tid >= 256 && more) build(tix + g);  // warp 8, during the other warps' second step
-        __syncthreads();  // kappa, the descriptor, V and Dn are free
-        if (leader && more) {
-            issue_k();
-            copy_desc(&tail->desc[0], &A.c.infos[tix + g]);
-            if (tix + 2 * g < ntiles) fetch_coords(A.c.infos, tix + 2 * g, co, mc);
-        }
+        const TileInfo &T = tail->desc[slot];
+        if (T.flags & TI_INTERIOR2) adj_pair_tile<true>(A, S, V, DS, T, tid, mid);
+        else adj_pair_tile<false>(A, S, V, DS, T, tid, mid);
+        if (inj && lister && more) build(tix + g);  // warp 8, during the core warps' second step
+        const int after = 3 - slot - next;
+        slot = next;
+        next = after;
     }
 }
 
@@ -536,7 +543,7 @@ __global__ void adj_inject_kernel(AdjArgs A, const int *__restrict__ rtiles) {
 
 template <typename K, typename Args>
 void launch_pdl2(K kernel, int grid, const Args &a, const TileMaps &maps, int ntiles, cudaStream_t s,
-                 size_t smem = kFwd2Smem) {
+                 size_t smem = kPair2Smem) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(32, NT2 / 32);
@@ -550,7 +557,7 @@ void launch_pdl2(K kernel, int grid, const Args &a, const TileMaps &maps, int nt
     cudaLaunchKernelEx(&cfg, kernel, a, maps, ntiles);
 }
 
-int occupancy_of(const void *fn, size_t smem = kFwd2Smem) {
+int occupancy_of(const void *fn, size_t smem = kPair2Smem) {
     int n = 0;
     cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, NT2, smem);
