@@ -18,16 +18,19 @@
 // and bottom ones to warp 9: ten full warps in step n, and a core thread
 // advances the same 16 cells in both steps, so D^{n+1} only passes through the
 // thread's own 64 bytes of shared memory.  16-byte accesses take 1.9 shared
-// loads per update where two columns per thread took 5.7, and the tile takes
-// 41 instead of 57 instructions per update.  What bounds it: latency at 20
-// warps per SM (FMA pipe 42 % busy, DRAM 34 %).
-// Forward, 64 shots of 400 x 1200: 64.4 -> 58.8 us per launch (two columns x
-// 9 rows per thread, sponge factors and bounds tests computed per row -> this).
+// loads per update where two columns per thread took 5.7.  kappa, shared by
+// all shots and L2-resident, is copied by each thread into slots of its own a
+// tile ahead (cp.async): no thread waits on a global load between the barriers.
+// What bounds it: latency at 20 warps per SM.  Forward, 64 shots of 400 x 1200,
+// per launch: 64.4 us (two columns x 9 rows per thread, sponge factors and
+// bounds tests computed per row) -> 58.8 (items, kappa and sponge factors loaded
+// where they are used) -> 48.5 (both copied a tile ahead).
 //
 // Sponge: the factor is separable and depends on the distances to the padded
 // domain's edges only, so the plan holds it per row and per slot's column
-// (zero outside the domain, which also masks the cells out there); a tile that
-// the sponge reaches reads 4 + 4 factors per item and needs no bounds tests.
+// (zero outside the domain, which also masks the cells out there); the tile's
+// 72 + 72 factors are copied a tile ahead, and a tile that the sponge reaches
+// needs no bounds tests.
 //
 // Sources: injected at both steps (q^n, q^{n+1}), also on ring cells.
 // Receivers: sample n from u^{n+1} in shared memory, sample n+1 from the
@@ -63,10 +66,20 @@ struct PairTail {
     TileInfo desc[3];
 };
 static_assert(sizeof(PairTail) % 16 == 0, "tail layout");
-// D^{n+1} of the core threads' cells between the steps (each thread its own
-// 4 x 16 bytes).
-typedef float4 DStash[4][256];
-constexpr size_t kPair2Smem = sizeof(Pair2Stage) + sizeof(VTile) + sizeof(DStash) + sizeof(PairTail);
+// Per-thread 16-byte slots: kappa of the thread's item (row rr at k[rr]),
+// which the thread copies itself (cp.async) for the next tile once it is done
+// with this one's, so that it needs no barrier; and D^{n+1} of the core threads'
+// cells between the steps.
+struct ItemSlots {
+    float4 k[4][320], d[4][256];
+};
+// Sponge factors of the tile's rows and columns, ring included; this tile's
+// and the next one's alternate.
+struct TileEdge {
+    float wz[E], wx[E];
+};
+constexpr size_t kPair2Smem =
+    sizeof(Pair2Stage) + sizeof(VTile) + sizeof(ItemSlots) + 2 * sizeof(TileEdge) + sizeof(PairTail);
 // The two-step adjoint's list of its next tile's data injection (grown
 // region, step k): offset of the cell in the staged D_nu (-1: a further
 // receiver of the cell before, already summed), kappa there, summed data.
@@ -98,44 +111,35 @@ __device__ __forceinline__ void item_of(int tid, int &lx, int &lz) {
     }
 }
 
-// Sponge factors of an item's rows, read from the plan's tables (L1 and L2
-// hits), and its source cell.
-struct ItemEdge {
-    const float *wz, *wx;
-    int src;  // 4 * row + column of the source inside the item, -1 without one
-    __device__ __forceinline__ ItemEdge(const StepCommon &c, const TileInfo &T, int lx, int lz) {
-        wz = c.wz + (T.z0 + lz + HALO);
-        wx = c.wx + ((long long)T.slot * (T.pitch + 2 * HALO) + T.x0 + lx + HALO);
-        const unsigned x = T.sx - (T.x0 + lx), z = T.sz - (T.z0 + lz);
-        src = x < 4u && z < (unsigned)R4 ? (int)(4 * z + x) : -1;
+// The source cell of a thread's item, as 4 * row + column, or -1.
+__device__ __forceinline__ int item_source(const TileInfo &T, int lx, int lz) {
+    const unsigned x = T.sx - (T.x0 + lx), z = T.sz - (T.z0 + lz);
+    return x < 4u && z < (unsigned)R4 ? (int)(4 * z + x) : -1;
+}
+// Sponge factors of the item's row rr.
+__device__ __forceinline__ q4 row_w(const TileEdge &We, int lx, int lz, int rr) {
+    const float z = We.wz[lz + rr + HALO];
+    const q4 x = ld4(&We.wx[lx + HALO]);
+    return q4{mul2(pk2(z, z), x.lo), mul2(pk2(z, z), x.hi)};
+}
+// This thread's kappa of a tile, from the L2-resident model array.  Rows and
+// quads outside the padded domain, whose sponge factor is zero, take some
+// cell's inside it.
+__device__ __forceinline__ void copy_kappa(ItemSlots &I, const StepCommon &c, const TileInfo &T, int tid) {
+    int lx, lz;
+    item_of(tid, lx, lz);
+    const float *m = c.kap + (long long)T.mc * c.mstride + min(max(T.mx + lx, 0), c.pf - 4);
+#pragma unroll
+    for (int rr = 0; rr < R4; rr++)
+        cp_async16(&I.k[rr][tid], m + min(max(T.z0 + lz + rr, 0), c.NZ - 1) * c.pf);
+}
+// A tile's sponge factors, copied by one warp.
+__device__ __forceinline__ void copy_edge(TileEdge &We, const StepCommon &c, const TileInfo &T, int lane) {
+    if (lane < E / 4) {
+        cp_async16(&We.wz[4 * lane], c.wz + T.z0 + 4 * lane);
+        cp_async16(&We.wx[4 * lane], c.wx + (long long)T.slot * (T.pitch + 2 * HALO) + T.x0 + 4 * lane);
     }
-    __device__ __forceinline__ q4 w(int rr) const {
-        const float z = __ldg(wz + rr);
-        const float4 x = __ldg(reinterpret_cast<const float4 *>(wx));
-        return q4{mul2(pk2(z, z), pk2(x.x, x.y)), mul2(pk2(z, z), pk2(x.z, x.w))};
-    }
-};
-// kappa of an item's row rr, from the L2-resident model array (both steps read
-// it there: staging it would cost 20 KB of shared memory).  Quads outside the
-// padded domain, whose sponge factor is zero, take some cell's inside it.
-template <bool FULL>
-struct ItemKappa {
-    const float *p;
-    int pf, i0, NZ;
-    __device__ __forceinline__ ItemKappa(const StepCommon &c, const TileInfo &T, int lx, int lz) {
-        pf = c.pf;
-        i0 = T.z0 + lz;
-        NZ = c.NZ;
-        const float *m = c.kap + (long long)T.mc * c.mstride;
-        if constexpr (FULL) p = m + (i0 * pf + T.mx + lx);
-        else p = m + min(max(T.mx + lx, 0), pf - 4);
-    }
-    __device__ __forceinline__ q4 row(int rr) const {
-        const float4 v = __ldg(reinterpret_cast<const float4 *>(
-            FULL ? p + rr * pf : p + min(max(i0 + rr, 0), NZ - 1) * pf));
-        return q4{pk2(v.x, v.y), pk2(v.z, v.w)};
-    }
-};
+}
 __device__ __forceinline__ void add_source(q4 &a, int scol, float q) {
     float2 l = upk(a.lo), h = upk(a.hi);
     if (scol == 0) l.x += q;
@@ -148,7 +152,7 @@ __device__ __forceinline__ void add_source(q4 &a, int scol, float q) {
 // mid(): called by every thread after the barrier that ends step n (the
 // stage is no longer read): the leader refills the stage.
 template <bool STORE_A, bool FULL, class MidFn>
-__device__ __forceinline__ void pair_tile(const FwdArgs &A, const Pair2Stage &S, VTile &V, DStash &DS,
+__device__ __forceinline__ void pair_tile(const FwdArgs &A, const Pair2Stage &S, VTile &V, ItemSlots &I, const TileEdge &We,
                                           const TileInfo &T, int tid, bool two, MidFn mid) {
     int lx, lz;
     item_of(tid, lx, lz);
@@ -158,8 +162,7 @@ __device__ __forceinline__ void pair_tile(const FwdArgs &A, const Pair2Stage &S,
     const int nrow = FULL ? R4 : A.c.NZ - i0;
     const bool ok = core && (FULL || j < T.nxw);
     const long long cbase = T.foff + (long long)i0 * pitch + j;
-    const ItemEdge ed(A.c, T, lx, lz);  // (unused where FULL)
-    const ItemKappa<FULL> kap(A.c, T, lx, lz);
+    const int src = FULL ? -1 : item_source(T, lx, lz);
 
     // ---- step n on the item ------------------------------------------------
     {
@@ -169,19 +172,19 @@ __device__ __forceinline__ void pair_tile(const FwdArgs &A, const Pair2Stage &S,
             q4 u;
             q4 a = col.row(rr, u);
             const q4 dv = ld4(&S.d[lz + rr + HALO][lx + HALO]);
-            const q4 kv = kap.row(rr);
+            const q4 kv = ld4(&I.k[rr][tid].x);
             q4 un, dn;
             if constexpr (FULL) {
                 dn = fma4(kv, a, dv);
                 un = add4(u, dn);
             } else {
-                if (rr == ed.src >> 2) add_source(a, ed.src & 3, A.c.wav[T.wav_off + n]);
-                const q4 w = ed.w(rr);
+                if (rr == src >> 2) add_source(a, src & 3, A.c.wav[T.wav_off + n]);
+                const q4 w = row_w(We, lx, lz, rr);
                 dn = mul4(w, fma4(kv, a, dv));
                 un = fma4(w, u, dn);
             }
             st4(&V[lz + rr + HALO][lx + HALO], un);
-            if (core) st4(&DS[rr][tid].x, dn);
+            if (core) st4(&I.d[rr][tid].x, dn);
             if (ok && rr < nrow) {
                 const long long c = cbase + (long long)rr * pitch;
                 if (!STORE_A && A.ck_u) {
@@ -210,7 +213,7 @@ __device__ __forceinline__ void pair_tile(const FwdArgs &A, const Pair2Stage &S,
             if (ok && rr < nrow) {
                 const long long c = cbase + (long long)rr * pitch;
                 st4(A.un + c, ld4(&V[lz + rr + HALO][lx + HALO]));
-                st4(A.dd_out + c, ld4(&DS[rr][tid].x));
+                st4(A.dd_out + c, ld4(&I.d[rr][tid].x));
             }
         }
         return;
@@ -221,14 +224,14 @@ __device__ __forceinline__ void pair_tile(const FwdArgs &A, const Pair2Stage &S,
         for (int rr = 0; rr < R4; rr++) {
             q4 u;
             q4 a = col.row(rr, u);
-            const q4 kv = kap.row(rr), dn = ld4(&DS[rr][tid].x);
+            const q4 kv = ld4(&I.k[rr][tid].x), dn = ld4(&I.d[rr][tid].x);
             q4 d2, un;
             if constexpr (FULL) {
                 d2 = fma4(kv, a, dn);
                 un = add4(u, d2);
             } else {
-                if (rr == ed.src >> 2) add_source(a, ed.src & 3, A.c.wav[T.wav_off + n + 1]);
-                const q4 w = ed.w(rr);
+                if (rr == src >> 2) add_source(a, src & 3, A.c.wav[T.wav_off + n + 1]);
+                const q4 w = row_w(We, lx, lz, rr);
                 d2 = mul4(w, fma4(kv, a, dn));
                 un = fma4(w, u, d2);
             }
@@ -254,8 +257,9 @@ __global__ void __launch_bounds__(NT2, 2) fwd_pair_kernel(FwdArgs A, const __gri
     extern __shared__ __align__(128) unsigned char smem_raw[];
     Pair2Stage &S = *reinterpret_cast<Pair2Stage *>(smem_raw);
     VTile &V = *reinterpret_cast<VTile *>(smem_raw + sizeof(Pair2Stage));
-    DStash &DS = *reinterpret_cast<DStash *>(smem_raw + sizeof(Pair2Stage) + sizeof(VTile));
-    PairTail *tail = reinterpret_cast<PairTail *>(smem_raw + sizeof(Pair2Stage) + sizeof(VTile) + sizeof(DStash));
+    ItemSlots &I = *reinterpret_cast<ItemSlots *>(smem_raw + sizeof(Pair2Stage) + sizeof(VTile));
+    TileEdge *We = reinterpret_cast<TileEdge *>(smem_raw + sizeof(Pair2Stage) + sizeof(VTile) + sizeof(ItemSlots));
+    PairTail *tail = reinterpret_cast<PairTail *>(We + 2);
     const int tid = threadIdx.x + threadIdx.y * 32;
     const bool leader = tid == LEADER;
     const unsigned bar = smem_u32(&tail->bar[0]);
@@ -281,12 +285,14 @@ __global__ void __launch_bounds__(NT2, 2) fwd_pair_kernel(FwdArgs A, const __gri
     };
     if (leader) issue(tail->desc[0]);
     __syncthreads();
+    copy_kappa(I, A.c, tail->desc[0], tid);
+    if (tid >= LEADER) copy_edge(We[0], A.c, tail->desc[0], tid - LEADER);
     unsigned phase = 0;
     int slot = 0, next = 1;
     for (int tix = b; tix < ntiles; tix += g) {
         const bool landed = mbar_wait(bar, phase);
         phase ^= 1u;
-        if (leader) cp_async_wait_all();
+        cp_async_wait_all();
         if (__syncthreads_or(!landed)) {
             if (leader) {
                 mbar_wait(bar, phase ^ 1u);  // copies in flight: a second bounded wait before leaving
@@ -294,16 +300,20 @@ __global__ void __launch_bounds__(NT2, 2) fwd_pair_kernel(FwdArgs A, const __gri
             }
             return;
         }
+        const bool more = tix + g < ntiles;
         auto mid = [&]() {  // after a barrier: every thread is done with the stage
-            if (leader && tix + g < ntiles) {
+            if (tid < LEADER || !more) return;
+            if (leader) {
                 issue(tail->desc[next]);
                 if (tix + 2 * g < ntiles) copy_desc(&tail->desc[3 - slot - next], &A.c.infos[tix + 2 * g]);
             }
+            copy_edge(We[phase], A.c, tail->desc[next], tid - LEADER);
         };
         const TileInfo &T = tail->desc[slot];
         const bool two = T.nt > A.n + 1;
-        if (T.flags & TI_FULL2) pair_tile<STORE_A, true>(A, S, V, DS, T, tid, two, mid);
-        else pair_tile<STORE_A, false>(A, S, V, DS, T, tid, two, mid);
+        if (T.flags & TI_FULL2) pair_tile<STORE_A, true>(A, S, V, I, We[phase ^ 1u], T, tid, two, mid);
+        else pair_tile<STORE_A, false>(A, S, V, I, We[phase ^ 1u], T, tid, two, mid);
+        if (more) copy_kappa(I, A.c, tail->desc[next], tid);
         const int after = 3 - slot - next;
         slot = next;
         next = after;
@@ -320,7 +330,7 @@ __global__ void __launch_bounds__(NT2, 2) fwd_pair_kernel(FwdArgs A, const __gri
 // nu^{k-1}, in that order, as two one-step launches would.
 // ---------------------------------------------------------------------------
 template <bool FULL, class MidFn>
-__device__ __forceinline__ void adj_pair_tile(const AdjArgs &A, Pair2Stage &S, VTile &V, DStash &DS,
+__device__ __forceinline__ void adj_pair_tile(const AdjArgs &A, Pair2Stage &S, VTile &V, ItemSlots &I, const TileEdge &We,
                                               const TileInfo &T, int tid, MidFn mid) {
     int lx, lz;
     item_of(tid, lx, lz);
@@ -330,8 +340,6 @@ __device__ __forceinline__ void adj_pair_tile(const AdjArgs &A, Pair2Stage &S, V
     const int nrow = FULL ? R4 : A.c.NZ - i0;
     const bool ok = core && (FULL || j < T.nxw);
     const long long cbase = T.foff + (long long)i0 * pitch + j;
-    const ItemEdge ed(A.c, T, lx, lz);  // (unused where FULL)
-    const ItemKappa<FULL> kap(A.c, T, lx, lz);
 
     // ---- step k on the item --------------------------------------------------
     {
@@ -341,18 +349,18 @@ __device__ __forceinline__ void adj_pair_tile(const AdjArgs &A, Pair2Stage &S, V
             q4 nu;
             const q4 a = col.row(rr, nu);
             const q4 dv = ld4(&S.d[lz + rr + HALO][lx + HALO]);
-            const q4 kv = kap.row(rr);
+            const q4 kv = ld4(&I.k[rr][tid].x);
             q4 nn, dn;
             if constexpr (FULL) {
                 dn = fma4(kv, a, dv);
                 nn = add4(nu, dn);
             } else {
-                const q4 w = ed.w(rr);
+                const q4 w = row_w(We, lx, lz, rr);
                 dn = mul4(w, fma4(kv, a, dv));
                 nn = fma4(w, nu, dn);
             }
             st4(&V[lz + rr + HALO][lx + HALO], nn);
-            if (core) st4(&DS[rr][tid].x, dn);
+            if (core) st4(&I.d[rr][tid].x, dn);
         }
     }
     // The image and the background terms of the second step (prefetched into
@@ -377,8 +385,9 @@ __device__ __forceinline__ void adj_pair_tile(const AdjArgs &A, Pair2Stage &S, V
         for (int e = T.rec_begin + tid; e < T.rec_end; e += NT2)
             if (e == T.rec_begin || A.c.recs[e - 1].cell != A.c.recs[e].cell) {
                 const int z = A.c.recs[e].cell / TX, x = A.c.recs[e].cell % TX;
-                const float kc = A.c.kap[T.mc * A.c.mstride + (long long)(T.z0 + z) * A.c.pf + T.mx + x];
-                float &d = (&DS[z % R4][(z / R4) * 16 + x / 4].x)[x % 4];
+                const int item = (z / R4) * 16 + x / 4;
+                const float kc = (&I.k[z % R4][item].x)[x % 4];
+                float &d = (&I.d[z % R4][item].x)[x % 4];
                 d = fmaf(kc, receiver_sum(A.c.recs, e, T.rec_end, rk), d);
             }
         __syncthreads();
@@ -395,13 +404,13 @@ __device__ __forceinline__ void adj_pair_tile(const AdjArgs &A, Pair2Stage &S, V
         q4 g = gq;
         const q4 a1 = a1q, a2 = a2q;
         if (rr + 1 < R4) fetch(rr + 1);
-        const q4 kv = kap.row(rr), dn = ld4(&DS[rr][tid].x);
+        const q4 kv = ld4(&I.k[rr][tid].x), dn = ld4(&I.d[rr][tid].x);
         q4 d2, nn;
         if constexpr (FULL) {
             d2 = fma4(kv, a, dn);
             nn = add4(nu, d2);
         } else {
-            const q4 w = ed.w(rr);
+            const q4 w = row_w(We, lx, lz, rr);
             d2 = mul4(w, fma4(kv, a, dn));
             nn = fma4(w, nu, d2);
         }
@@ -420,8 +429,9 @@ __global__ void __launch_bounds__(NT2, 2) adj_pair_kernel(AdjArgs A, const __gri
     extern __shared__ __align__(128) unsigned char smem_raw[];
     Pair2Stage &S = *reinterpret_cast<Pair2Stage *>(smem_raw);
     VTile &V = *reinterpret_cast<VTile *>(smem_raw + sizeof(Pair2Stage));
-    DStash &DS = *reinterpret_cast<DStash *>(smem_raw + sizeof(Pair2Stage) + sizeof(VTile));
-    PairTail *tail = reinterpret_cast<PairTail *>(smem_raw + sizeof(Pair2Stage) + sizeof(VTile) + sizeof(DStash));
+    ItemSlots &I = *reinterpret_cast<ItemSlots *>(smem_raw + sizeof(Pair2Stage) + sizeof(VTile));
+    TileEdge *We = reinterpret_cast<TileEdge *>(smem_raw + sizeof(Pair2Stage) + sizeof(VTile) + sizeof(ItemSlots));
+    PairTail *tail = reinterpret_cast<PairTail *>(We + 2);
     InjBuf &IB = *reinterpret_cast<InjBuf *>(smem_raw + kPair2Smem);
     const int tid = threadIdx.x + threadIdx.y * 32;
     const bool leader = tid == LEADER;
@@ -481,12 +491,14 @@ __global__ void __launch_bounds__(NT2, 2) adj_pair_kernel(AdjArgs A, const __gri
     if (leader) issue(tail->desc[0]);
     if (inj && lister) build(b);
     __syncthreads();
+    copy_kappa(I, A.c, tail->desc[0], tid);
+    if (tid >= LEADER) copy_edge(We[0], A.c, tail->desc[0], tid - LEADER);
     unsigned phase = 0;
     int slot = 0, next = 1;
     for (int tix = b; tix < ntiles; tix += g) {
         const bool landed = mbar_wait(bar, phase);
         phase ^= 1u;
-        if (leader) cp_async_wait_all();
+        cp_async_wait_all();
         if (__syncthreads_or(!landed)) {
             if (leader) {
                 mbar_wait(bar, phase ^ 1u);  // copies in flight: a second bounded wait before leaving
@@ -505,15 +517,18 @@ __global__ void __launch_bounds__(NT2, 2) adj_pair_kernel(AdjArgs A, const __gri
         }
         const bool more = tix + g < ntiles;
         auto mid = [&]() {  // after a barrier: every thread is done with the stage
-            if (leader && more) {
+            if (tid < LEADER || !more) return;
+            if (leader) {
                 issue(tail->desc[next]);
                 if (tix + 2 * g < ntiles) copy_desc(&tail->desc[3 - slot - next], &A.c.infos[tix + 2 * g]);
             }
+            copy_edge(We[phase], A.c, tail->desc[next], tid - LEADER);
         };
         const TileInfo &T = tail->desc[slot];
-        if (T.flags & TI_INTERIOR2) adj_pair_tile<true>(A, S, V, DS, T, tid, mid);
-        else adj_pair_tile<false>(A, S, V, DS, T, tid, mid);
+        if (T.flags & TI_INTERIOR2) adj_pair_tile<true>(A, S, V, I, We[phase ^ 1u], T, tid, mid);
+        else adj_pair_tile<false>(A, S, V, I, We[phase ^ 1u], T, tid, mid);
         if (inj && lister && more) build(tix + g);  // warp 8, during the core warps' second step
+        if (more) copy_kappa(I, A.c, tail->desc[next], tid);
         const int after = 3 - slot - next;
         slot = next;
         next = after;
