@@ -83,9 +83,10 @@ struct dhfwi_ctx {
     // Step-kernel launch choice per kind: forward, forward+segment store,
     // adjoint, Born.  Picked by autotune() for the current plan.
     StepLaunch launch[4];
-    // Time steps per launch (1 or 2) of the forward and the adjoint sweeps,
-    // chosen by the autotuner.
-    int depth[2] = {2, 2};
+    // Time steps per launch (1 or 2) of the forward and the adjoint sweeps, of
+    // Born demigration and of Born from a stored history, chosen by the
+    // autotuner.
+    int depth[4] = {2, 2, 2, 2};
     // Reuse of the stored forward wavefield between calls (dhfwi_set_reuse):
     // the identity of the last complete backward-capable forward pass (plan
     // hash, model hash, history segments, checkpoint interval) whose a^n
@@ -709,8 +710,7 @@ int tune_depth(dhfwi_ctx *ctx, cudaStream_t st, const float *one_step_ms, int re
 
 // Autotuner: for the current plan, time every step-kernel variant of each
 // kind on the plan's full tile list (all shots active) using the scratch
-// field pools, and keep the fastest; then the time-blocking depth of the
-// forward and adjoint sweeps (tune_depth).  The pools are zeroed again by the
+// field pools, and keep the fastest; then the time-blocking depth of each sweep (tune_depth).  The pools are zeroed again by the
 // call that follows, so tuning leaves no trace in the results.  Runs once per
 // geometry; DHFWI_STEP_VARIANT=<0..6> pins a variant instead (and the depth
 // stays two unless DHFWI_TIME_BLOCK says otherwise).
@@ -854,11 +854,43 @@ int adj_pair_maps(dhfwi_ctx *ctx, const AdjArgs &b, TileMaps *M) {
     return tensor_map(ctx, b.a2, MAP_POOL_CELL, &M->m[5]);
 }
 
-// Time-blocking depth of the forward and the adjoint sweeps: `reps` launches
-// of the two-step kernel on the plan's full tile list against twice the
-// chosen one-step kernel's time for as many launches (one_step_ms: the
-// variant loop's best time of `reps` launches per kind: forward, forward with
-// store, adjoint, Born).  The faster depth is kept.
+// Maps of a two-step Born launch (p^n with the doubled halo, D_p with its
+// ring; a^n and a^{n+1}, which the kernel only prefetches into L2).
+int born_pair_maps(dhfwi_ctx *ctx, const BornArgs &b, TileMaps *M) {
+    int rc;
+    if ((rc = tensor_map(ctx, b.p, MAP_POOL_HALO2, &M->m[0]))) return rc;
+    if ((rc = tensor_map(ctx, b.dp, MAP_POOL_HALO, &M->m[1]))) return rc;
+    if ((rc = tensor_map(ctx, b.a, MAP_POOL_CELL, &M->m[2]))) return rc;
+    return tensor_map(ctx, b.a2, MAP_POOL_CELL, &M->m[3]);
+}
+
+// Maps of a two-step joint Born launch (u0^n and p^n with the doubled halo,
+// D_u0 and D_p with their rings).
+int born_joint_maps(dhfwi_ctx *ctx, const BornArgs &b, TileMaps *M) {
+    int rc;
+    if ((rc = tensor_map(ctx, b.u, MAP_POOL_HALO2, &M->m[0]))) return rc;
+    if ((rc = tensor_map(ctx, b.p, MAP_POOL_HALO2, &M->m[1]))) return rc;
+    if ((rc = tensor_map(ctx, b.du, MAP_POOL_HALO, &M->m[2]))) return rc;
+    return tensor_map(ctx, b.dp, MAP_POOL_HALO, &M->m[3]);
+}
+
+// Maps of a one-step Born launch from the history (p^n halo, D_p, kappa, d
+// kappa, a^n).
+int born_hist_maps(dhfwi_ctx *ctx, const BornArgs &b, TileMaps *M) {
+    int rc;
+    if ((rc = tensor_map(ctx, b.p, MAP_POOL_HALO, &M->m[0]))) return rc;
+    if ((rc = tensor_map(ctx, b.dp, MAP_POOL_CELL, &M->m[1]))) return rc;
+    if ((rc = tensor_map(ctx, b.c.kap, MAP_MODEL, &M->m[2]))) return rc;
+    if ((rc = tensor_map(ctx, b.dkap, MAP_MODEL, &M->m[3]))) return rc;
+    return tensor_map(ctx, b.a, MAP_POOL_CELL, &M->m[4]);
+}
+
+// Time-blocking depth of the forward and the adjoint sweeps, of Born and of
+// Born from the history: `reps` launches of the two-step kernel(s) on the
+// plan's full tile list against twice the chosen one-step kernel's time for as
+// many launches (one_step_ms: the variant loop's best time of `reps` launches
+// per kind: forward, forward with store, adjoint, Born).  The faster depth is
+// kept.
 int tune_depth(dhfwi_ctx *ctx, cudaStream_t st, const float *one_step_ms, int reps) {
     if (!encode_tiled()) return DHFWI_OK;
     const Plan &P = ctx->plan;
@@ -869,7 +901,9 @@ int tune_depth(dhfwi_ctx *ctx, cudaStream_t st, const float *one_step_ms, int re
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
     int rc = DHFWI_OK;
-    for (int which = 0; which < 2 && !rc; which++) {
+    float hist_ms = 0.f;  // one step of Born from the history
+    // which: 0 forward, 1 adjoint, 2 Born, 3 one step of Born from the history, 4 two of them.
+    for (int which = 0; which < 5 && !rc; which++) {
         float ms = 0.f;
         for (int rep = -1; rep < reps && !rc; rep++) {
             if (rep == 0) cudaEventRecord(e0, st);
@@ -885,7 +919,33 @@ int tune_depth(dhfwi_ctx *ctx, cudaStream_t st, const float *one_step_ms, int re
                 a.n = 0;
                 if (!(rc = pair_maps(ctx, a, &M))) launch_fwd_pair(a, ntiles, M, st);
                 ctx->stats.kernel_launches++;
-            } else {
+            }
+            if (which >= 2 && !rc) {
+                BornArgs b{};
+                b.c = common(ctx);
+                b.p = F + 3 * pool;
+                b.pn = F + 4 * pool;
+                b.dp = F + 5 * pool;
+                b.dp_out = F + 6 * pool;
+                b.dkap = (const float *)ctx->kap.p;
+                b.d = (float *)ctx->dtmp.p;
+                b.u = F;
+                b.un = F + pool;
+                b.du = F + 2 * pool;
+                b.du_out = F + 7 * pool;
+                b.a = F;
+                b.a2 = F + pool;
+                b.n = 0;
+                if (which == 2) {
+                    if (!(rc = born_joint_maps(ctx, b, &M))) launch_born_joint(b, ntiles, M, st);
+                } else if (which == 3) {
+                    if (!(rc = born_hist_maps(ctx, b, &M))) launch_born_hist_step(b, ntiles, M, st);
+                } else {
+                    if (!(rc = born_pair_maps(ctx, b, &M))) launch_born_pair(b, ntiles, M, st);
+                }
+                ctx->stats.kernel_launches++;
+            }
+            if (which == 1) {
                 AdjArgs b{};
                 b.c = common(ctx);
                 b.nu = F;
@@ -913,14 +973,18 @@ int tune_depth(dhfwi_ctx *ctx, cudaStream_t st, const float *one_step_ms, int re
         }
         if (rc) break;
         cudaEventElapsedTime(&ms, e0, e1);
-        const float one = one_step_ms[which == 0 ? 0 : 2];
-        ctx->depth[which] = ms <= 2.f * one ? 2 : 1;
+        if (which == 3) {
+            hist_ms = ms;
+            continue;
+        }
+        const float one = which == 4 ? hist_ms : one_step_ms[which == 0 ? 0 : which + 1];
+        ctx->depth[which == 4 ? 3 : which] = ms <= 2.f * one ? 2 : 1;
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (rc) {  // no two-step launch possible here: one step per launch
         ctx->err.clear();
-        ctx->depth[0] = ctx->depth[1] = 1;
+        for (int &d : ctx->depth) d = 1;
     }
     return DHFWI_OK;
 }
@@ -1409,7 +1473,7 @@ int born_demig(dhfwi_ctx *ctx, const float *v0_dev, const dhfwi_geom *geom, cons
     const long long pool = P.pool_floats;
     if ((rc = ensure(ctx, ctx->fields, NPOOLS * sizeof(float) * (size_t)pool, "wavefield pools"))) return rc;
     float *F = (float *)ctx->fields.p;
-    CK(cudaMemsetAsync(F, 0, sizeof(float) * 6 * (size_t)pool, st));
+    CK(cudaMemsetAsync(F, 0, sizeof(float) * 8 * (size_t)pool, st));
     BornArgs a{};
     a.c = common(ctx);
     a.dkap = (const float *)ctx->dkap.p;
@@ -1417,28 +1481,58 @@ int born_demig(dhfwi_ctx *ctx, const float *v0_dev, const dhfwi_geom *geom, cons
     float *u = F, *un = F + pool, *p = F + 2 * pool, *pn = F + 3 * pool;
     a.du = F + 4 * pool;
     a.dp = F + 5 * pool;
+    float *du2 = F + 6 * pool, *dp2 = F + 7 * pool;  // second D pools of the two-step launches
     const long long l0 = ctx->stats.kernel_launches, c0 = ctx->stats.cell_updates;
     phase_begin(ctx, 2, st);
     // Background from the stored forward pass at this model (every step of
     // it in the history, TMA available): only the scattered field advances.
     if (forward_reusable(ctx) && (long long)ctx->hist_segs * ctx->ck_every >= P.nt_max && encode_tiled()) {
         float *hist = (float *)ctx->hist.p;
-        for (int n = 0; n < P.nt_max; n++) {
+        const bool two = time_blocking(ctx, 3);
+        for (int n = 0; n < P.nt_max; n += two ? 2 : 1) {
             a.p = p;
             a.pn = pn;
             a.n = n;
             a.a = hist + ctx->hoff[n];
             TileMaps M;
-            if ((rc = tensor_map(ctx, a.p, MAP_POOL_HALO, &M.m[0])) || (rc = tensor_map(ctx, a.dp, MAP_POOL_CELL, &M.m[1])) ||
-                (rc = tensor_map(ctx, a.c.kap, MAP_MODEL, &M.m[2])) || (rc = tensor_map(ctx, a.dkap, MAP_MODEL, &M.m[3])) ||
-                (rc = tensor_map(ctx, a.a, MAP_POOL_CELL, &M.m[4])))
-                return rc;
-            launch_born_hist_step(a, active_tiles(P, n), M, st);
+            if (two) {
+                a.a2 = hist + ctx->hoff[std::min(n + 1, P.nt_max - 1)];  // (unused past the last step)
+                a.dp_out = dp2;
+                if ((rc = born_pair_maps(ctx, a, &M))) return rc;
+                launch_born_pair(a, active_tiles(P, n), M, st);
+                ctx->stats.cell_updates += active_cells(P, n + 1, ctx->NZ);
+                std::swap(a.dp, dp2);
+            } else {
+                if ((rc = born_hist_maps(ctx, a, &M))) return rc;
+                launch_born_hist_step(a, active_tiles(P, n), M, st);
+            }
             ctx->stats.kernel_launches++;
             ctx->stats.cell_updates += active_cells(P, n, ctx->NZ);
             std::swap(p, pn);
         }
         ctx->stats.reused |= 2;
+        phase_end(ctx, 2, st, ctx->stats.kernel_launches - l0, ctx->stats.cell_updates - c0);
+        return end_call(ctx);
+    }
+    if (time_blocking(ctx, 2)) {  // two steps per launch
+        for (int n = 0; n < P.nt_max; n += 2) {
+            a.u = u;
+            a.un = un;
+            a.p = p;
+            a.pn = pn;
+            a.du_out = du2;
+            a.dp_out = dp2;
+            a.n = n;
+            TileMaps M;
+            if ((rc = born_joint_maps(ctx, a, &M))) return rc;
+            launch_born_joint(a, active_tiles(P, n), M, st);
+            ctx->stats.kernel_launches++;
+            ctx->stats.cell_updates += 2 * (active_cells(P, n, ctx->NZ) + active_cells(P, n + 1, ctx->NZ));
+            std::swap(u, un);
+            std::swap(p, pn);
+            std::swap(a.du, du2);
+            std::swap(a.dp, dp2);
+        }
         phase_end(ctx, 2, st, ctx->stats.kernel_launches - l0, ctx->stats.cell_updates - c0);
         return end_call(ctx);
     }

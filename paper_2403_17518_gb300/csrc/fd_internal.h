@@ -173,6 +173,11 @@ struct BornArgs {
     // Background term a^n = D u0^n + q^n read from a stored forward history
     // (launch_born_hist_step; the u fields are then not used).
     const float *a = nullptr;
+    // Two-step kernels only (steps n and n+1): D^n of the fields is du and dp,
+    // D^{n+2} goes to du_out and dp_out, u0^{n+2} to un, p^{n+2} to pn; from the
+    // history, a2 = a^{n+1}.
+    float *du_out = nullptr, *dp_out = nullptr;
+    const float *a2 = nullptr;
 };
 
 // Step-kernel variants.  Variants 0-2: tiles staged by per-thread cp.async,
@@ -213,6 +218,12 @@ void launch_born_step_tma(const BornArgs &a, int ntiles, int variant, int grid, 
 // 0 p^n halo, 1 D_p, 2 kappa, 3 d kappa, 4 a^n cell box): only the
 // scattered field is advanced; the same bits as the joint step.
 void launch_born_hist_step(const BornArgs &a, int ntiles, const TileMaps &maps, cudaStream_t s);
+// Two such steps, n and n+1, of the tiles active at step n (fd_tma2.cu; maps:
+// 0 p^n HALO2 box, 1 D_p halo box, 2 a^n and 3 a^{n+1} cell boxes).
+void launch_born_pair(const BornArgs &a, int ntiles, const TileMaps &maps, cudaStream_t s);
+// Two joint Born steps, n and n+1, of both fields (fd_tma2.cu; maps: 0 u0^n and
+// 1 p^n HALO2 boxes, 2 D_u0 and 3 D_p halo boxes).
+void launch_born_joint(const BornArgs &a, int ntiles, const TileMaps &maps, cudaStream_t s);
 int tma_occupancy(int kind, int variant);
 
 struct StepLaunch {

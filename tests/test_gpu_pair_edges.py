@@ -57,8 +57,14 @@ def _run(c, v, blocking, history, monkeypatch):
     J, g = ctx.fwi_gradient(vd, geom, 0.5 * d, d_syn=ds)
     b = ctx.born_demig(vd, geom, to_dev(f32(synth.gaussian_field(v.shape, seed=12))))
     m = ctx.rtm_mig(vd, geom, d)
-    out = [to_host(x) for x in (d, ds, g, b, m)] + [J]
+    # Born from the forward pass that the gradient stored (all of it, or recomputed segments).
+    ctx.set_reuse(True)
+    ctx.fwi_gradient(vd, geom, 0.5 * d)
+    br = ctx.born_demig(vd, geom, to_dev(f32(synth.gaussian_field(v.shape, seed=12))))
+    assert ctx.stats()["reused"] == (0 if history else 2)
+    out = [to_host(x) for x in (d, ds, g, b, m, br)] + [J]
     ctx.close()
+    np.testing.assert_array_equal(out[3], out[5])
     return out
 
 
@@ -68,6 +74,6 @@ def test_two_steps_equal_one_step_at_the_edges(shape, history, monkeypatch):
     c, v = _case(*shape)
     one = _run(c, v, False, history, monkeypatch)
     two = _run(c, v, True, history, monkeypatch)
-    assert np.all(np.isfinite(one[0])) and np.linalg.norm(one[0]) > 0
+    assert np.all(np.isfinite(one[0])) and np.linalg.norm(one[0]) > 0 and np.linalg.norm(one[3]) > 0
     for a, b in zip(one, two):
         np.testing.assert_array_equal(a, b)
