@@ -39,16 +39,14 @@ struct Plan {
     std::vector<TileRec> recs;
     std::vector<TileInfo> infos;       // per tile, same order (no sentinel)
     std::vector<int> tiles_prefix;     // tiles of the first m slots
-    std::vector<int> rtiles;           // tiles with receivers, in tile order
-    std::vector<int> rtiles_prefix;    // of those, the tiles of the first m slots
     std::vector<TileRec> xrecs;        // receivers of each tile's grown region (StepCommon::xrecs)
     std::vector<int> xrec_off;         // per tile, with a final end offset
-    bool xinj = false;                 // every grown region holds at most kInjCap entries
     long long pool_floats = 0;
     int pitch = 0;                     // row pitch of every window in a pool
     long long n_data = 0;
     long long cells_per_step_all = 0;  // padded cells of all shots
-    DevBuf d_shots, d_tiles, d_recs, d_slot_of, d_wav, d_infos, d_rtiles, d_xrecs, d_xrec_off, d_sponge;
+    DevBuf d_shots, d_tiles, d_recs, d_slot_of, d_wav, d_infos, d_xrecs, d_xrec_off, d_sponge;
+    DevBuf d_act, d_done;              // FlowArgs::act (nt_max entries), FlowArgs::done (one per tile)
     int nwz = 0;                       // row factors at the head of d_sponge, then the slots' column factors
 };
 
@@ -70,6 +68,7 @@ struct dhfwi_ctx {
     // Step n holds the active slots only: hoff[n] is its offset in floats.
     DevBuf hist;
     std::vector<long long> hoff;
+    DevBuf d_hoff;          // the same on the device
     int hist_segs = 0;
     unsigned long long hist_plan = 0;  // plan hash and limit the split was made for
     long long hist_limit = -2;
@@ -283,11 +282,8 @@ int get_plan(dhfwi_ctx *ctx, const dhfwi_geom *G) {
     P.tiles.clear();
     P.recs.clear();
     P.tiles_prefix.assign(ns + 1, 0);
-    P.rtiles.clear();
-    P.rtiles_prefix.assign(ns + 1, 0);
     P.xrecs.clear();
     P.xrec_off.clear();
-    P.xinj = true;
     // One row pitch for all windows: a pool is then a [slot][NZ][pitch] array
     // that a single 3-D tensor map describes.
     int pitch = POOL_ALIGN;
@@ -357,16 +353,9 @@ int get_plan(dhfwi_ctx *ctx, const dhfwi_geom *G) {
                     return a.cell < b.cell || (a.cell == b.cell && a.r < b.r);
                 });
                 P.xrec_off.push_back((int)P.xrecs.size());
-                if ((int)bk.size() > kInjCap) P.xinj = false;
                 for (const TileRec &e : bk) P.xrecs.push_back(e);
             }
         }
-        for (int ti = P.tiles_prefix[k]; ti < P.tiles_prefix[k + 1]; ti++) {
-            const int rb = P.tiles[ti].rec_begin;
-            const int re = ti + 1 < (int)P.tiles.size() ? P.tiles[ti + 1].rec_begin : (int)P.recs.size();
-            if (re > rb) P.rtiles.push_back(ti);
-        }
-        P.rtiles_prefix[k + 1] = (int)P.rtiles.size();
     }
     P.xrec_off.push_back((int)P.xrecs.size());  // end of the last tile's list
     if (P.xrecs.empty()) P.xrecs.push_back(TileRec{0, 0});  // (a valid device pointer)
@@ -412,7 +401,13 @@ int get_plan(dhfwi_ctx *ctx, const dhfwi_geom *G) {
     if ((rc = upload(ctx, P.d_slot_of, P.slot_of_shot, "slot table"))) return rc;
     if ((rc = upload(ctx, P.d_wav, wav, "wavelets"))) return rc;
     if ((rc = upload(ctx, P.d_infos, P.infos, "tile descriptors"))) return rc;
-    if ((rc = upload(ctx, P.d_rtiles, P.rtiles, "receiver tile list"))) return rc;
+    std::vector<int> act(P.nt_max);
+    for (int n = 0, k = ns; n < P.nt_max; n++) {  // slots by record length: the active ones are a prefix
+        while (k > 0 && P.nt_sorted[k - 1] <= n) k--;
+        act[n] = P.tiles_prefix[k];
+    }
+    if ((rc = upload(ctx, P.d_act, act, "active tile counts"))) return rc;
+    if ((rc = ensure(ctx, P.d_done, sizeof(unsigned) * P.infos.size(), "tile progress"))) return rc;
     if ((rc = upload(ctx, P.d_xrecs, P.xrecs, "grown-region receiver table"))) return rc;
     if ((rc = upload(ctx, P.d_xrec_off, P.xrec_off, "grown-region receiver offsets"))) return rc;
     // Sponge factors of the rows and of each slot's columns.
@@ -471,10 +466,8 @@ StepCommon common(dhfwi_ctx *ctx) {
     c.tflag = (unsigned *)ctx->status.p + TFLAG_WORD;
     c.wz = (const float *)ctx->plan.d_sponge.p;
     c.wx = c.wz + ctx->plan.nwz;
-    if (ctx->plan.xinj) {
-        c.xrecs = (const TileRec *)ctx->plan.d_xrecs.p;
-        c.xrec_off = (const int *)ctx->plan.d_xrec_off.p;
-    }
+    c.xrecs = (const TileRec *)ctx->plan.d_xrecs.p;
+    c.xrec_off = (const int *)ctx->plan.d_xrec_off.p;
     return c;
 }
 
@@ -832,48 +825,6 @@ bool time_blocking(const dhfwi_ctx *ctx, int which) {
     return ctx->depth[which] == 2;
 }
 
-// Maps of a two-step forward launch (u^n with the doubled halo, D^n with
-// its ring).
-int pair_maps(dhfwi_ctx *ctx, const FwdArgs &a, TileMaps *M) {
-    int rc;
-    if ((rc = tensor_map(ctx, a.u, MAP_POOL_HALO2, &M->m[0]))) return rc;
-    return tensor_map(ctx, a.dd, MAP_POOL_HALO, &M->m[1]);
-}
-
-// Maps of a two-step adjoint launch (nu^{k+1} with the doubled halo, D_nu
-// with its ring; the image, a^{k-1} and a^{k-2}, which
-// the kernel only prefetches into L2).  A history step's map spans all
-// slots from its base: the spare pool at the history's end keeps it inside
-// the allocation.
-int adj_pair_maps(dhfwi_ctx *ctx, const AdjArgs &b, TileMaps *M) {
-    int rc;
-    if ((rc = tensor_map(ctx, b.nu, MAP_POOL_HALO2, &M->m[0]))) return rc;
-    if ((rc = tensor_map(ctx, b.dd, MAP_POOL_HALO, &M->m[1]))) return rc;
-    if ((rc = tensor_map(ctx, b.g, MAP_POOL_CELL, &M->m[3]))) return rc;
-    if ((rc = tensor_map(ctx, b.a, MAP_POOL_CELL, &M->m[4]))) return rc;
-    return tensor_map(ctx, b.a2, MAP_POOL_CELL, &M->m[5]);
-}
-
-// Maps of a two-step Born launch (p^n with the doubled halo, D_p with its
-// ring; a^n and a^{n+1}, which the kernel only prefetches into L2).
-int born_pair_maps(dhfwi_ctx *ctx, const BornArgs &b, TileMaps *M) {
-    int rc;
-    if ((rc = tensor_map(ctx, b.p, MAP_POOL_HALO2, &M->m[0]))) return rc;
-    if ((rc = tensor_map(ctx, b.dp, MAP_POOL_HALO, &M->m[1]))) return rc;
-    if ((rc = tensor_map(ctx, b.a, MAP_POOL_CELL, &M->m[2]))) return rc;
-    return tensor_map(ctx, b.a2, MAP_POOL_CELL, &M->m[3]);
-}
-
-// Maps of a two-step joint Born launch (u0^n and p^n with the doubled halo,
-// D_u0 and D_p with their rings).
-int born_joint_maps(dhfwi_ctx *ctx, const BornArgs &b, TileMaps *M) {
-    int rc;
-    if ((rc = tensor_map(ctx, b.u, MAP_POOL_HALO2, &M->m[0]))) return rc;
-    if ((rc = tensor_map(ctx, b.p, MAP_POOL_HALO2, &M->m[1]))) return rc;
-    if ((rc = tensor_map(ctx, b.du, MAP_POOL_HALO, &M->m[2]))) return rc;
-    return tensor_map(ctx, b.dp, MAP_POOL_HALO, &M->m[3]);
-}
-
 // Maps of a one-step Born launch from the history (p^n halo, D_p, kappa, d
 // kappa, a^n).
 int born_hist_maps(dhfwi_ctx *ctx, const BornArgs &b, TileMaps *M) {
@@ -885,83 +836,221 @@ int born_hist_maps(dhfwi_ctx *ctx, const BornArgs &b, TileMaps *M) {
     return tensor_map(ctx, b.a, MAP_POOL_CELL, &M->m[4]);
 }
 
+// ---------------------------------------------------------------------------
+// Two-step launches (fd_tma2.cu).  A launch takes at most FLOW_PAIRS step pairs,
+// so that it ends within a fraction of a second at any size; one pair when all
+// its tiles are resident at once (see flow_pairs).
+// ---------------------------------------------------------------------------
+constexpr int FLOW_PAIRS = 256;
+
+// The slots [s0, s1) that a sequence of two-step launches advances through all
+// its steps before the next ones.
+struct Group {
+    int s0, s1;
+};
+
+int group_nt(const Plan &P, const Group &g) { return P.nt_sorted[g.s0]; }  // its longest record
+
+// Cells of the group's shots active at step n.
+long long group_cells(const Plan &P, const Group &g, int n, int NZ) {
+    long long c = 0;
+    for (int k = g.s0; k < g.s1 && P.nt_sorted[k] > n; k++) c += (long long)P.shots[k].nxw * NZ;
+    return c;
+}
+
+// Step pairs per launch.  With at most one tile per resident CTA every tile
+// waits for its neighbours' stores of the pair before either way, and the end of
+// a launch (its successor a programmatic dependent) passes them on faster than
+// the per-tile flags: 101 x 101, 4 shots (36 tiles), 4.6 us per pair against
+// 6.2; from the second tile per CTA on the flags win (150 x 500, 25 shots, 525
+// tiles, migration: 14.5 ms against 16.5).
+int flow_pairs(const Plan &P, const Group &g, int kind) {
+    return P.tiles_prefix[g.s1] - P.tiles_prefix[g.s0] <= flow_ctas(kind) ? 1 : FLOW_PAIRS;
+}
+
+// Common part of a launch over the group's tiles that are active at step n_any,
+// the step of the launch at which most of them are; zeroes their progress.
+int flow_args(dhfwi_ctx *ctx, const Group &g, int n_any, int npairs, FlowArgs *f, cudaStream_t st) {
+    const Plan &P = ctx->plan;
+    f->t0 = P.tiles_prefix[g.s0];
+    f->nt = std::min(active_tiles(P, n_any), P.tiles_prefix[g.s1]) - f->t0;
+    f->npairs = npairs;
+    f->act = (const int *)P.d_act.p;
+    f->done = (unsigned *)P.d_done.p;
+    if (npairs > 1) CK(cudaMemsetAsync(f->done + f->t0, 0, sizeof(unsigned) * f->nt, st));
+    return DHFWI_OK;
+}
+
+// Halo maps of both buffers of a field (HALO2 boxes) and of its D (halo boxes).
+int flow_maps(dhfwi_ctx *ctx, float *const u[2], float *const d[2], CUtensorMap *mu, CUtensorMap *md) {
+    int rc;
+    for (int i = 0; i < 2; i++) {
+        if ((rc = tensor_map(ctx, u[i], MAP_POOL_HALO2, mu + i))) return rc;
+        if ((rc = tensor_map(ctx, d[i], MAP_POOL_HALO, md + i))) return rc;
+    }
+    return DHFWI_OK;
+}
+
+// Steps [n0, n1) of the group's shots, n1 - n0 even or n1 past their longest
+// record: the forward state (u in *cur, D in *dcur; the others are scratch and
+// take turns).  a holds what the launch stores and samples.
+int fwd_flow(dhfwi_ctx *ctx, FwdFlow &a, const Group &g, int n0, int n1, float *&cur, float *&nxt, float *&dcur,
+             float *&dnxt, cudaStream_t st) {
+    n1 = std::min(n1, group_nt(ctx->plan, g));
+    const int most = flow_pairs(ctx->plan, g, FLOW_FWD);
+    for (int n = n0; n < n1; n += 2 * most) {
+        const int np = std::min(most, (n1 - n + 1) / 2);
+        int rc;
+        if ((rc = flow_args(ctx, g, n, np, &a.f, st))) return rc;
+        a.n0 = n;
+        a.u[0] = cur;
+        a.u[1] = nxt;
+        a.d[0] = dcur;
+        a.d[1] = dnxt;
+        TileMaps M;
+        if ((rc = flow_maps(ctx, a.u, a.d, &M.m[0], &M.m[2]))) return rc;
+        launch_fwd_flow(a, M, st);
+        ctx->stats.kernel_launches++;
+        for (int i = n; i < n + 2 * np && i < n1; i++) ctx->stats.cell_updates += group_cells(ctx->plan, g, i, ctx->NZ);
+        if (np & 1) {
+            std::swap(cur, nxt);
+            std::swap(dcur, dnxt);
+        }
+    }
+    CK(cudaGetLastError());
+    return DHFWI_OK;
+}
+
+// Adjoint steps k1 .. n0 + 1 (an even number) of the group's shots, state as
+// above; those with shorter records join as k comes down to them.
+int adj_flow(dhfwi_ctx *ctx, AdjFlow &b, const Group &g, int k1, int n0, float *&cur, float *&nxt, float *&dcur,
+             float *&dnxt, cudaStream_t st) {
+    const int most = flow_pairs(ctx->plan, g, FLOW_ADJ);
+    for (int k = k1; k > n0; k -= 2 * most) {
+        const int np = std::min(most, (k - n0) / 2);
+        int rc;
+        if ((rc = flow_args(ctx, g, k - 2 * np, np, &b.f, st))) return rc;
+        b.k1 = k;
+        b.nu[0] = cur;
+        b.nu[1] = nxt;
+        b.d[0] = dcur;
+        b.d[1] = dnxt;
+        TileMaps M;
+        if ((rc = flow_maps(ctx, b.nu, b.d, &M.m[0], &M.m[2]))) return rc;
+        launch_adj_flow(b, M, st);
+        ctx->stats.kernel_launches++;
+        for (int i = k - 2 * np; i < k; i++) ctx->stats.cell_updates += group_cells(ctx->plan, g, i, ctx->NZ);
+        if (np & 1) {
+            std::swap(cur, nxt);
+            std::swap(dcur, dnxt);
+        }
+    }
+    CK(cudaGetLastError());
+    return DHFWI_OK;
+}
+
+// Born steps [0, n1) of the group's shots from zero state: both fields, or
+// (from_history) the scattered one with a^n from b.a.
+int born_flow(dhfwi_ctx *ctx, BornFlow b, const Group &g, int n1, bool from_history, cudaStream_t st) {
+    n1 = std::min(n1, group_nt(ctx->plan, g));
+    const int most = flow_pairs(ctx->plan, g, from_history ? FLOW_BORN_HIST : FLOW_BORN);
+    for (int n = 0; n < n1; n += 2 * most) {
+        const int np = std::min(most, (n1 - n + 1) / 2);
+        int rc;
+        if ((rc = flow_args(ctx, g, n, np, &b.f, st))) return rc;
+        b.n0 = n;
+        TileMaps M;
+        if (from_history) {
+            if ((rc = flow_maps(ctx, b.p, b.dp, &M.m[0], &M.m[2]))) return rc;
+            launch_born_hist_flow(b, M, st);
+        } else {
+            if ((rc = flow_maps(ctx, b.u, b.du, &M.m[0], &M.m[4]))) return rc;
+            if ((rc = flow_maps(ctx, b.p, b.dp, &M.m[2], &M.m[6]))) return rc;
+            launch_born_joint_flow(b, M, st);
+        }
+        ctx->stats.kernel_launches++;
+        for (int i = n; i < n + 2 * np && i < n1; i++)
+            ctx->stats.cell_updates += (from_history ? 1 : 2) * group_cells(ctx->plan, g, i, ctx->NZ);
+        if (np & 1) {
+            std::swap(b.u[0], b.u[1]);
+            std::swap(b.du[0], b.du[1]);
+            std::swap(b.p[0], b.p[1]);
+            std::swap(b.dp[0], b.dp[1]);
+        }
+    }
+    CK(cudaGetLastError());
+    return DHFWI_OK;
+}
+
+// Groups of the slots for the two-step launches: all of them together.
+std::vector<Group> groups_of(const Plan &P) { return {Group{0, P.n_shots}}; }
+
 // Time-blocking depth of the forward and the adjoint sweeps, of Born and of
-// Born from the history: `reps` launches of the two-step kernel(s) on the
-// plan's full tile list against twice the chosen one-step kernel's time for as
-// many launches (one_step_ms: the variant loop's best time of `reps` launches
-// per kind: forward, forward with store, adjoint, Born).  The faster depth is
-// kept.
+// Born from the history: a two-step launch of a few pairs on the plan's full
+// tile list against the chosen one-step kernel's time for as many steps
+// (one_step_ms: the variant loop's best time of `reps` launches per kind:
+// forward, forward with store, adjoint, Born).  The faster depth is kept.
 int tune_depth(dhfwi_ctx *ctx, cudaStream_t st, const float *one_step_ms, int reps) {
     if (!encode_tiled()) return DHFWI_OK;
     const Plan &P = ctx->plan;
     const long long pool = P.pool_floats;
     float *F = (float *)ctx->fields.p;
-    const int ntiles = active_tiles(P, 0);
+    const int np = std::min(4, P.nt_max / 2);  // pairs timed
+    for (int &d : ctx->depth) d = 1;
+    if (np == 0) return DHFWI_OK;
+    const Group all{0, P.n_shots};
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
     int rc = DHFWI_OK;
-    float hist_ms = 0.f;  // one step of Born from the history
+    float hist_ms = 0.f;  // Born from the history, one step per launch
     // which: 0 forward, 1 adjoint, 2 Born, 3 one step of Born from the history, 4 two of them.
     for (int which = 0; which < 5 && !rc; which++) {
         float ms = 0.f;
-        for (int rep = -1; rep < reps && !rc; rep++) {
-            if (rep == 0) cudaEventRecord(e0, st);
-            TileMaps M;
+        for (int rep = 0; rep < 2 && !rc; rep++) {  // one warm-up
+            if (rep == 1) cudaEventRecord(e0, st);
             if (which == 0) {
-                FwdArgs a{};
+                FwdFlow a{};
                 a.c = common(ctx);
-                a.u = F;
-                a.un = F + pool;
-                a.dd = F + 2 * pool;
-                a.dd_out = F + 7 * pool;
-                a.d = (float *)ctx->dtmp.p;
-                a.n = 0;
-                if (!(rc = pair_maps(ctx, a, &M))) launch_fwd_pair(a, ntiles, M, st);
-                ctx->stats.kernel_launches++;
-            }
-            if (which >= 2 && !rc) {
+                a.rec = (float *)ctx->dtmp.p;
+                float *u = F, *un = F + pool, *d = F + 2 * pool, *dn = F + 7 * pool;
+                rc = fwd_flow(ctx, a, all, 0, 2 * np, u, un, d, dn, st);
+            } else if (which == 1) {
+                AdjFlow b{};
+                b.c = common(ctx);
+                b.a.base = F + 3 * pool;
+                b.g = F + 4 * pool;
+                b.r = (const float *)ctx->rtmp.p;
+                float *u = F, *un = F + pool, *d = F + 2 * pool, *dn = F + 8 * pool;
+                rc = adj_flow(ctx, b, all, 2 * np, 0, u, un, d, dn, st);
+            } else if (which == 3) {
                 BornArgs b{};
                 b.c = common(ctx);
                 b.p = F + 3 * pool;
                 b.pn = F + 4 * pool;
                 b.dp = F + 5 * pool;
-                b.dp_out = F + 6 * pool;
                 b.dkap = (const float *)ctx->kap.p;
                 b.d = (float *)ctx->dtmp.p;
-                b.u = F;
-                b.un = F + pool;
-                b.du = F + 2 * pool;
-                b.du_out = F + 7 * pool;
-                b.a = F;
-                b.a2 = F + pool;
-                b.n = 0;
-                if (which == 2) {
-                    if (!(rc = born_joint_maps(ctx, b, &M))) launch_born_joint(b, ntiles, M, st);
-                } else if (which == 3) {
-                    if (!(rc = born_hist_maps(ctx, b, &M))) launch_born_hist_step(b, ntiles, M, st);
-                } else {
-                    if (!(rc = born_pair_maps(ctx, b, &M))) launch_born_pair(b, ntiles, M, st);
-                }
-                ctx->stats.kernel_launches++;
-            }
-            if (which == 1) {
-                AdjArgs b{};
+                b.a = F + 8 * pool;
+                TileMaps M;
+                for (int i = 0; i < 2 * np && !rc; i++)
+                    if (!(rc = born_hist_maps(ctx, b, &M))) launch_born_hist_step(b, active_tiles(P, 0), M, st);
+                ctx->stats.kernel_launches += 2 * np;
+            } else {
+                BornFlow b{};
                 b.c = common(ctx);
-                b.nu = F;
-                b.nun = F + pool;
-                b.dd = F + 2 * pool;
-                b.dd_out = F + 8 * pool;
-                b.a = F + 3 * pool;
-                b.a2 = F + 5 * pool;
-                b.g = F + 4 * pool;
-                b.r = (const float *)ctx->rtmp.p;
-                b.k = 2;
-                b.inject_here = P.xinj ? 1 : 0;
-                const int nrt = P.xinj ? 0 : P.rtiles_prefix[active_slots(P, 1)];
-                launch_adj_inject(b, (const int *)P.d_rtiles.p, nrt, st);
-                if (!(rc = adj_pair_maps(ctx, b, &M))) launch_adj_pair(b, ntiles, M, st);
-                ctx->stats.kernel_launches += 1 + (nrt > 0);
+                b.dkap = (const float *)ctx->kap.p;
+                b.rec = (float *)ctx->dtmp.p;
+                b.a.base = F + 8 * pool;
+                b.u[0] = F;
+                b.u[1] = F + pool;
+                b.du[0] = F + 2 * pool;
+                b.du[1] = F + 7 * pool;
+                b.p[0] = F + 3 * pool;
+                b.p[1] = F + 4 * pool;
+                b.dp[0] = F + 5 * pool;
+                b.dp[1] = F + 6 * pool;
+                rc = born_flow(ctx, b, all, 2 * np, which == 4, st);
             }
         }
         cudaEventRecord(e1, st);
@@ -977,8 +1066,8 @@ int tune_depth(dhfwi_ctx *ctx, cudaStream_t st, const float *one_step_ms, int re
             hist_ms = ms;
             continue;
         }
-        const float one = which == 4 ? hist_ms : one_step_ms[which == 0 ? 0 : which + 1];
-        ctx->depth[which == 4 ? 3 : which] = ms <= 2.f * one ? 2 : 1;
+        const float one = which == 4 ? hist_ms : one_step_ms[which == 0 ? 0 : which + 1] * (2.f * np / reps);
+        ctx->depth[which == 4 ? 3 : which] = ms <= one ? 2 : 1;
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -989,39 +1078,24 @@ int tune_depth(dhfwi_ctx *ctx, cudaStream_t st, const float *one_step_ms, int re
     return DHFWI_OK;
 }
 
-// Advances the forward state from step n: two steps with one two-step launch
-// when blocking is on and n + 1 < n_end, else one.  State: u in *cur (next
-// in *nxt), D in *dcur (*dnxt: the two-step kernel's output pool).  a_slot(n)
-// gives the segment slot for a^n (nullptr: no segment store).  Returns the
-// number of steps taken, or a negative error code.
+// Advances the forward state by step n, one step per launch.  State: u in *cur
+// (next in *nxt), D in place.  a_slot(n) gives the slot for a^n (nullptr: no
+// store).
 template <typename SlotFn>
-int forward_steps(dhfwi_ctx *ctx, FwdArgs &a, int n, int n_end, float *&cur, float *&nxt, float *&dcur,
-                  float *&dnxt, const StepLaunch &L, bool blocking, SlotFn a_slot, cudaStream_t st) {
+int forward_step(dhfwi_ctx *ctx, FwdArgs &a, int n, float *&cur, float *&nxt, float *d, const StepLaunch &L,
+                 SlotFn a_slot, cudaStream_t st) {
     const Plan &P = ctx->plan;
     a.u = cur;
     a.un = nxt;
-    a.dd = dcur;
+    a.dd = d;
     a.n = n;
     a.a_out = a_slot(n);
-    int rc;
-    if (blocking && n + 1 < n_end) {
-        a.dd_out = dnxt;
-        a.a_out2 = a.a_out ? a_slot(n + 1) : nullptr;
-        TileMaps M;
-        if ((rc = pair_maps(ctx, a, &M))) return rc;
-        launch_fwd_pair(a, active_tiles(P, n), M, st);
-        ctx->stats.kernel_launches++;
-        ctx->stats.cell_updates += active_cells(P, n, ctx->NZ) + active_cells(P, n + 1, ctx->NZ);
-        std::swap(cur, nxt);
-        std::swap(dcur, dnxt);
-        return 2;
-    }
-    a.dd_out = a.a_out2 = nullptr;
-    if ((rc = fwd_step(ctx, a, active_tiles(P, n), L, st))) return rc;
+    const int rc = fwd_step(ctx, a, active_tiles(P, n), L, st);
+    if (rc) return rc;
     ctx->stats.kernel_launches++;
     ctx->stats.cell_updates += active_cells(P, n, ctx->NZ);
     std::swap(cur, nxt);
-    return 1;
+    return DHFWI_OK;
 }
 
 // Forward pass over all steps.  State pools uA (u^0), uB (scratch), dd
@@ -1032,35 +1106,59 @@ int forward_steps(dhfwi_ctx *ctx, FwdArgs &a, int n, int n_end, float *&cur, flo
 int run_forward(dhfwi_ctx *ctx, float *uA, float *uB, float *dd, float *dd2, float *d, bool backward,
                 cudaStream_t st) {
     const Plan &P = ctx->plan;
-    FwdArgs a{};
-    a.c = common(ctx);
-    a.d = d;
-    float *cur = uA, *nxt = uB, *dcur = dd, *dnxt = dd2;
     const long long pool = P.pool_floats;
-    const bool blocking = time_blocking(ctx, 0);
     const int K = ctx->ck_every, S = backward ? ctx->hist_segs : 0;
     const int H = std::min(S * K, P.nt_max);  // steps whose a^n are stored
     float *ck = (float *)ctx->ck.p, *hist = (float *)ctx->hist.p;
-    auto slot = [&](int n) -> float * { return n < H ? hist + ctx->hoff[n] : nullptr; };
     const long long l0 = ctx->stats.kernel_launches, c0 = ctx->stats.cell_updates;
     if (backward) ctx->fws.valid = false;  // the history and checkpoints are about to change
     phase_begin(ctx, 0, st);
-    for (int n = 0; n < P.nt_max;) {
-        // K and H are even and two-step launches start at even n: a launch
-        // never straddles a segment or the end of the history.
-        if (backward && n >= H && n % K == 0) {
-            const long long j = n / K - S;
-            a.ck_u = ck + (2 * j) * pool;
-            a.ck_d = ck + (2 * j + 1) * pool;
-        } else {
-            a.ck_u = a.ck_d = nullptr;
+    int rc;
+    if (time_blocking(ctx, 0)) {
+        // K and H are even (or H is the last step): a pair never straddles a
+        // segment or the end of the history.
+        for (const Group &g : groups_of(P)) {
+            float *cur = uA, *nxt = uB, *dcur = dd, *dnxt = dd2;
+            const long long cn = ctx->stats.cell_updates;
+            if (H > 0) {
+                FwdFlow a{};
+                a.c = common(ctx);
+                a.rec = d;
+                a.a.base = hist;
+                a.a.off = (const long long *)ctx->d_hoff.p;
+                a.a.last = H - 1;
+                if ((rc = fwd_flow(ctx, a, g, 0, H, cur, nxt, dcur, dnxt, st))) return rc;
+                ctx->stats.history_cells += ctx->stats.cell_updates - cn;
+            }
+            FwdFlow a{};
+            a.c = common(ctx);
+            a.rec = d;
+            if (backward && H < P.nt_max) {
+                a.ck = ck;
+                a.ck_every = K;
+                a.ck_first = S;
+                a.pool = pool;
+            }
+            if ((rc = fwd_flow(ctx, a, g, H, P.nt_max, cur, nxt, dcur, dnxt, st))) return rc;
         }
-        const long long cn = ctx->stats.cell_updates;
-        const int rc = forward_steps(ctx, a, n, P.nt_max, cur, nxt, dcur, dnxt, ctx->launch[n < H ? 1 : 0], blocking,
-                                     slot, st);
-        if (rc < 0) return rc;
-        if (n < H) ctx->stats.history_cells += ctx->stats.cell_updates - cn;
-        n += rc;
+    } else {
+        FwdArgs a{};
+        a.c = common(ctx);
+        a.d = d;
+        float *cur = uA, *nxt = uB;
+        auto slot = [&](int n) -> float * { return n < H ? hist + ctx->hoff[n] : nullptr; };
+        for (int n = 0; n < P.nt_max; n++) {
+            if (backward && n >= H && n % K == 0) {
+                const long long j = n / K - S;
+                a.ck_u = ck + (2 * j) * pool;
+                a.ck_d = ck + (2 * j + 1) * pool;
+            } else {
+                a.ck_u = a.ck_d = nullptr;
+            }
+            const long long cn = ctx->stats.cell_updates;
+            if ((rc = forward_step(ctx, a, n, cur, nxt, dd, ctx->launch[n < H ? 1 : 0], slot, st))) return rc;
+            if (n < H) ctx->stats.history_cells += ctx->stats.cell_updates - cn;
+        }
     }
     if (backward) {
         ctx->stats.history_steps = H;
@@ -1098,77 +1196,87 @@ int run_backward(dhfwi_ctx *ctx, float *w, float *w2, float *w3, float *w4, floa
     const Plan &P = ctx->plan;
     const long long pool = P.pool_floats;
     const int K = ctx->ck_every, S = ctx->hist_segs;
-    const int nseg = (P.nt_max + K - 1) / K;
+    const int H = std::min(S * K, P.nt_max);  // steps whose a^n are stored
     const bool blocking = time_blocking(ctx, 0), blocking_adj = time_blocking(ctx, 1);
     float *ck = (float *)ctx->ck.p, *abuf = (float *)ctx->abuf.p, *hist = (float *)ctx->hist.p;
-    FwdArgs f{};
-    f.c = common(ctx);
-    AdjArgs b{};
-    b.c = f.c;
-    b.r = r;
-    b.g = gpool;
-    float *ncur = nuA, *nnxt = nuB, *dcur_nu = nud, *dnxt_nu = nud2;
     const long long l0 = ctx->stats.kernel_launches, c0 = ctx->stats.cell_updates;
+    int rc;
     phase_begin(ctx, 1, st);
-    for (int js = nseg - 1; js >= 0; js--) {
-        const int n0 = js * K, n1 = std::min(n0 + K, P.nt_max);
-        const bool stored = js < S;
-        auto slot = [&](int n) -> float * {
-            return stored ? hist + ctx->hoff[n] : abuf + (long long)(n - n0) * pool;
+    // Groups share no state, so each goes back through all its steps by itself
+    // (one group when a part of the sweep takes one step per launch).
+    const std::vector<Group> groups = blocking && blocking_adj ? groups_of(P) : std::vector<Group>{{0, P.n_shots}};
+    for (const Group &g : groups) {
+        const int nt = group_nt(P, g);
+        const int t0 = P.tiles_prefix[g.s0];
+        const size_t goff = P.shots[g.s0].foff, glen = (size_t)(g.s1 - g.s0) * ctx->NZ * P.pitch;
+        float *ncur = nuA, *nnxt = nuB, *dcur_nu = nud, *dnxt_nu = nud2;
+        // The adjoint over the steps n1 .. n0 + 1, a^n from sa.
+        auto adjoint = [&](int n0, int n1, const ASteps &sa, auto slot) -> int {
+            AdjArgs b{};
+            b.c = common(ctx);
+            b.c.infos += t0;
+            b.c.tiles += t0;
+            b.r = r;
+            b.g = gpool;
+            int k = n1;
+            for (; k > n0 && (!blocking_adj || (k - n0) % 2); k--) {  // one step per launch
+                b.nu = ncur;
+                b.nun = nnxt;
+                b.dd = dcur_nu;
+                b.a = slot(k - 1);
+                b.k = k;
+                const int tiles = std::min(active_tiles(P, k - 1), P.tiles_prefix[g.s1]) - t0;
+                if ((rc = adj_step(ctx, b, tiles, ctx->launch[2], st))) return rc;
+                ctx->stats.kernel_launches++;
+                ctx->stats.cell_updates += group_cells(P, g, k - 1, ctx->NZ);
+                std::swap(ncur, nnxt);
+            }
+            if (k == n0) return DHFWI_OK;
+            AdjFlow f{};
+            f.c = common(ctx);
+            f.r = r;
+            f.g = gpool;
+            f.a = sa;
+            return adj_flow(ctx, f, g, k, n0, ncur, nnxt, dcur_nu, dnxt_nu, st);
         };
-        if (!stored) {
+        // Segments whose a^n is recomputed from checkpoints, the last first.
+        for (int js = (nt + K - 1) / K - 1; js >= S; js--) {
+            const int n0 = js * K, n1 = std::min(n0 + K, nt);
             float *cur = ck + (2 * (long long)(js - S)) * pool, *nxt = w;
             float *dcur = ck + (2 * (long long)(js - S) + 1) * pool, *dnxt = w2;
             if (ctx->reuse) {
-                CK(cudaMemcpyAsync(w3, cur, sizeof(float) * (size_t)pool, cudaMemcpyDeviceToDevice, st));
-                CK(cudaMemcpyAsync(w4, dcur, sizeof(float) * (size_t)pool, cudaMemcpyDeviceToDevice, st));
+                CK(cudaMemcpyAsync(w3 + goff, cur + goff, sizeof(float) * glen, cudaMemcpyDeviceToDevice, st));
+                CK(cudaMemcpyAsync(w4 + goff, dcur + goff, sizeof(float) * glen, cudaMemcpyDeviceToDevice, st));
                 cur = w3;
                 dcur = w4;
             } else {
                 ctx->fws.valid = false;
             }
-            f.d = nullptr;
-            f.ck_u = f.ck_d = nullptr;
-            for (int n = n0; n < n1;) {
-                const int rc = forward_steps(ctx, f, n, n1, cur, nxt, dcur, dnxt, ctx->launch[1], blocking, slot, st);
-                if (rc < 0) return rc;
-                n += rc;
+            ASteps sa;
+            sa.base = abuf;
+            sa.first = n0;
+            sa.stride = pool;
+            auto slot = [&](int n) -> float * { return abuf + (long long)(n - n0) * pool; };
+            if (blocking) {
+                FwdFlow f{};
+                f.c = common(ctx);
+                f.a = sa;
+                if ((rc = fwd_flow(ctx, f, g, n0, n1, cur, nxt, dcur, dnxt, st))) return rc;
+            } else {
+                FwdArgs f{};
+                f.c = common(ctx);
+                for (int n = n0; n < n1; n++)
+                    if ((rc = forward_step(ctx, f, n, cur, nxt, dcur, ctx->launch[1], slot, st))) return rc;
             }
+            if ((rc = adjoint(n0, n1, sa, slot))) return rc;
         }
-        for (int k = n1; k >= n0 + 1;) {
-            b.nu = ncur;
-            b.nun = nnxt;
-            b.dd = dcur_nu;
-            b.a = slot(k - 1);
-            b.k = k;
-            if (blocking_adj && k - 1 >= n0 + 1) {
-                // Steps k and k-1: the data of step k go into D_nu first (in
-                // the kernel's staged tiles, or by the separate pass when a
-                // tile's grown region holds too many receivers).
-                b.inject_here = P.xinj ? 1 : 0;
-                const int nrt = P.xinj ? 0 : P.rtiles_prefix[active_slots(P, k - 1)];
-                launch_adj_inject(b, (const int *)P.d_rtiles.p, nrt, st);
-                b.dd_out = dnxt_nu;
-                b.a2 = slot(k - 2);
-                TileMaps M;
-                int rc = adj_pair_maps(ctx, b, &M);
-                if (rc) return rc;
-                launch_adj_pair(b, active_tiles(P, k - 2), M, st);
-                ctx->stats.kernel_launches += 1 + (nrt > 0);
-                ctx->stats.cell_updates += active_cells(P, k - 1, ctx->NZ) + active_cells(P, k - 2, ctx->NZ);
-                std::swap(ncur, nnxt);
-                std::swap(dcur_nu, dnxt_nu);
-                k -= 2;
-                continue;
-            }
-            b.dd_out = nullptr;
-            b.a2 = nullptr;
-            int rc = adj_step(ctx, b, active_tiles(P, k - 1), ctx->launch[2], st);
-            if (rc) return rc;
-            ctx->stats.kernel_launches++;
-            ctx->stats.cell_updates += active_cells(P, k - 1, ctx->NZ);
-            std::swap(ncur, nnxt);
-            k--;
+        if (H > 0) {  // the stored steps
+            ASteps sa;
+            sa.base = hist;
+            sa.off = (const long long *)ctx->d_hoff.p;
+            sa.last = H - 1;
+            auto slot = [&](int n) -> float * { return hist + ctx->hoff[n]; };
+            if ((rc = adjoint(0, std::min(H, nt), sa, slot))) return rc;
         }
         CK(cudaGetLastError());
     }
@@ -1255,6 +1363,7 @@ int ensure_backward_ws_impl(dhfwi_ctx *ctx) {
             ctx->hoff[n] = off;
             off += (long long)active_slots(P, (int)n) * ctx->NZ * P.pitch;
         }
+        if (S > 0 && (rc = upload(ctx, ctx->d_hoff, ctx->hoff, "history offsets"))) return rc;
         ctx->hist_plan = P.hash;
         ctx->hist_limit = limit;
     }
@@ -1349,7 +1458,8 @@ void dhfwi_destroy(dhfwi_ctx *ctx) {
     DevBuf *bufs[] = {&ctx->kap, &ctx->dkap, &ctx->status, &ctx->partial, &ctx->fields,
                       &ctx->ck, &ctx->abuf, &ctx->hist, &ctx->dtmp, &ctx->rtmp, &ctx->plan.d_shots, &ctx->plan.d_tiles,
                       &ctx->plan.d_recs, &ctx->plan.d_slot_of, &ctx->plan.d_wav, &ctx->plan.d_infos,
-                      &ctx->plan.d_rtiles, &ctx->plan.d_xrecs, &ctx->plan.d_xrec_off, &ctx->plan.d_sponge};
+                      &ctx->plan.d_xrecs, &ctx->plan.d_xrec_off, &ctx->plan.d_sponge, &ctx->plan.d_act, &ctx->plan.d_done,
+                      &ctx->d_hoff};
     for (DevBuf *b : bufs) release(*b);
     if (ctx->h_status) cudaFreeHost(ctx->h_status);
     if (ctx->h_partial) cudaFreeHost(ctx->h_partial);
@@ -1481,58 +1591,51 @@ int born_demig(dhfwi_ctx *ctx, const float *v0_dev, const dhfwi_geom *geom, cons
     float *u = F, *un = F + pool, *p = F + 2 * pool, *pn = F + 3 * pool;
     a.du = F + 4 * pool;
     a.dp = F + 5 * pool;
-    float *du2 = F + 6 * pool, *dp2 = F + 7 * pool;  // second D pools of the two-step launches
+    BornFlow b{};  // two steps at a time
+    b.c = a.c;
+    b.dkap = a.dkap;
+    b.rec = d_dev;
+    b.u[0] = u;
+    b.u[1] = un;
+    b.p[0] = p;
+    b.p[1] = pn;
+    b.du[0] = a.du;
+    b.du[1] = F + 6 * pool;
+    b.dp[0] = a.dp;
+    b.dp[1] = F + 7 * pool;
     const long long l0 = ctx->stats.kernel_launches, c0 = ctx->stats.cell_updates;
     phase_begin(ctx, 2, st);
     // Background from the stored forward pass at this model (every step of
     // it in the history, TMA available): only the scattered field advances.
-    if (forward_reusable(ctx) && (long long)ctx->hist_segs * ctx->ck_every >= P.nt_max && encode_tiled()) {
+    const bool from_history =
+        forward_reusable(ctx) && (long long)ctx->hist_segs * ctx->ck_every >= P.nt_max && encode_tiled();
+    if (time_blocking(ctx, from_history ? 3 : 2)) {
+        if (from_history) {
+            b.a.base = (float *)ctx->hist.p;
+            b.a.off = (const long long *)ctx->d_hoff.p;
+            b.a.last = P.nt_max - 1;
+            ctx->stats.reused |= 2;
+        }
+        for (const Group &g : groups_of(P))
+            if ((rc = born_flow(ctx, b, g, P.nt_max, from_history, st))) return rc;
+        phase_end(ctx, 2, st, ctx->stats.kernel_launches - l0, ctx->stats.cell_updates - c0);
+        return end_call(ctx);
+    }
+    if (from_history) {
         float *hist = (float *)ctx->hist.p;
-        const bool two = time_blocking(ctx, 3);
-        for (int n = 0; n < P.nt_max; n += two ? 2 : 1) {
+        for (int n = 0; n < P.nt_max; n++) {
             a.p = p;
             a.pn = pn;
             a.n = n;
             a.a = hist + ctx->hoff[n];
             TileMaps M;
-            if (two) {
-                a.a2 = hist + ctx->hoff[std::min(n + 1, P.nt_max - 1)];  // (unused past the last step)
-                a.dp_out = dp2;
-                if ((rc = born_pair_maps(ctx, a, &M))) return rc;
-                launch_born_pair(a, active_tiles(P, n), M, st);
-                ctx->stats.cell_updates += active_cells(P, n + 1, ctx->NZ);
-                std::swap(a.dp, dp2);
-            } else {
-                if ((rc = born_hist_maps(ctx, a, &M))) return rc;
-                launch_born_hist_step(a, active_tiles(P, n), M, st);
-            }
+            if ((rc = born_hist_maps(ctx, a, &M))) return rc;
+            launch_born_hist_step(a, active_tiles(P, n), M, st);
             ctx->stats.kernel_launches++;
             ctx->stats.cell_updates += active_cells(P, n, ctx->NZ);
             std::swap(p, pn);
         }
         ctx->stats.reused |= 2;
-        phase_end(ctx, 2, st, ctx->stats.kernel_launches - l0, ctx->stats.cell_updates - c0);
-        return end_call(ctx);
-    }
-    if (time_blocking(ctx, 2)) {  // two steps per launch
-        for (int n = 0; n < P.nt_max; n += 2) {
-            a.u = u;
-            a.un = un;
-            a.p = p;
-            a.pn = pn;
-            a.du_out = du2;
-            a.dp_out = dp2;
-            a.n = n;
-            TileMaps M;
-            if ((rc = born_joint_maps(ctx, a, &M))) return rc;
-            launch_born_joint(a, active_tiles(P, n), M, st);
-            ctx->stats.kernel_launches++;
-            ctx->stats.cell_updates += 2 * (active_cells(P, n, ctx->NZ) + active_cells(P, n + 1, ctx->NZ));
-            std::swap(u, un);
-            std::swap(p, pn);
-            std::swap(a.du, du2);
-            std::swap(a.dp, dp2);
-        }
         phase_end(ctx, 2, st, ctx->stats.kernel_launches - l0, ctx->stats.cell_updates - c0);
         return end_call(ctx);
     }

@@ -87,7 +87,7 @@ struct StepCommon {
     // (TX + 2 HALO)^2 square, cell = ez * (TX + 2 HALO) + ex), by cell then
     // receiver: tile t's are xrecs[xrec_off[t] .. xrec_off[t + 1]).  The
     // two-step adjoint applies the data injection of its first step to the
-    // staged D_nu from them (nullable: no such lists, separate injection).
+    // staged D_nu from them.
     const TileRec *xrecs = nullptr;
     const int *xrec_off = nullptr;
     // Sponge factors by row and by window column (the factor of a cell is
@@ -99,7 +99,7 @@ struct StepCommon {
     const float *wx = nullptr;
 };
 // Most grown-region receiver entries the two-step adjoint's shared-memory
-// list holds; plans with more use the separate injection pass.
+// list holds (tiles with more read them from global memory when they open).
 constexpr int kInjCap = 256;
 
 // Tensor maps of one TMA-staged step launch (kernel parameters).  A field
@@ -110,8 +110,9 @@ constexpr int kInjCap = 256;
 //   forward: 0 u^n (halo), 1 D^n, 2 kappa
 //   adjoint: 0 nu^{k+1} (halo), 1 D_nu, 2 kappa, 3 a^{k-1}, 4 image
 //   Born:    0 u0^n (halo), 1 p^n (halo), 2 D_u0, 3 D_p, 4 kappa, 5 d kappa
+// The two-step launches' maps are given with their structs.
 struct TileMaps {
-    CUtensorMap m[6];
+    CUtensorMap m[8];
 };
 
 // Every propagated field is kept in "summed" form: the field u^n and its
@@ -133,11 +134,6 @@ struct FwdArgs {
     float *a_out;     // nullable: store a^n = D u^n + q^n (history or segment buffer slot)
     float *d;         // nullable: packed records, sample n written from u^{n+1}
     int n;
-    // Two-step kernel only (steps n and n+1 in one launch): D^n is read with a
-    // ring of neighbour cells, so D^{n+2} goes to another pool; u^{n+2} goes
-    // to un; a^{n+1} to a_out2; tiles of shots with nt = n+1 take one step.
-    float *dd_out;
-    float *a_out2;
 };
 
 // Adjoint step k for the scaled multiplier nu = kappa w lambda, which obeys
@@ -152,14 +148,6 @@ struct AdjArgs {
     const float *a;       // pool: a^{k-1} of the background forward field
     float *g;             // pool: per-shot image accumulator, += a^{k-1} nu^k
     int k;
-    // Two-step kernel only (steps k and k-1 in one launch): dd holds D_nu^{k+1}
-    // with the data of step k already injected (launch_adj_inject), D_nu^{k-1}
-    // goes to dd_out, nu^{k-1} to nun, a2 = a^{k-2}.  With inject_here set
-    // the data of step k are not in dd: each tile adds them to its staged
-    // D_nu from c.xrecs (same arithmetic as launch_adj_inject).
-    float *dd_out;
-    const float *a2;
-    int inject_here = 0;
 };
 
 // Born joint step n: background u0 and scattered p advance together.
@@ -173,11 +161,6 @@ struct BornArgs {
     // Background term a^n = D u0^n + q^n read from a stored forward history
     // (launch_born_hist_step; the u fields are then not used).
     const float *a = nullptr;
-    // Two-step kernels only (steps n and n+1): D^n of the fields is du and dp,
-    // D^{n+2} goes to du_out and dp_out, u0^{n+2} to un, p^{n+2} to pn; from the
-    // history, a2 = a^{n+1}.
-    float *du_out = nullptr, *dp_out = nullptr;
-    const float *a2 = nullptr;
 };
 
 // Step-kernel variants.  Variants 0-2: tiles staged by per-thread cp.async,
@@ -196,19 +179,67 @@ int step_variants(int kind);
 // Resident CTAs per SM of a step kernel; kind 0 forward, 1 adjoint, 2 Born.
 int step_occupancy(int kind, int variant, int store_a);
 
-// Two-step (time-blocked) TMA forward kernel (fd_tma2.cu): steps n and n+1
-// of the tiles active at step n.  maps: 0 u^n (HALO2 box), 1 D^n (halo box).
+// Two-step (time-blocked) launches (fd_tma2.cu): npairs step pairs of the nt
+// tiles from t0 on, in one cooperative launch.
 constexpr int HALO2 = 2 * HALO;
 constexpr int U2PITCH = TX + 2 * HALO2 + 4;  // columns of its u^n box (shared-memory row pitch)
-void launch_fwd_pair(const FwdArgs &a, int ntiles, const TileMaps &maps, cudaStream_t s);
-int fwd_pair_occupancy();
-// Two-step adjoint (fd_tma2.cu): steps k and k-1 of the tiles active at step
-// k-1; maps: 0 nu^{k+1} (HALO2 box), 1 D_nu (halo box), 3 image, 4 a^{k-1}, 5
-// a^{k-2} (cell boxes).  Before it, launch_adj_inject adds kappa r^{k-1} (the data of step k,
-// receivers sharing a cell summed in order) to D_nu at the receiver cells of
-// the first nrtiles tiles listed in rtiles (tiles with receivers, by slot).
-void launch_adj_pair(const AdjArgs &a, int ntiles, const TileMaps &maps, cudaStream_t s);
-void launch_adj_inject(const AdjArgs &a, const int *rtiles, int nrtiles, cudaStream_t s);
+struct FlowArgs {
+    unsigned *done;  // per tile of the plan: pairs done by this launch (zeroed before a launch of several)
+    const int *act;  // act[n]: tiles of the plan with nt > n (a prefix)
+    int t0, nt, npairs;
+};
+// a^n per step: base + off[n] (a stored history; off has last + 1 entries), or,
+// without off, base + (n - first) * stride.
+struct ASteps {
+    float *base = nullptr;
+    const long long *off = nullptr;
+    int first = 0, last = 0;
+    long long stride = 0;
+};
+// Steps n0 .. n0 + 2 npairs - 1 (a shot stops at its own nt).  Pair m reads
+// u[m & 1] and d[m & 1] and writes the others; with a.base the a^n are stored, else with ck
+// the checkpoints (u^n, D^n) of every ck_every-th step, step n's at ck + 2 (n /
+// ck_every - ck_first) pools.  maps: u HALO2 boxes 0 and 1, d halo boxes 2 and 3.
+struct FwdFlow {
+    FlowArgs f;
+    StepCommon c;
+    float *u[2], *d[2];
+    float *rec = nullptr;  // packed records (nullable)
+    ASteps a;
+    float *ck = nullptr;
+    int ck_every = 1, ck_first = 0;
+    long long pool = 0;
+    int n0 = 0;
+};
+// Adjoint steps k1 .. k1 - 2 npairs + 1 with the data r injected and the image
+// accumulated in g; buffers and maps as FwdFlow's (nu, d).
+struct AdjFlow {
+    FlowArgs f;
+    StepCommon c;
+    float *nu[2], *d[2];
+    float *g;
+    const float *r;
+    ASteps a;
+    int k1;
+};
+// Born: both fields (maps: u and p HALO2 boxes 0-3, du and dp halo boxes 4-7),
+// or the scattered field with a^n from a (maps: p 0 and 1, dp 2 and 3).
+struct BornFlow {
+    FlowArgs f;
+    StepCommon c;
+    float *u[2], *du[2], *p[2], *dp[2];
+    const float *dkap;
+    float *rec;
+    ASteps a;
+    int n0 = 0;
+};
+// CTAs of a two-step kernel that are resident at once.
+enum { FLOW_FWD = 0, FLOW_ADJ = 1, FLOW_BORN = 2, FLOW_BORN_HIST = 3 };
+int flow_ctas(int kind);
+void launch_fwd_flow(const FwdFlow &a, const TileMaps &maps, cudaStream_t s);
+void launch_adj_flow(const AdjFlow &a, const TileMaps &maps, cudaStream_t s);
+void launch_born_joint_flow(const BornFlow &a, const TileMaps &maps, cudaStream_t s);
+void launch_born_hist_flow(const BornFlow &a, const TileMaps &maps, cudaStream_t s);
 
 // TMA-staged step kernels (fd_tma.cu); variant >= FIRST_TMA_VARIANT.
 void launch_fwd_step_tma(const FwdArgs &a, int ntiles, int variant, int grid, const TileMaps &maps, cudaStream_t s);
@@ -218,12 +249,6 @@ void launch_born_step_tma(const BornArgs &a, int ntiles, int variant, int grid, 
 // 0 p^n halo, 1 D_p, 2 kappa, 3 d kappa, 4 a^n cell box): only the
 // scattered field is advanced; the same bits as the joint step.
 void launch_born_hist_step(const BornArgs &a, int ntiles, const TileMaps &maps, cudaStream_t s);
-// Two such steps, n and n+1, of the tiles active at step n (fd_tma2.cu; maps:
-// 0 p^n HALO2 box, 1 D_p halo box, 2 a^n and 3 a^{n+1} cell boxes).
-void launch_born_pair(const BornArgs &a, int ntiles, const TileMaps &maps, cudaStream_t s);
-// Two joint Born steps, n and n+1, of both fields (fd_tma2.cu; maps: 0 u0^n and
-// 1 p^n HALO2 boxes, 2 D_u0 and 3 D_p halo boxes).
-void launch_born_joint(const BornArgs &a, int ntiles, const TileMaps &maps, cudaStream_t s);
 int tma_occupancy(int kind, int variant);
 
 struct StepLaunch {
