@@ -228,12 +228,14 @@ struct PairSmem {
 // tensor loads wait until the tile and its neighbours have done the pair
 // before (they also have read what the item overwrites by then).  An item of a
 // pair with few tiles is published (fence, release) as soon as its stores are
-// issued; one of a pair with four or more tiles per CTA in the middle of the
-// CTA's next item, when the stores have long drained and the fence
-// delays no one, and nobody waits for the flag yet.  That deferral cannot
-// deadlock: what depends on such an item comes at least 4 gridDim.x items after
-// it, the CTA's next item gridDim.x after it, so the next item depends (through
-// any chain) only on deferred items before this one, which are published first.
+// issued; one of a pair with two or more tiles per CTA in the middle of the CTA's
+// next item, when the stores have long drained and the fence delays no one, and
+// nobody waits for the flag yet (from two tiles per CTA on: 16 and 20 shots of
+// 400 x 1200, gradient, 64.4 -> 60.6 and 77.7 -> 72.0 ms against from four on).
+// That deferral cannot deadlock: what depends on such an item comes more than
+// gridDim.x items after it, the CTA's next item gridDim.x after it, so the next
+// item depends (through any chain) only on deferred items before this one, which
+// are published first.
 //
 // One stage, refilled in the middle of a tile so that the next tile's loads
 // overlap step n+1; the barrier that opens a tile also certifies that every
@@ -342,7 +344,7 @@ __device__ __forceinline__ void run_flow(const FlowArgs &F, const StepCommon &c,
             it.need = k.need(m, T);
             it.row = k.row(m, T);
             it.two = T.nt > n + 1;
-            it.eager = cnt < 4 * (int)gridDim.x + T.pitch / TX + 2;  // (neighbours: up to a tile row + 1 apart)
+            it.eager = cnt < 2 * (int)gridDim.x + T.pitch / TX + 2;  // (neighbours: up to a tile row + 1 apart)
         }
         __syncwarp();
     };
