@@ -36,6 +36,9 @@ struct FpropArgs {
     unsigned *err;              // nullable: set to 1 by a tensor-core GEMM whose bounded wait ran out
     const __nv_bfloat16 *act;   // EPI_BF16_LEAKYBWD: activation [M][act_stride] at act_off
     int act_stride, act_off;
+    // EPI_F32 through launch_fprop_split only: the columns from N / 2 on go, as
+    // bf16 in space-to-depth layout [img][Ho/2][Wo/2][2a+b][N/2], here.
+    __nv_bfloat16 *up = nullptr;
 };
 
 // Split-k weight-gradient GEMM; see igemm_wgrad_kernel.
@@ -61,6 +64,11 @@ struct WgradArgs {
 // mma.sync GEMM (igemm_fprop_kernel), or the tcgen05 one (nn_umma.cu) when
 // DHFWI_NN_GEMM=tc.
 void launch_fprop(const FpropArgs &a, int epi, cudaStream_t s);
+// The input gradient d(cat) of a decoder level's first convolution, split by the
+// GEMM's epilogue: columns n < N / 2 (the skip half) to dst_f32, the upsampled
+// half to a.up.  False (nothing launched) where the tcgen05 kernels do not take
+// the GEMM or N / 2 is no multiple of 16: launch_fprop and launch_split_cat then.
+bool launch_fprop_split(const FpropArgs &a, cudaStream_t s);
 void launch_fprop_umma(const FpropArgs &a, int epi, cudaStream_t s);
 // TMA-fed tcgen05 kernel for the 3x3 convolutions with >= 64 output channels
 // (nn_umma.cu); false when the GEMM is not of that form (nothing launched).

@@ -231,6 +231,22 @@ __global__ void __launch_bounds__(128) igemm_fprop_kernel(FpropArgs P) {
     }
 }
 
+// Four values per access (sizes, strides and offsets multiples of 4, aligned
+// pointers); the per-element arithmetic of the scalar forms.
+struct alignas(8) Bf16x4 {
+    __nv_bfloat162 lo, hi;
+};
+__device__ __forceinline__ float4 bf4_to_f4(Bf16x4 v) {
+    const float2 a = __bfloat1622float2(v.lo), b = __bfloat1622float2(v.hi);
+    return make_float4(a.x, a.y, b.x, b.y);
+}
+__device__ __forceinline__ Bf16x4 f4_to_bf4(float4 v) {
+    Bf16x4 r;
+    r.lo = __halves2bfloat162(__float2bfloat16_rn(v.x), __float2bfloat16_rn(v.y));
+    r.hi = __halves2bfloat162(__float2bfloat16_rn(v.z), __float2bfloat16_rn(v.w));
+    return r;
+}
+
 // Split-k reduction of the fprop partials (fixed split order) with the
 // epilogue of igemm_fprop_kernel.
 // Sum over the splits z = 0 .. splits-1 of p[z * stride], in split order;
@@ -248,6 +264,81 @@ __device__ __forceinline__ float split_sum(const float *__restrict__ p, int spli
     }
     for (; z < splits; z++) s += p[(long long)z * stride];
     return s;
+}
+
+// The sum over the splits in order for four adjacent outputs (see split_sum).
+__device__ __forceinline__ float4 split_sum4(const float *__restrict__ p, int splits, long long stride) {
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    int z = 0;
+    for (; z + 8 <= splits; z += 8) {
+        float4 v[8];
+#pragma unroll
+        for (int k = 0; k < 8; k++) v[k] = *reinterpret_cast<const float4 *>(p + (long long)(z + k) * stride);
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+            s.x += v[k].x;
+            s.y += v[k].y;
+            s.z += v[k].z;
+            s.w += v[k].w;
+        }
+    }
+    for (; z < splits; z++) {
+        const float4 v = *reinterpret_cast<const float4 *>(p + (long long)z * stride);
+        s.x += v.x;
+        s.y += v.y;
+        s.z += v.z;
+        s.w += v.w;
+    }
+    return s;
+}
+
+// fprop_reduce_kernel with four columns per thread: N, the strides and offsets
+// multiples of 4, 16-byte aligned pointers, M N / 4 below 2^31 (32-bit indexes).
+// Bound by the latency of its few loads per output; at 32 x 8 x 8 pixels x 512
+// columns, one column per thread took 8-19 us per reduction.
+template <int EPI>
+__global__ void fprop_reduce4_kernel(FpropArgs P, int splits) {
+    const int N4 = P.N / 4, total = P.M * N4, HWo = P.Ho * P.Wo;
+    const long long MN = (long long)P.M * P.N;
+    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += gridDim.x * blockDim.x) {
+        const int m = idx / N4, n = 4 * (idx - m * N4);
+        float4 v = split_sum4(P.part + 4ll * idx, splits, MN);
+        const long long o = (long long)m * P.dst_stride + P.dst_off + n;
+        if (EPI == EPI_BF16_LEAKY || EPI == EPI_BF16) {
+            const float4 b = *reinterpret_cast<const float4 *>(P.bias + n);
+            v = make_float4(v.x + b.x, v.y + b.y, v.z + b.z, v.w + b.w);
+            if (EPI == EPI_BF16_LEAKY)
+                v = make_float4(v.x > 0.f ? v.x : P.slope * v.x, v.y > 0.f ? v.y : P.slope * v.y,
+                                v.z > 0.f ? v.z : P.slope * v.z, v.w > 0.f ? v.w : P.slope * v.w);
+            *reinterpret_cast<Bf16x4 *>(P.dst_bf16 + o) = f4_to_bf4(v);
+        } else if (EPI == EPI_BF16_CONVT || (EPI == EPI_F32 && P.up && n >= P.N / 2)) {
+            const int img = m / HWo, r = m - img * HWo, ho = r / P.Wo, wo = r - ho * P.Wo;
+            if (EPI == EPI_BF16_CONVT) {
+                const int Co = P.N >> 2, tap = n / Co, co = n - tap * Co, a = tap >> 1, b = tap & 1;
+                const float4 bi = *reinterpret_cast<const float4 *>(P.bias + co);
+                v = make_float4(v.x + bi.x, v.y + bi.y, v.z + bi.z, v.w + bi.w);
+                const long long pix = ((long long)img * (2 * P.Ho) + 2 * ho + a) * (2 * P.Wo) + 2 * wo + b;
+                *reinterpret_cast<Bf16x4 *>(P.dst_bf16 + pix * P.dst_stride + P.dst_off + co) = f4_to_bf4(v);
+            } else {
+                const long long q = (((long long)img * (P.Ho / 2) + ho / 2) * (P.Wo / 2) + wo / 2) * 4 +
+                                    (ho & 1) * 2 + (wo & 1);
+                *reinterpret_cast<Bf16x4 *>(P.up + q * (P.N / 2) + n - P.N / 2) = f4_to_bf4(v);
+            }
+        } else if (EPI == EPI_BF16_LEAKYBWD) {
+            const float4 a = bf4_to_f4(
+                *reinterpret_cast<const Bf16x4 *>(P.act + (long long)m * P.act_stride + P.act_off + n));
+            *reinterpret_cast<Bf16x4 *>(P.dst_bf16 + o) =
+                f4_to_bf4(make_float4(v.x * (a.x > 0.f ? 1.0f : P.slope), v.y * (a.y > 0.f ? 1.0f : P.slope),
+                                      v.z * (a.z > 0.f ? 1.0f : P.slope), v.w * (a.w > 0.f ? 1.0f : P.slope)));
+        } else {
+            float4 *d = reinterpret_cast<float4 *>(P.dst_f32 + o);
+            if (EPI == EPI_F32_ADD) {
+                const float4 y = *d;
+                v = make_float4(v.x + y.x, v.y + y.y, v.z + y.z, v.w + y.w);
+            }
+            *d = v;
+        }
+    }
 }
 
 // One thread per output (grid-stride), the splits summed in order.
@@ -274,6 +365,11 @@ __global__ void fprop_reduce_kernel(FpropArgs P, int splits) {
         } else if (EPI == EPI_BF16_LEAKYBWD) {
             const float av = __bfloat162float(P.act[(long long)m * P.act_stride + P.act_off + n]);
             P.dst_bf16[(long long)m * P.dst_stride + P.dst_off + n] = __float2bfloat16_rn(v * (av > 0.f ? 1.0f : P.slope));
+        } else if (EPI == EPI_F32 && P.up && n >= P.N / 2) {
+            const int img = m / HWo, r = m - img * HWo, ho = r / P.Wo, wo = r - ho * P.Wo;
+            const long long q =
+                (((long long)img * (P.Ho / 2) + ho / 2) * (P.Wo / 2) + wo / 2) * 4 + (ho & 1) * 2 + (wo & 1);
+            P.up[q * (P.N / 2) + n - P.N / 2] = __float2bfloat16_rn(v);
         } else {
             const long long o = (long long)m * P.dst_stride + P.dst_off + n;
             if (EPI == EPI_F32_ADD) v += P.dst_f32[o];
@@ -508,6 +604,44 @@ __global__ void wgrad_reduce_kernel(const float *__restrict__ part, int splits, 
     dw[o] = s;
 }
 
+// The same with four columns per thread and a row per blockIdx.y (nw a multiple
+// of 4, 16-byte aligned partials and dw); the rows from M on are the bias
+// gradients, whose values a block stages in shared memory before one thread adds
+// them in the order of the scalar form (a transposed conv's 4 splits serial loads
+// took 46 us at its top level).
+__global__ void __launch_bounds__(128) wgrad_reduce4_kernel(const float *__restrict__ part, int splits, int M, int N,
+                                                            int nw, int mode, int co_n, float *__restrict__ dw,
+                                                            float *__restrict__ db) {
+    const long long MN = (long long)M * N;
+    const int nbias = mode == WG_CONV ? M : co_n;
+    for (int m = blockIdx.y; m < M + nbias; m += gridDim.y) {
+        if (m >= M) {
+            if (blockIdx.x) return;  // (and for every later row)
+            __shared__ float val[512];
+            const int c = m - M, rows = mode == WG_CONV ? 1 : 4, count = rows * splits;
+            float s = 0.f;
+            for (int base = 0; base < count; base += 512) {
+                const int k = min(512, count - base);
+                for (int i = threadIdx.x; i < k; i += blockDim.x) {
+                    const int ab = (base + i) / splits, z = base + i - ab * splits;
+                    val[i] = part[z * MN + (long long)(ab * co_n + c) * N + nw];
+                }
+                __syncthreads();
+                if (threadIdx.x == 0)
+#pragma unroll 8
+                    for (int i = 0; i < k; i++) s += val[i];
+                __syncthreads();
+            }
+            if (threadIdx.x == 0) db[c] = s;
+            continue;
+        }
+        const int ab = mode == WG_CONV ? 0 : m / co_n;
+        float *out = dw + (mode == WG_CONV ? (long long)m : (long long)(m - ab * co_n) * 4 + ab) * nw;
+        for (int n = 4 * (blockIdx.x * blockDim.x + threadIdx.x); n < nw; n += 4 * gridDim.x * blockDim.x)
+            *reinterpret_cast<float4 *>(out + n) = split_sum4(part + (long long)m * N + n, splits, MN);
+    }
+}
+
 // One warp per channel: lane l sums the partials l, l+32, ..., then a
 // shuffle tree (fixed order, so deterministic).
 __global__ void bias_grad_final_kernel(const float *__restrict__ part, int nblk, int C, float *__restrict__ db) {
@@ -628,22 +762,6 @@ __global__ void leaky_bwd_kernel(const float *__restrict__ dA, const __nv_bfloat
         const float av = __bfloat162float(a[p * as + ao + c]);
         g[i] = __float2bfloat16_rn(dA[i] * (av > 0.f ? 1.0f : slope));
     }
-}
-
-// Four channels per thread (C, strides and offsets multiples of 4, aligned
-// pointers): the same per-element arithmetic as the kernels above and below.
-struct alignas(8) Bf16x4 {
-    __nv_bfloat162 lo, hi;
-};
-__device__ __forceinline__ float4 bf4_to_f4(Bf16x4 v) {
-    const float2 a = __bfloat1622float2(v.lo), b = __bfloat1622float2(v.hi);
-    return make_float4(a.x, a.y, b.x, b.y);
-}
-__device__ __forceinline__ Bf16x4 f4_to_bf4(float4 v) {
-    Bf16x4 r;
-    r.lo = __halves2bfloat162(__float2bfloat16_rn(v.x), __float2bfloat16_rn(v.y));
-    r.hi = __halves2bfloat162(__float2bfloat16_rn(v.z), __float2bfloat16_rn(v.w));
-    return r;
 }
 
 __global__ void leaky_bwd4_kernel(const float4 *__restrict__ dA, const __nv_bfloat16 *__restrict__ a, int as, int ao,
@@ -784,6 +902,85 @@ __global__ void avgpool_fwd4_kernel(const __nv_bfloat16 *__restrict__ x, int xs,
             }
             const float k = 1.0f / 9.0f;
             y[(long long)row * Wo * C4 + t] = f4_to_bf4(make_float4(s.x * k, s.y * k, s.z * k, s.w * k));
+        }
+    }
+}
+
+// Eight channels per thread (16-byte bf16 accesses; C, strides and offsets
+// multiples of 8), all loads of an output issued before its sum: the sums of the
+// four-channel kernels in their order.
+struct alignas(16) Bf16x8 {
+    Bf16x4 a, b;
+};
+__global__ void avgpool_fwd8_kernel(const __nv_bfloat16 *__restrict__ x, int xs, int xo, int nimg, int H, int W,
+                                    int C8, Bf16x8 *__restrict__ y) {
+    const int Ho = (H - 1) / 2 + 1, Wo = (W - 1) / 2 + 1, rows = nimg * Ho;
+    for (int row = blockIdx.y; row < rows; row += gridDim.y) {
+        const int img = row / Ho, ho = row - img * Ho;
+        for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < Wo * C8; t += gridDim.x * blockDim.x) {
+            const int wo = t / C8, c = (t - wo * C8) * 8;
+            Bf16x8 v[9];
+            bool in[9];
+#pragma unroll
+            for (int k = 0; k < 9; k++) {
+                const int h = 2 * ho + k / 3 - 1, w = 2 * wo + k % 3 - 1;
+                in[k] = h >= 0 && h < H && w >= 0 && w < W;
+                if (in[k]) v[k] = *reinterpret_cast<const Bf16x8 *>(x + (((long long)img * H + h) * W + w) * xs + xo + c);
+            }
+            float4 s = make_float4(0.f, 0.f, 0.f, 0.f), u = s;
+#pragma unroll
+            for (int k = 0; k < 9; k++) {
+                if (!in[k]) continue;
+                const float4 p = bf4_to_f4(v[k].a), q = bf4_to_f4(v[k].b);
+                s = make_float4(s.x + p.x, s.y + p.y, s.z + p.z, s.w + p.w);
+                u = make_float4(u.x + q.x, u.y + q.y, u.z + q.z, u.w + q.w);
+            }
+            const float k = 1.0f / 9.0f;
+            y[(long long)row * Wo * C8 + t] = Bf16x8{f4_to_bf4(make_float4(s.x * k, s.y * k, s.z * k, s.w * k)),
+                                                    f4_to_bf4(make_float4(u.x * k, u.y * k, u.z * k, u.w * k))};
+        }
+    }
+}
+
+__global__ void avgpool_bwd_leaky8_kernel(const float4 *__restrict__ dy, int nimg, int H, int W, int C8,
+                                          const float4 *__restrict__ skip, const __nv_bfloat16 *__restrict__ act,
+                                          int as, int ao, float slope, Bf16x8 *__restrict__ g) {
+    const int Ho = (H - 1) / 2 + 1, Wo = (W - 1) / 2 + 1, rows = nimg * H;
+    for (int rw = blockIdx.y; rw < rows; rw += gridDim.y) {
+        const int img = rw / H, h = rw - img * H;
+        for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < W * C8; t += gridDim.x * blockDim.x) {
+            const int w = t / C8, c = t - w * C8;
+            const long long r0 = (long long)rw * W + w, i = r0 * C8 + c;
+            // The windows over (h, w): rows h / 2 and, for odd h, h / 2 + 1; columns likewise.
+            float4 v[4][2];
+            bool in[4];
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                const int ho = h / 2 + k / 2, wo = w / 2 + k % 2;
+                in[k] = (k / 2 == 0 || (h & 1)) && (k % 2 == 0 || (w & 1)) && ho < Ho && wo < Wo;
+                if (in[k]) {
+                    const long long o = (((long long)img * Ho + ho) * Wo + wo) * (2 * C8) + 2 * c;
+                    v[k][0] = dy[o];
+                    v[k][1] = dy[o + 1];
+                }
+            }
+            const float4 o0 = skip[2 * i], o1 = skip[2 * i + 1];
+            const Bf16x8 a8 = *reinterpret_cast<const Bf16x8 *>(act + r0 * as + ao + 8 * c);
+            Bf16x4 out[2];
+#pragma unroll
+            for (int q = 0; q < 2; q++) {
+                float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int k = 0; k < 4; k++)
+                    if (in[k]) s = make_float4(s.x + v[k][q].x, s.y + v[k][q].y, s.z + v[k][q].z, s.w + v[k][q].w);
+                const float k = 1.0f / 9.0f;
+                const float4 o = q ? o1 : o0, av = bf4_to_f4(q ? a8.b : a8.a);
+                const float4 d = make_float4(__fadd_rn(__fmul_rn(s.x, k), o.x), __fadd_rn(__fmul_rn(s.y, k), o.y),
+                                             __fadd_rn(__fmul_rn(s.z, k), o.z), __fadd_rn(__fmul_rn(s.w, k), o.w));
+                out[q] = f4_to_bf4(make_float4(d.x * (av.x > 0.f ? 1.0f : slope), d.y * (av.y > 0.f ? 1.0f : slope),
+                                               d.z * (av.z > 0.f ? 1.0f : slope), d.w * (av.w > 0.f ? 1.0f : slope)));
+            }
+            g[i] = Bf16x8{out[0], out[1]};
         }
     }
 }
@@ -995,6 +1192,12 @@ __global__ void input_pack_kernel(const float *__restrict__ x, long long P, int 
         const int c = (int)(i % Cp);
         y[i] = __float2bfloat16_rn(c == 0 ? x[i / Cp] : 0.f);
     }
+}
+
+// The same for eight channels per pixel: one 16-byte store each.
+__global__ void input_pack8_kernel(const float *__restrict__ x, long long P, uint4 *__restrict__ y) {
+    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < P; p += (long long)gridDim.x * blockDim.x)
+        y[p] = make_uint4(__bfloat16_as_ushort(__float2bfloat16_rn(x[p])), 0u, 0u, 0u);
 }
 
 // Patches: dst[b][i][j] = img[oz + i][ox + j] * scale for patch b = sel[b]
@@ -1388,9 +1591,36 @@ static void fprop_launch(const FpropArgs &a, cudaStream_t s) {
     }
 }
 
+// Four columns per thread where the sizes and the alignment allow it.
+template <int EPI>
+static bool fprop_reduce4(const FpropArgs &a, int splits, cudaStream_t s) {
+    const long long total = (long long)a.M * (a.N / 4);
+    const int Co = EPI == EPI_BF16_CONVT ? a.N / 4 : 4;
+    if (((a.N | a.dst_stride | a.dst_off | Co) & 3) || total >= (1LL << 31) - (1 << 24)) return false;
+    uintptr_t p16 = (uintptr_t)a.part, p8 = 0;
+    if (EPI == EPI_F32 || EPI == EPI_F32_ADD) p16 |= (uintptr_t)a.dst_f32, p8 |= (uintptr_t)a.up;
+    else p8 |= (uintptr_t)a.dst_bf16;
+    if (EPI == EPI_BF16_LEAKY || EPI == EPI_BF16 || EPI == EPI_BF16_CONVT) p16 |= (uintptr_t)a.bias;
+    if (EPI == EPI_BF16_LEAKYBWD) {
+        if ((a.act_stride | a.act_off) & 3) return false;
+        p8 |= (uintptr_t)a.act;
+    }
+    if ((p16 & 15) || (p8 & 7)) return false;
+    fprop_reduce4_kernel<EPI><<<grid_for(total), 256, 0, s>>>(a, splits);
+    return true;
+}
+
 void launch_fprop_reduce(const FpropArgs &a, int epi, int splits, cudaStream_t s) {
     const int g = grid_for((long long)a.M * a.N);
     const int b = 256;
+    switch (epi) {
+    case EPI_BF16_LEAKY: if (fprop_reduce4<EPI_BF16_LEAKY>(a, splits, s)) return; break;
+    case EPI_BF16: if (fprop_reduce4<EPI_BF16>(a, splits, s)) return; break;
+    case EPI_BF16_CONVT: if (fprop_reduce4<EPI_BF16_CONVT>(a, splits, s)) return; break;
+    case EPI_F32: if (fprop_reduce4<EPI_F32>(a, splits, s)) return; break;
+    case EPI_BF16_LEAKYBWD: if (fprop_reduce4<EPI_BF16_LEAKYBWD>(a, splits, s)) return; break;
+    default: if (fprop_reduce4<EPI_F32_ADD>(a, splits, s)) return; break;
+    }
     switch (epi) {
     case EPI_BF16_LEAKY: fprop_reduce_kernel<EPI_BF16_LEAKY><<<g, b, 0, s>>>(a, splits); break;
     case EPI_BF16: fprop_reduce_kernel<EPI_BF16><<<g, b, 0, s>>>(a, splits); break;
@@ -1483,6 +1713,12 @@ void launch_fprop(const FpropArgs &a, int epi, cudaStream_t s) {
     }
 }
 
+bool launch_fprop_split(const FpropArgs &a, cudaStream_t s) {
+    if (gemm_mode() != GEMM_DEFAULT || !a.up || a.N % 32 != 0 || (a.Ho | a.Wo) & 1) return false;
+    if (((uintptr_t)a.up & 15) || ((uintptr_t)a.dst_f32 & 15)) return false;
+    return launch_conv3_patch(a, EPI_F32, s) || launch_conv3_tma(a, EPI_F32, s);
+}
+
 // Tile shape of the weight-gradient GEMM for an M-row problem.
 static bool wgrad_narrow(int M) { return M <= 32; }
 
@@ -1512,23 +1748,30 @@ static void wgrad_launch(const WgradArgs &a, int splits, cudaStream_t s) {
 
 int launch_wgrad(const WgradArgs &a, int splits, float *dw, float *db, cudaStream_t s) {
     const long long mn = (long long)a.M * a.N;
-    const int tsp = launch_wgrad_tma(a, splits, s);
-    if (tsp > 0) {  // partials with the bias column: weight and bias gradients in one reduction
-        wgrad_reduce_kernel<<<(int)((mn + 255) / 256), 256, 0, s>>>(a.part, tsp, a.M, a.N, a.nw, a.mode, a.co, dw,
-                                                                     db);
-        return 2;
+    // Partials with the bias column: weight and bias gradients in one reduction.
+    int sp = launch_wgrad_tma(a, splits, s);
+    if (sp == 0) {
+        sp = splits;
+        if (wgrad_narrow(a.M)) wgrad_launch<1, 4>(a, splits, s);
+        else wgrad_launch<2, 2>(a, splits, s);
     }
-    if (wgrad_narrow(a.M)) wgrad_launch<1, 4>(a, splits, s);
-    else wgrad_launch<2, 2>(a, splits, s);
-    wgrad_reduce_kernel<<<(int)((mn + 255) / 256), 256, 0, s>>>(a.part, splits, a.M, a.N, a.nw, a.mode, a.co, dw,
-                                                                 db);
+    if (((a.nw | a.N) & 3) == 0 && (((uintptr_t)a.part | (uintptr_t)dw) & 15) == 0) {
+        const int rows = a.M + (a.mode == WG_CONV ? a.M : a.co);
+        const dim3 grid((a.nw / 4 + 127) / 128, std::min(rows, 65535));
+        wgrad_reduce4_kernel<<<grid, 128, 0, s>>>(a.part, sp, a.M, a.N, a.nw, a.mode, a.co, dw, db);
+    } else {
+        wgrad_reduce_kernel<<<(int)((mn + 255) / 256), 256, 0, s>>>(a.part, sp, a.M, a.N, a.nw, a.mode, a.co, dw, db);
+    }
     return 2;
 }
 
 void launch_avgpool_fwd(const __nv_bfloat16 *x, int xs, int xo, int nimg, int H, int W, int C, __nv_bfloat16 *y,
                         cudaStream_t s) {
     const long long n = (long long)nimg * ((H - 1) / 2 + 1) * ((W - 1) / 2 + 1) * C;
-    if (C % 4 == 0 && ((xs | xo) & 3) == 0 && (((uintptr_t)x | (uintptr_t)y) & 7) == 0)
+    if (C % 8 == 0 && ((xs | xo) & 7) == 0 && (((uintptr_t)x | (uintptr_t)y) & 15) == 0)
+        avgpool_fwd8_kernel<<<row_grid(((W - 1) / 2 + 1) * (C / 8), nimg * ((H - 1) / 2 + 1)), 256, 0, s>>>(
+            x, xs, xo, nimg, H, W, C / 8, reinterpret_cast<Bf16x8 *>(y));
+    else if (C % 4 == 0 && ((xs | xo) & 3) == 0 && (((uintptr_t)x | (uintptr_t)y) & 7) == 0)
         avgpool_fwd4_kernel<<<row_grid(((W - 1) / 2 + 1) * (C / 4), nimg * ((H - 1) / 2 + 1)), 256, 0, s>>>(
             x, xs, xo, nimg, H, W, C / 4,
                                                             reinterpret_cast<Bf16x4 *>(y));
@@ -1561,7 +1804,12 @@ bool launch_avgpool_bwd_leaky(const float *dy, int nimg, int H, int W, int C, co
     if (C % 4 != 0 || ((as | ao) & 3) != 0 || (((uintptr_t)dy | (uintptr_t)skip) & 15) != 0 ||
         (((uintptr_t)act | (uintptr_t)g) & 7) != 0)
         return false;
-    const long long n = (long long)nimg * H * W * C;
+    if (C % 8 == 0 && ((as | ao) & 7) == 0 && (((uintptr_t)act | (uintptr_t)g) & 15) == 0) {
+        avgpool_bwd_leaky8_kernel<<<row_grid(W * (C / 8), nimg * H), 256, 0, s>>>(
+            reinterpret_cast<const float4 *>(dy), nimg, H, W, C / 8, reinterpret_cast<const float4 *>(skip), act, as, ao,
+            slope, reinterpret_cast<Bf16x8 *>(g));
+        return true;
+    }
     avgpool_bwd_leaky4_kernel<<<row_grid(W * (C / 4), nimg * H), 256, 0, s>>>(dy, nimg, H, W, C / 4,
                                                               reinterpret_cast<const float4 *>(skip), act, as, ao,
                                                               slope, reinterpret_cast<Bf16x4 *>(g));
@@ -1639,7 +1887,10 @@ void launch_convt_tapmajor_batch(const __nv_bfloat16 *w, __nv_bfloat16 *wp, cons
 }
 
 void launch_input_pack(const float *x, long long P, int Cp, __nv_bfloat16 *y, cudaStream_t s) {
-    input_pack_kernel<<<grid_for(P * Cp), 256, 0, s>>>(x, P, Cp, y);
+    if (Cp == 8 && ((uintptr_t)y & 15) == 0)
+        input_pack8_kernel<<<grid_for(P), 256, 0, s>>>(x, P, reinterpret_cast<uint4 *>(y));
+    else
+        input_pack_kernel<<<grid_for(P * Cp), 256, 0, s>>>(x, P, Cp, y);
 }
 void launch_gather_patches(const float *img, int nx, const int *oz, const int *ox, const int *sel, int nb, int p,
                            const float *scale, int mute, float *dst, cudaStream_t s) {

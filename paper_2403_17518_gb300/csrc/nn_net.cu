@@ -610,9 +610,19 @@ struct FuseNext {
     __nv_bfloat16 *g = nullptr;
 };
 
+// A decoder level's d(cat) split by the GEMM that computes it: the skip half
+// (f32) and the upsampled half (bf16, space-to-depth), where that GEMM can
+// (done set), else d(cat) whole in dx.
+struct SplitCat {
+    float *skip = nullptr;
+    __nv_bfloat16 *up = nullptr;
+    bool *done = nullptr;
+};
+
 void block_bwd(NetState &N, int li, const float *dA, const __nv_bfloat16 *a, int as, int ao, const __nv_bfloat16 *x,
                int xs, int xo, int ci, int nimg, int H, int W, float *dx, cudaStream_t s,
-               const __nv_bfloat16 *g_in = nullptr, const FuseNext &next = FuseNext()) {
+               const __nv_bfloat16 *g_in = nullptr, const FuseNext &next = FuseNext(),
+               const SplitCat &cat = SplitCat()) {
     const LayerDesc &d = N.L[li];
     const long long P = (long long)nimg * H * W;
     const __nv_bfloat16 *g = g_in;
@@ -690,6 +700,18 @@ void block_bwd(NetState &N, int li, const float *dA, const __nv_bfloat16 *a, int
             a.slope = 0.2f;
             launch_fprop(a, EPI_BF16_LEAKYBWD, s);
         } else {
+            if (cat.up) {
+                FpropArgs c = a;
+                c.dst_f32 = cat.skip;
+                c.dst_stride = ci / 2;
+                c.up = cat.up;
+                before_gbuf_write(N, cat.up, s);
+                *cat.done = launch_fprop_split(c, s);
+                if (*cat.done) {
+                    N.launches += 2;
+                    return;
+                }
+            }
             a.dst_f32 = dx;
             launch_fprop(a, EPI_F32, s);
         }
@@ -743,33 +765,41 @@ void backward_impl(NetState &N, int n, int H, int W, cudaStream_t s) {
                              N.grad + dout.off, s);
     N.launches += 2;
     float *dA = V.dA, *dB = V.dB;
+    // The two gradient buffers take turns: g holds the output gradient of the
+    // block at hand, other receives the next one's.
+    __nv_bfloat16 *g = V.gbuf, *other = V.gbuf2;
     for (int l = Lv; l >= 1; l--) {
         const int r = Lv - l;
         const int Hr = H >> r, Wr = W >> r;
         const long long Pr = (long long)n * Hr * Wr;
-        // up_l.1: output dec1, input dec0; its input gradient goes straight into
-        // up_l.0's output gradient (dec0's activation backward fused).
+        // up_l.1: output dec1, input dec0, its output gradient in g (from the
+        // output layer's or the transposed conv's backward); its input gradient
+        // goes straight into up_l.0's (dec0's activation backward fused).
         FuseNext fu;
         fu.act = V.dec0[r];
         fu.stride = C(r);
-        fu.g = V.gbuf2;
-        const __nv_bfloat16 *g_top = l == Lv ? V.gbuf : nullptr;  // from the output layer's backward
-        block_bwd(N, layer_index_up(N, l, 2), g_top ? nullptr : dA, V.dec1[r], C(r), 0, V.dec0[r], C(r), 0, C(r), n,
-                  Hr, Wr, nullptr, s, g_top, fu);
-        // up_l.0: output dec0, input cat (2C).
+        fu.g = other;
+        block_bwd(N, layer_index_up(N, l, 2), nullptr, nullptr, 0, 0, V.dec0[r], C(r), 0, C(r), n, Hr, Wr, nullptr, s,
+                  g, fu);
+        // up_l.0: output dec0, input cat (2C).  d(cat) [Pr][2C] is split into the
+        // skip half, kept, and the upsampled half in bf16 and space-to-depth
+        // layout on the coarse grid (the transposed conv's gradients are then
+        // one-tap GEMMs): by the GEMM's epilogue, or in a pass over d(cat).
+        bool split = false;
+        SplitCat cat;
+        cat.skip = V.dskip[r];
+        cat.up = g;
+        cat.done = &split;
         block_bwd(N, layer_index_up(N, l, 1), nullptr, nullptr, 0, 0, V.cat[r], 2 * C(r), 0, 2 * C(r), n, Hr, Wr, dA,
-                  s, V.gbuf2);
-        // dA = d(cat) [Pr][2C]: skip half kept, up half to bf16 in
-        // space-to-depth layout on the coarse grid (the transposed conv's
-        // gradients are then one-tap GEMMs).
-        before_gbuf_write(N, V.gbuf, s);
-        const bool s2d = launch_split_cat(dA, n, Hr, Wr, C(r), V.dskip[r], V.gbuf, s);
+                  s, other, FuseNext(), cat);
+        before_gbuf_write(N, g, s);
+        const bool s2d = split || launch_split_cat(dA, n, Hr, Wr, C(r), V.dskip[r], g, s);
         if (s2d) {
-            N.launches++;
+            N.launches += split ? 0 : 1;
         } else {
             cudaMemsetAsync(V.dskip[r], 0, sizeof(float) * Pr * C(r), s);
             launch_add_slice(dA, 2 * C(r), 0, Pr, C(r), V.dskip[r], s);
-            launch_f32_to_bf16_slice(dA, 2 * C(r), C(r), Pr, C(r), V.gbuf, s);
+            launch_f32_to_bf16_slice(dA, 2 * C(r), C(r), Pr, C(r), g, s);
             N.launches += 2;
         }
         // Transposed conv: input is the level-(r+1) activation.
@@ -779,7 +809,7 @@ void backward_impl(NetState &N, int n, int H, int W, cudaStream_t s) {
         const int Hc = H >> (r + 1), Wc = W >> (r + 1);
         WgradArgs w{};
         w.mode = WG_CONVT;
-        w.g = V.gbuf;
+        w.g = g;
         w.g_stride = s2d ? 4 * C(r) : C(r);
         w.g_s2d = s2d;
         w.x = xin;
@@ -799,9 +829,9 @@ void backward_impl(NetState &N, int n, int H, int W, cudaStream_t s) {
         const int sp = wgrad_splits((long long)n * Hc * Wc, w.M, w.N);
         fork_wgrad(N, s);
         launch_wgrad(w, sp, N.grad + dt.off, N.grad + dt.off + dt.nw, wgrad_stream(N, s));
-        after_wgrad(N, V.gbuf);
+        after_wgrad(N, g);
         FpropArgs a{};
-        a.src = V.gbuf;
+        a.src = g;
         a.src_off = 0;
         if (s2d) {  // input gradient: the one-tap GEMM over the 4 C(r) space-to-depth channels
             a.src_stride = 4 * C(r);
@@ -828,19 +858,27 @@ void backward_impl(NetState &N, int n, int H, int W, cudaStream_t s) {
         a.M = n * Hc * Wc;
         a.N = C(r + 1);
         a.bt = N.wt16 + dt.off;
-        a.dst_f32 = dB;
+        // Its input is the output of the level below (or of the bottom block):
+        // the input gradient times that activation's derivative is that block's
+        // output gradient.
+        a.act = xin;
+        a.act_stride = C(r + 1);
+        a.act_off = 0;
+        a.slope = 0.2f;
+        a.dst_bf16 = other;
         a.dst_stride = C(r + 1);
         a.dst_off = 0;
         a.part = N.fp_part;
         a.part_floats = (long long)N.fp_part_floats;
         a.err = N.err;
-        launch_fprop(a, EPI_F32, s);
+        before_gbuf_write(N, other, s);
+        launch_fprop(a, EPI_BF16_LEAKYBWD, s);
         N.launches += 5;
-        std::swap(dA, dB);
+        std::swap(g, other);
     }
-    // dA: gradient of the bottom activation.  gin: the next block's output
-    // gradient (bf16, gbuf) when the pool's backward already produced it.
-    const __nv_bfloat16 *gin = nullptr;
+    // gin: the next block's output gradient (bf16, in g) when the pass before
+    // already produced it, as the last transposed conv did.
+    const __nv_bfloat16 *gin = g;
     for (int r = Lv; r >= 1; r--) {
         const int Hr = H >> r, Wr = W >> r;
         const long long Pr = (long long)n * Hr * Wr;
@@ -853,22 +891,24 @@ void backward_impl(NetState &N, int n, int H, int W, cudaStream_t s) {
         FuseNext fd;
         fd.act = V.tmp[r];
         fd.stride = C(r);
-        fd.g = V.gbuf2;
+        fd.g = other;
         block_bwd(N, layer_index_down(N, r, 1), gin ? nullptr : dA, ar, ars, 0, V.tmp[r], C(r), 0, C(r), n, Hr, Wr,
                   nullptr, s, gin, fd);
         block_bwd(N, layer_index_down(N, r, 0), nullptr, nullptr, 0, 0, V.pool[r], C(r - 1), 0, C(r - 1), n, Hr, Wr,
-                  dA, s, V.gbuf2);
+                  dA, s, other);
         // Level r-1's output gradient: the pool's backward of dA plus the skip
         // gradient, times the LeakyReLU derivative of that output (cat[r-1]'s
         // first half), straight to bf16 for the next block.
-        before_gbuf_write(N, V.gbuf, s);
+        before_gbuf_write(N, g, s);
         if (launch_avgpool_bwd_leaky(dA, n, H >> (r - 1), W >> (r - 1), C(r - 1), V.dskip[r - 1], V.cat[r - 1],
-                                     2 * C(r - 1), 0, 0.2f, V.gbuf, s)) {
-            gin = V.gbuf;
+                                     2 * C(r - 1), 0, 0.2f, g, s)) {
+            gin = g;
         } else {
             launch_avgpool_bwd(dA, n, H >> (r - 1), W >> (r - 1), C(r - 1), dB, 0, s);
             std::swap(dA, dB);
             gin = nullptr;
+            g = V.gbuf;  // (where block_bwd puts an output gradient it computes itself)
+            other = V.gbuf2;
         }
         N.launches++;
     }
@@ -879,9 +919,9 @@ void backward_impl(NetState &N, int n, int H, int W, cudaStream_t s) {
     FuseNext f0;
     f0.act = V.a_inc0;
     f0.stride = C(0);
-    f0.g = V.gbuf2;
+    f0.g = other;
     block_bwd(N, 1, gin ? nullptr : dA, V.cat[0], 2 * C(0), 0, V.a_inc0, C(0), 0, C(0), n, H, W, nullptr, s, gin, f0);
-    block_bwd(N, 0, nullptr, nullptr, 0, 0, V.xin, CPAD, 0, CPAD, n, H, W, nullptr, s, V.gbuf2);
+    block_bwd(N, 0, nullptr, nullptr, 0, 0, V.xin, CPAD, 0, CPAD, n, H, W, nullptr, s, other);
 }
 
 // Loss of the current batch: MSE against yf; writes g_out (bf16) to the

@@ -543,6 +543,15 @@ __device__ __forceinline__ void conv_tile_epilogue(const FpropArgs &P, const Con
                         o[e] = __float2bfloat16_rn(v[e] * (av > 0.f ? 1.0f : P.slope));
                     }
             }
+        } else if (EPI == EPI_F32 && P.up && nb >= P.N / 2) {  // N / 2 a multiple of 16: the chunk is one half's
+            const long long q = (((long long)img * (P.Ho / 2) + ho / 2) * (P.Wo / 2) + wo / 2) * 4 + (ho & 1) * 2 +
+                                (wo & 1);
+            __nv_bfloat16 *o = P.up + q * (P.N / 2) + nb - P.N / 2;
+            __align__(16) __nv_bfloat16 h[16];
+#pragma unroll
+            for (int e = 0; e < 16; e++) h[e] = __float2bfloat16_rn(v[e]);
+            reinterpret_cast<uint4 *>(o)[0] = reinterpret_cast<const uint4 *>(h)[0];
+            reinterpret_cast<uint4 *>(o)[1] = reinterpret_cast<const uint4 *>(h)[1];
         } else {  // EPI_F32 / EPI_F32_ADD
             float *o = P.dst_f32 + m * P.dst_stride + P.dst_off + nb;
             if (full16 && ((uintptr_t)o & 15) == 0) {  // 16-byte loads and stores
