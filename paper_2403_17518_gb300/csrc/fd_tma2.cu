@@ -775,15 +775,18 @@ __global__ void __launch_bounds__(NT2, 2)
 // steps n and n+1 in one launch, so each field crosses HBM once per two steps
 // (16 bytes per cell and step of both, where the one-step kernel moves 32) and
 // a^n stays in registers between the two updates of a cell.  Both fields' stages
-// fill most of the shared memory, so one CTA of 20 warps takes a tile: items of
-// 4 x 2 cells, 512 of the core and 128 of the ring.  Bound by shared-memory
-// reads (53 % of the wavefronts) and latency at 20 warps per SM.  64 shots of
-// 400 x 1200, 3983 steps: 272 ms (one step per launch, DRAM 64 % busy) -> 215 ms;
-// 32 shots: 149.5 -> 114 ms.
+// fill most of the shared memory, so one CTA takes a tile, and a thread may hold
+// twice the registers of the other two-step kernels: items of 4 x 4 cells (256 of
+// the core, 64 of the ring), both D of the core in registers between the steps,
+// only kappa and its perturbation in slots.  Bound by latency at 10 warps per SM.
+// 64 shots of 400 x 1200, 3983 steps: 272 ms (one step per launch, DRAM 64 % busy)
+// -> 215 ms with items of 4 x 2 cells (20 warps, D in slots).  Those against 4 x 4:
+// 30 shots 105.6 -> 102.7 ms, 8 shots 29.3 -> 27.4, 4 shots of 101 x 101 (36 tiles,
+// latency of a step only) 1.90 -> 1.83; 4 x 4 with D in slots 102.0, 28.1 and 1.92.
 // A forward pair launch that stores a^n and a scattered-field one that reads it
 // (24 bytes) took 270 ms.
 // ---------------------------------------------------------------------------
-constexpr int RJ = 2, NTJ = 640, NCOREJ = 512, LEADERJ = 608;
+constexpr int RJ = 4, NTJ = 320, NCOREJ = 256, LEADERJ = 288;
 struct JointStage {
     float u[U2R][U2PITCH], p[U2R][U2PITCH];
     float du[E][E], dp[E][E];
@@ -792,7 +795,7 @@ constexpr unsigned kJointStageBytes = sizeof(JointStage);
 struct JointSmem {
     JointStage S;
     VTile Vu, Vp;
-    float4 k[RJ][NTJ], dk[RJ][NTJ], du[RJ][NCOREJ], dp[RJ][NCOREJ];  // per-thread slots, see ItemSlots
+    float4 k[RJ][NTJ], dk[RJ][NTJ];  // per-thread slots, see ItemSlots
     TileEdge We[2];
     PairTail tail;
 };
@@ -810,48 +813,46 @@ __device__ __forceinline__ void joint_tile(const BornFlow &A, JointSmem &P, cons
     const bool ok = core && (FULL || T.x0 + lx < T.nxw);
     const int off = lz * T.pitch + lx;
     const int src = FULL ? -1 : item_source<RJ>(T, lx, lz);
-    q4 a0[RJ];
+    q4 a0[RJ], du[RJ], dp[RJ];
 
     // ---- step n on the item: the background, then the scattered field --------
     {
         LapColumn<U2PITCH> col(&P.S.u[lz + HALO][lx + HALO2]);
 #pragma unroll
         for (int rr = 0; rr < RJ; rr++) {
-            q4 u, un, dn;
+            q4 u, un;
             a0[rr] = col.row(rr, u);
             if (rr == 0) cp_async_wait<0>();
             const q4 dv = ld4(&P.S.du[lz + rr + HALO][lx + HALO]), kv = ld4(&P.k[rr][tid].x);
             if constexpr (FULL) {
-                dn = fma4(kv, a0[rr], dv);
-                un = add4(u, dn);
+                du[rr] = fma4(kv, a0[rr], dv);
+                un = add4(u, du[rr]);
             } else {
                 if (rr == src >> 2) add_source(a0[rr], src & 3, A.c.wav[T.wav_off + it.n]);
                 const q4 w = row_w(We, lx, lz, rr);
-                dn = mul4(w, fma4(kv, a0[rr], dv));
-                un = fma4(w, u, dn);
+                du[rr] = mul4(w, fma4(kv, a0[rr], dv));
+                un = fma4(w, u, du[rr]);
             }
             st4(&P.Vu[lz + rr + HALO][lx + HALO], un);
-            if (core) st4(&P.du[rr][tid].x, dn);
         }
     }
     {
         LapColumn<U2PITCH> col(&P.S.p[lz + HALO][lx + HALO2]);
 #pragma unroll
         for (int rr = 0; rr < RJ; rr++) {
-            q4 p, pn, dn;
+            q4 p, pn;
             const q4 ap = col.row(rr, p);
             const q4 dv = ld4(&P.S.dp[lz + rr + HALO][lx + HALO]), kv = ld4(&P.k[rr][tid].x);
             const q4 t = fma4(ld4(&P.dk[rr][tid].x), a0[rr], fma4(kv, ap, dv));
             if constexpr (FULL) {
-                dn = t;
-                pn = add4(p, dn);
+                dp[rr] = t;
+                pn = add4(p, dp[rr]);
             } else {
                 const q4 w = row_w(We, lx, lz, rr);
-                dn = mul4(w, t);
-                pn = fma4(w, p, dn);
+                dp[rr] = mul4(w, t);
+                pn = fma4(w, p, dp[rr]);
             }
             st4(&P.Vp[lz + rr + HALO][lx + HALO], pn);
-            if (core) st4(&P.dp[rr][tid].x, dn);
         }
     }
     __syncthreads();  // u0^{n+1} and p^{n+1} complete; the stage is no longer read
@@ -868,14 +869,14 @@ __device__ __forceinline__ void joint_tile(const BornFlow &A, JointSmem &P, cons
             for (int rr = 0; rr < RJ; rr++) {
                 q4 u, un, d2;
                 a0[rr] = col.row(rr, u);
-                const q4 kv = ld4(&P.k[rr][tid].x), dv = ld4(&P.du[rr][tid].x);
+                const q4 kv = ld4(&P.k[rr][tid].x);
                 if constexpr (FULL) {
-                    d2 = fma4(kv, a0[rr], dv);
+                    d2 = fma4(kv, a0[rr], du[rr]);
                     un = add4(u, d2);
                 } else {
                     if (rr == src >> 2) add_source(a0[rr], src & 3, A.c.wav[T.wav_off + it.n + 1]);
                     const q4 w = row_w(We, lx, lz, rr);
-                    d2 = mul4(w, fma4(kv, a0[rr], dv));
+                    d2 = mul4(w, fma4(kv, a0[rr], du[rr]));
                     un = fma4(w, u, d2);
                 }
                 if (rr < nrow) {
@@ -890,8 +891,8 @@ __device__ __forceinline__ void joint_tile(const BornFlow &A, JointSmem &P, cons
         for (int rr = 0; rr < RJ; rr++) {
             q4 p, pn, d2;
             const q4 ap = col.row(rr, p);
-            const q4 kv = ld4(&P.k[rr][tid].x), dv = ld4(&P.dp[rr][tid].x);
-            const q4 t = fma4(ld4(&P.dk[rr][tid].x), a0[rr], fma4(kv, ap, dv));
+            const q4 kv = ld4(&P.k[rr][tid].x);
+            const q4 t = fma4(ld4(&P.dk[rr][tid].x), a0[rr], fma4(kv, ap, dp[rr]));
             if constexpr (FULL) {
                 d2 = t;
                 pn = add4(p, d2);
