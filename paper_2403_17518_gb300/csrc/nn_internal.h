@@ -136,7 +136,8 @@ void launch_transpose_w_batch(const __nv_bfloat16 *w, __nv_bfloat16 *wt, const T
 // tap-major (n = tap * co + channel) in every EPI_BF16_CONVT epilogue.
 void launch_convt_tapmajor_batch(const __nv_bfloat16 *w, __nv_bfloat16 *wp, const TransposeJobs &jobs,
                                  cudaStream_t s);
-void launch_input_pack(const float *x, long long P, int Cp, __nv_bfloat16 *y, cudaStream_t s);
+// y: 8 channels per pixel, 16-byte aligned.
+void launch_input_pack(const float *x, long long P, __nv_bfloat16 *y, cudaStream_t s);
 void launch_gather_patches(const float *img, int nx, const int *oz, const int *ox, const int *sel, int nb, int p,
                            const float *scale, int mute, float *dst, cudaStream_t s);
 void launch_pad_image(const float *img, int nz, int nx, int Hp, int Wp, const float *scale, int mute, float *dst,

@@ -294,8 +294,9 @@ __device__ __forceinline__ float4 split_sum4(const float *__restrict__ p, int sp
 
 // fprop_reduce_kernel with four columns per thread: N, the strides and offsets
 // multiples of 4, 16-byte aligned pointers, M N / 4 below 2^31 (32-bit indexes).
-// Bound by the latency of its few loads per output; at 32 x 8 x 8 pixels x 512
-// columns, one column per thread took 8-19 us per reduction.
+// Bound by the latency of its few loads per output: 6-8 us per reduction (launch
+// included) in a training step on 32 patches of 128 x 128 at base 32, 8-19 us with one
+// column per thread, which stays for other widths and unaligned destinations.
 template <int EPI>
 __global__ void fprop_reduce4_kernel(FpropArgs P, int splits) {
     const int N4 = P.N / 4, total = P.M * N4, HWo = P.Ho * P.Wo;
@@ -608,7 +609,9 @@ __global__ void wgrad_reduce_kernel(const float *__restrict__ part, int splits, 
 // of 4, 16-byte aligned partials and dw); the rows from M on are the bias
 // gradients, whose values a block stages in shared memory before one thread adds
 // them in the order of the scalar form (a transposed conv's 4 splits serial loads
-// took 46 us at its top level).
+// took 46 us at its top level, this form 15).  The 21 reductions of a training step
+// on 32 patches of 128 x 128 at base 32: 196.7 -> 135.5 us.  The scalar form stays
+// for unaligned parameter offsets.
 __global__ void __launch_bounds__(128) wgrad_reduce4_kernel(const float *__restrict__ part, int splits, int M, int N,
                                                             int nw, int mode, int co_n, float *__restrict__ dw,
                                                             float *__restrict__ db) {
@@ -839,76 +842,12 @@ __global__ void to_bf16_s2d_kernel(const float *__restrict__ x, int nimg, int H,
     }
 }
 
-// Backward of the 3x3 / stride-2 average pool (as avgpool_bwd4_kernel),
-// plus the skip gradient of the same activation, times the LeakyReLU
-// derivative of that activation (bf16 act, stride as, offset ao): the next
-// block's output gradient g in bf16, as avgpool_bwd, add_slice and
-// leaky_bwd in turn would give it.
-__global__ void avgpool_bwd_leaky4_kernel(const float *__restrict__ dy, int nimg, int H, int W, int C4,
-                                          const float4 *__restrict__ skip, const __nv_bfloat16 *__restrict__ act,
-                                          int as, int ao, float slope, Bf16x4 *__restrict__ g) {
-    const int Ho = (H - 1) / 2 + 1, Wo = (W - 1) / 2 + 1, rows = nimg * H;
-    const float4 *dy4 = reinterpret_cast<const float4 *>(dy);
-    for (int rw = blockIdx.y; rw < rows; rw += gridDim.y)
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < W * C4; t += gridDim.x * blockDim.x) {
-        const long long img = rw / H;
-        const int h = rw - (int)img * H, w = t / C4, c = t - w * C4;
-        const long long r0 = (long long)rw * W + w, i = r0 * C4 + c;
-        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int ho = (h > 0 ? h / 2 : 0); ho <= (h + 1) / 2 && ho < Ho; ho++) {
-            if (2 * ho - 1 > h || 2 * ho + 1 < h) continue;
-            for (int wo = (w > 0 ? w / 2 : 0); wo <= (w + 1) / 2 && wo < Wo; wo++) {
-                if (2 * wo - 1 > w || 2 * wo + 1 < w) continue;
-                const float4 v = dy4[((img * Ho + ho) * Wo + wo) * C4 + c];
-                s.x += v.x;
-                s.y += v.y;
-                s.z += v.z;
-                s.w += v.w;
-            }
-        }
-        const float k = 1.0f / 9.0f;
-        const float4 o = skip[i];
-        // Rounded product then sum (no contraction), as the separate passes.
-        const float4 d = make_float4(__fadd_rn(__fmul_rn(s.x, k), o.x), __fadd_rn(__fmul_rn(s.y, k), o.y),
-                                     __fadd_rn(__fmul_rn(s.z, k), o.z), __fadd_rn(__fmul_rn(s.w, k), o.w));
-        const float4 av = bf4_to_f4(*reinterpret_cast<const Bf16x4 *>(act + r0 * as + ao + 4 * c));
-        g[i] = f4_to_bf4(make_float4(d.x * (av.x > 0.f ? 1.0f : slope), d.y * (av.y > 0.f ? 1.0f : slope),
-                                     d.z * (av.z > 0.f ? 1.0f : slope), d.w * (av.w > 0.f ? 1.0f : slope)));
-    }
-}
-
-__global__ void avgpool_fwd4_kernel(const __nv_bfloat16 *__restrict__ x, int xs, int xo, int nimg, int H, int W,
-                                    int C4, Bf16x4 *__restrict__ y) {
-    // Rows (img, ho) on blockIdx.y, (wo, channel quad) on x: no 64-bit index division.
-    const int Ho = (H - 1) / 2 + 1, Wo = (W - 1) / 2 + 1, rows = nimg * Ho;
-    for (int row = blockIdx.y; row < rows; row += gridDim.y) {
-        const int img = row / Ho, ho = row - img * Ho;
-        for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < Wo * C4; t += gridDim.x * blockDim.x) {
-            const int wo = t / C4, c = (t - wo * C4) * 4;
-            float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-            for (int a = 0; a < 3; a++) {
-                const int h = 2 * ho + a - 1;
-                if (h < 0 || h >= H) continue;
-                for (int b = 0; b < 3; b++) {
-                    const int w = 2 * wo + b - 1;
-                    if (w < 0 || w >= W) continue;
-                    const float4 v = bf4_to_f4(
-                        *reinterpret_cast<const Bf16x4 *>(x + (((long long)img * H + h) * W + w) * xs + xo + c));
-                    s.x += v.x;
-                    s.y += v.y;
-                    s.z += v.z;
-                    s.w += v.w;
-                }
-            }
-            const float k = 1.0f / 9.0f;
-            y[(long long)row * Wo * C4 + t] = f4_to_bf4(make_float4(s.x * k, s.y * k, s.z * k, s.w * k));
-        }
-    }
-}
-
-// Eight channels per thread (16-byte bf16 accesses; C, strides and offsets
-// multiples of 8), all loads of an output issued before its sum: the sums of the
-// four-channel kernels in their order.
+// The 3x3 / stride-2 average pool with eight channels per thread (16-byte bf16
+// accesses; C, strides and offsets multiples of 8, which every network width is).
+// Bound by HBM at the top level and by load latency below, so all loads of an output
+// are issued before its sum (in the window's order).  Its four launches on 32 patches
+// of 128 x 128 at base 32 take 50 us, what four channels per thread took too: the
+// form its backward needs, kept alone.
 struct alignas(16) Bf16x8 {
     Bf16x4 a, b;
 };
@@ -942,6 +881,12 @@ __global__ void avgpool_fwd8_kernel(const __nv_bfloat16 *__restrict__ x, int xs,
     }
 }
 
+// Backward of the pool, plus the skip gradient of the same activation, times the
+// LeakyReLU derivative of that activation (bf16 act, stride as, offset ao): the next
+// block's output gradient g in bf16, as avgpool_bwd, add_slice and leaky_bwd in turn
+// would give it.  Eight channels per thread and the up to four windows' loads first:
+// 108.4 -> 80.0 us for the four launches of the size above (four channels, one
+// window at a time).
 __global__ void avgpool_bwd_leaky8_kernel(const float4 *__restrict__ dy, int nimg, int H, int W, int C8,
                                           const float4 *__restrict__ skip, const __nv_bfloat16 *__restrict__ act,
                                           int as, int ao, float slope, Bf16x8 *__restrict__ g) {
@@ -1184,18 +1129,9 @@ __global__ void convt_tapmajor_batch_kernel(const __nv_bfloat16 *__restrict__ w,
     }
 }
 
-// Input image (float32 [img][H][W]) into a bf16 NHWC tensor of Cp channels
-// (channel 0 = the image, others 0).
-__global__ void input_pack_kernel(const float *__restrict__ x, long long P, int Cp, __nv_bfloat16 *__restrict__ y) {
-    const long long n = P * Cp;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(i % Cp);
-        y[i] = __float2bfloat16_rn(c == 0 ? x[i / Cp] : 0.f);
-    }
-}
-
-// The same for eight channels per pixel: one 16-byte store each.
-__global__ void input_pack8_kernel(const float *__restrict__ x, long long P, uint4 *__restrict__ y) {
+// Input image (float32 [img][H][W]) into a bf16 NHWC tensor of 8 channels (channel
+// 0 = the image, others 0): one 16-byte store per pixel.
+__global__ void input_pack_kernel(const float *__restrict__ x, long long P, uint4 *__restrict__ y) {
     for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < P; p += (long long)gridDim.x * blockDim.x)
         y[p] = make_uint4(__bfloat16_as_ushort(__float2bfloat16_rn(x[p])), 0u, 0u, 0u);
 }
@@ -1771,10 +1707,6 @@ void launch_avgpool_fwd(const __nv_bfloat16 *x, int xs, int xo, int nimg, int H,
     if (C % 8 == 0 && ((xs | xo) & 7) == 0 && (((uintptr_t)x | (uintptr_t)y) & 15) == 0)
         avgpool_fwd8_kernel<<<row_grid(((W - 1) / 2 + 1) * (C / 8), nimg * ((H - 1) / 2 + 1)), 256, 0, s>>>(
             x, xs, xo, nimg, H, W, C / 8, reinterpret_cast<Bf16x8 *>(y));
-    else if (C % 4 == 0 && ((xs | xo) & 3) == 0 && (((uintptr_t)x | (uintptr_t)y) & 7) == 0)
-        avgpool_fwd4_kernel<<<row_grid(((W - 1) / 2 + 1) * (C / 4), nimg * ((H - 1) / 2 + 1)), 256, 0, s>>>(
-            x, xs, xo, nimg, H, W, C / 4,
-                                                            reinterpret_cast<Bf16x4 *>(y));
     else
         avgpool_fwd_kernel<<<grid_for(n), 256, 0, s>>>(x, xs, xo, nimg, H, W, C, y);
 }
@@ -1801,18 +1733,12 @@ void launch_to_bf16_s2d(const float *x, int nimg, int H, int W, int C, __nv_bflo
 bool launch_avgpool_bwd_leaky(const float *dy, int nimg, int H, int W, int C, const float *skip,
                               const __nv_bfloat16 *act, int as, int ao, float slope, __nv_bfloat16 *g,
                               cudaStream_t s) {
-    if (C % 4 != 0 || ((as | ao) & 3) != 0 || (((uintptr_t)dy | (uintptr_t)skip) & 15) != 0 ||
-        (((uintptr_t)act | (uintptr_t)g) & 7) != 0)
+    if (C % 8 != 0 || ((as | ao) & 7) != 0 ||
+        (((uintptr_t)dy | (uintptr_t)skip | (uintptr_t)act | (uintptr_t)g) & 15) != 0)
         return false;
-    if (C % 8 == 0 && ((as | ao) & 7) == 0 && (((uintptr_t)act | (uintptr_t)g) & 15) == 0) {
-        avgpool_bwd_leaky8_kernel<<<row_grid(W * (C / 8), nimg * H), 256, 0, s>>>(
-            reinterpret_cast<const float4 *>(dy), nimg, H, W, C / 8, reinterpret_cast<const float4 *>(skip), act, as, ao,
-            slope, reinterpret_cast<Bf16x8 *>(g));
-        return true;
-    }
-    avgpool_bwd_leaky4_kernel<<<row_grid(W * (C / 4), nimg * H), 256, 0, s>>>(dy, nimg, H, W, C / 4,
-                                                              reinterpret_cast<const float4 *>(skip), act, as, ao,
-                                                              slope, reinterpret_cast<Bf16x4 *>(g));
+    avgpool_bwd_leaky8_kernel<<<row_grid(W * (C / 8), nimg * H), 256, 0, s>>>(
+        reinterpret_cast<const float4 *>(dy), nimg, H, W, C / 8, reinterpret_cast<const float4 *>(skip), act, as, ao,
+        slope, reinterpret_cast<Bf16x8 *>(g));
     return true;
 }
 void launch_leaky_bwd(const float *dA, const __nv_bfloat16 *a, int as, int ao, long long P, int C, float slope,
@@ -1886,11 +1812,8 @@ void launch_convt_tapmajor_batch(const __nv_bfloat16 *w, __nv_bfloat16 *wp, cons
     convt_tapmajor_batch_kernel<<<dim3(grid_for(most), jobs.n), 256, 0, s>>>(w, wp, jobs);
 }
 
-void launch_input_pack(const float *x, long long P, int Cp, __nv_bfloat16 *y, cudaStream_t s) {
-    if (Cp == 8 && ((uintptr_t)y & 15) == 0)
-        input_pack8_kernel<<<grid_for(P), 256, 0, s>>>(x, P, reinterpret_cast<uint4 *>(y));
-    else
-        input_pack_kernel<<<grid_for(P * Cp), 256, 0, s>>>(x, P, Cp, y);
+void launch_input_pack(const float *x, long long P, __nv_bfloat16 *y, cudaStream_t s) {
+    input_pack_kernel<<<grid_for(P), 256, 0, s>>>(x, P, reinterpret_cast<uint4 *>(y));
 }
 void launch_gather_patches(const float *img, int nx, const int *oz, const int *ox, const int *sel, int nb, int p,
                            const float *scale, int mute, float *dst, cudaStream_t s) {

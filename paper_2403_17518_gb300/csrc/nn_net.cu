@@ -26,7 +26,7 @@ using namespace nn;
 
 namespace {
 
-constexpr int CPAD = 8;          // first-layer input channels after padding
+constexpr int CPAD = 8;          // first-layer input channels after padding (launch_input_pack's)
 constexpr int MSE_BLOCKS = 256;
 constexpr int RED_BLOCKS = 512;  // max blocks of the bias reductions
 
@@ -487,7 +487,7 @@ void forward(NetState &N, int n, int H, int W, cudaStream_t s) {
     const int Lv = N.levels;
     auto C = [&](int r) { return N.base << r; };
     NetState::Views &V = N.V;
-    launch_input_pack(V.xf, (long long)n * H * W, CPAD, V.xin, s);
+    launch_input_pack(V.xf, (long long)n * H * W, V.xin, s);
     N.launches++;
     // First layer: one real input channel, on CUDA cores (the GEMM would
     // spend 7 of its 8 padded channels on zeros).
@@ -1386,7 +1386,7 @@ int deblur_layer(dhfwi_ctx *ctx, int kind, int op, int n, int H, int W, int ci, 
     }
     long long launches = 0;
     if (first) {  // the network's first layer: one input channel padded to CPAD, CUDA-core kernels
-        if (x_dev) launch_input_pack(x_dev, Pin, CPAD, x16, s), launches++;
+        if (x_dev) launch_input_pack(x_dev, Pin, x16, s), launches++;
         if (w_dev) launch_to_bf16(w_dev, nw, w16, s), launches++;
         if (op == DHFWI_LAYER_FWD) {
             if (!launch_first_conv(x16, CPAD, n, H, W, w16, b_dev, co, 0.2f, y16, co, s)) {
