@@ -259,6 +259,7 @@ KERNEL_SOURCES = {
     "fwd_pair_kernel": ["fd_tma2.cu", "fd_tma.cuh", "fd_device.cuh"],
     "adj_pair_kernel": ["fd_tma2.cu", "fd_tma.cuh", "fd_device.cuh"],
     "born_tma_kernel": ["fd_tma.cu", "fd_tma.cuh", "fd_device.cuh"],
+    "born_joint_kernel": ["fd_tma2.cu", "fd_tma.cuh", "fd_device.cuh"],
 }
 
 
@@ -569,7 +570,7 @@ def main():
     # Library phases (CUDA events on the call's stream): 0 forward passes,
     # 1 backward sweeps, 2 Born joint passes.
     ph = [{"ms": 0.0, "launches": 0, "cells": 0} for _ in range(3)]
-    hist = {"cells": 0, "steps": 0, "fwd_steps": 0}
+    hist = {"cells": 0, "steps": 0, "fwd_steps": 0, "born_steps": 0}
     nt_max = int(max(case.geom.nt))
     launches = [0]
 
@@ -603,6 +604,7 @@ def main():
                 hist["cells"] += st["history_cells"]
                 hist["steps"] = max(hist["steps"], st["history_steps"])
                 hist["fwd_steps"] += nt_max if st["phase_launches"][0] > 0 else 0
+                hist["born_steps"] += nt_max if st["phase_launches"][2] > 0 else 0
         return J
 
     for _ in range(args.warmup):
@@ -634,6 +636,11 @@ def main():
     peak, peak_kind = peaks()
     variants = ctx.stats()["step_variant"]
     fwd_pair = hist["fwd_steps"] / max(ph[0]["launches"], 1) > 1.5  # two time steps per launch
+    born_pair = hist["born_steps"] / max(ph[2]["launches"], 1) > 1.5
+    if born_pair:
+        born_kernel = "born_pair_kernel" if args.reuse else "born_joint_kernel"
+    else:
+        born_kernel = "born_tma_kernel" if variants[3] >= 3 else "born_step_kernel"
     kernels = [
         ("fwd_pair_kernel" if fwd_pair else forward_kernel(variants[0]),
          "forward passes of fwi_gradient and rtm_mig, storing the a^n history",
@@ -644,7 +651,7 @@ def main():
          "backward sweeps of fwi_gradient and rtm_mig (adjoint steps with imaging, a^n read from the history)",
          ADJ_BYTES_PER_CELL * ph[1]["cells"],
          f"{ADJ_BYTES_PER_CELL} B per update (12 B for the adjoint field + 4 B to read a^n)"),
-        ("born_tma_kernel" if variants[3] >= 3 else "born_step_kernel",
+        (born_kernel,
          "Born joint passes of born_demig (background and scattered fields)",
          BORN_BYTES_PER_CELL_STEP * ph[2]["cells"] // 2,
          f"{BORN_BYTES_PER_CELL_STEP} B per cell-step (two fields, 24 B, + 4 B for dv)"),

@@ -124,9 +124,11 @@ typedef struct {
      * either way. */
     int history_steps;
     long long history_cells;   /* phase-0 cell updates that also stored a^n */
-    /* Time steps per launch (1 or 2) of the forward and the adjoint sweeps:
-     * the autotuner times both depths per geometry; DHFWI_TIME_BLOCK=0
-     * (environment) forces 1, any other value 2. */
+    /* Time steps (1 or 2) by which a tile of the forward and the adjoint
+     * sweeps advances at a time: the autotuner times both depths per geometry
+     * (of Born the form that reads the history; both fields together take 2);
+     * DHFWI_TIME_BLOCK=0 (environment) forces 1, any other value 2.  A launch of the two-step kernels covers many such pairs
+     * (kernel_launches and phase_launches count launches, not steps). */
     int time_block[2];
     /* What the last call took from the stored forward pass of an earlier
      * call (dhfwi_set_reuse): bit 0, rtm_mig skipped its forward pass; bit 1,
