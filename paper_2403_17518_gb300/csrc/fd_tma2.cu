@@ -780,9 +780,9 @@ __global__ void __launch_bounds__(NT2, 2)
 // the core, 64 of the ring), both D of the core in registers between the steps,
 // only kappa and its perturbation in slots.  Bound by latency at 10 warps per SM.
 // 64 shots of 400 x 1200, 3983 steps: 272 ms (one step per launch, DRAM 64 % busy)
-// -> 215 ms with items of 4 x 2 cells (20 warps, D in slots).  Those against 4 x 4:
-// 30 shots 105.6 -> 102.7 ms, 8 shots 29.3 -> 27.4, 4 shots of 101 x 101 (36 tiles,
-// latency of a step only) 1.90 -> 1.83; 4 x 4 with D in slots 102.0, 28.1 and 1.92.
+// -> 222.5 with items of 4 x 2 cells (20 warps, D in slots) -> 218.4 with these; 30
+// shots 105.6 -> 102.7, 8 shots 29.3 -> 27.4, 4 shots of 101 x 101 (36 tiles, latency
+// of a step only) 1.90 -> 1.83; 4 x 4 with D in slots 102.0, 28.1 and 1.92.
 // A forward pair launch that stores a^n and a scattered-field one that reads it
 // (24 bytes) took 270 ms.
 // ---------------------------------------------------------------------------

@@ -1,7 +1,7 @@
 """Whole gradients of the network at sizes where the backward pass changes route:
 the decoder's d(cat) split by the GEMM's epilogue (tcgen05 kernels, 32-channel
-levels and above) or by a separate pass (16- and 48-channel levels), eight- and
-four-channel pooling kernels, ragged patch tiles, split-k reductions of four
+levels and above) or by a separate pass (16- and 48-channel levels), eight-
+channel pooling kernels, ragged patch tiles, split-k reductions of four
 columns.  Against the float64 oracle with its bfloat16 operand rounding, at the
 tolerances of the other whole-network gradients (1e-2 of the gradient's norm, 0.1
 per tensor: the effect of flipped bfloat16 roundings)."""
