@@ -98,6 +98,13 @@ struct StepCommon {
     const float *wz = nullptr;
     const float *wx = nullptr;
 };
+// Offset of padded row z, clamped into the domain, in a model array.  64-bit: an
+// array may hold 2^31 cells and more (with narrow windows it still fits the
+// device; each copy is then 8 GB).
+__host__ __device__ inline long long model_row(int z, int NZ, int pf) {
+    const int i = z < 0 ? 0 : z < NZ ? z : NZ - 1;
+    return (long long)i * pf;
+}
 // Most grown-region receiver entries the two-step adjoint's shared-memory
 // list holds (tiles with more read them from global memory when they open).
 constexpr int kInjCap = 256;

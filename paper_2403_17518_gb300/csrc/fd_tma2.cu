@@ -177,7 +177,7 @@ __device__ __forceinline__ void copy_item(float4 (*slots)[NT], const float *mode
     const float *m = model + (long long)T.mc * c.mstride + min(max(T.mx + lx, 0), c.pf - 4);
 #pragma unroll
     for (int rr = 0; rr < R; rr++)
-        cp_async16(&slots[rr][tid], m + min(max(T.z0 + lz + rr, 0), c.NZ - 1) * c.pf);
+        cp_async16(&slots[rr][tid], m + model_row(T.z0 + lz + rr, c.NZ, c.pf));
 }
 // A tile's sponge factors, copied by one warp.
 __device__ __forceinline__ void copy_edge(TileEdge &We, const StepCommon &c, const TileInfo &T, int lane) {
