@@ -277,7 +277,7 @@ __device__ __forceinline__ void bar_arrive() { asm volatile("bar.arrive %0, %1;"
 
 // Leader warp: whether the item's tile and its neighbours have done `need`
 // pairs; with wait, waits for it (bounded) and returns false when it did not
-// come.  True orders the loads that follow after their stores.
+// come.  True orders the loads that follow, of any lane, after their stores.
 __device__ __forceinline__ bool deps_done(const FlowArgs &F, const StepCommon &c, const FlowItem &it, int lane,
                                           bool wait) {
     if (it.need == 0) return true;
@@ -296,6 +296,7 @@ __device__ __forceinline__ bool deps_done(const FlowArgs &F, const StepCommon &c
                 if (__any_sync(0xffffffffu, stop)) return false;
             }
     }
+    __syncwarp();  // the vote orders no memory: every lane's acquire before what any lane does next
     return ok;
 }
 
