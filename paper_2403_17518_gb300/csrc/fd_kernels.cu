@@ -497,25 +497,25 @@ void launch_prep_model(const float *v, const float *dv, int rel, int nz, int nx,
 }
 
 // ---------------------------------------------------------------------------
-// Sponge tables of a plan (blockIdx.y = 0: rows, 1 + slot: that slot's columns)
+// Sponge tables of a plan: the rows (table 0), then the columns of slot 0, 1, ...
+// (any number of shots: blockIdx.y strides over the tables)
 // ---------------------------------------------------------------------------
-__global__ void sponge_tables_kernel(const ShotDesc *__restrict__ shots, int NZ, int nb, int pitch,
+__global__ void sponge_tables_kernel(const ShotDesc *__restrict__ shots, int n_shots, int NZ, int nb, int pitch,
                                      float *__restrict__ wz, int nwz, float *__restrict__ wx) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool rows = blockIdx.y == 0;
-    const int len = rows ? nwz : pitch + 2 * HALO;
-    if (t >= len) return;
-    const int slot = (int)blockIdx.y - 1;
-    const int N = rows ? NZ : shots[slot].nxw;
-    const int i = t - HALO;
-    const float w = i >= 0 && i < N ? sponge1(i, N, nb) : 0.f;
-    (rows ? wz : wx + (long long)slot * len)[t] = w;
+    const int i = t - HALO, lx = pitch + 2 * HALO;
+    for (int k = blockIdx.y; k <= n_shots; k += gridDim.y) {
+        const int N = k == 0 ? NZ : shots[k - 1].nxw;
+        if (t < (k == 0 ? nwz : lx))
+            (k == 0 ? wz : wx + (k - 1ll) * lx)[t] = i >= 0 && i < N ? sponge1(i, N, nb) : 0.f;
+    }
 }
 
 void launch_sponge_tables(const ShotDesc *shots, int n_shots, int NZ, int nb, int pitch, float *wz, int nwz,
                           float *wx, cudaStream_t s) {
     const int len = nwz > pitch + 2 * HALO ? nwz : pitch + 2 * HALO;
-    sponge_tables_kernel<<<dim3((len + 127) / 128, 1 + n_shots), 128, 0, s>>>(shots, NZ, nb, pitch, wz, nwz, wx);
+    const int tables = n_shots < 65535 ? 1 + n_shots : 65535;  // the most that gridDim.y takes
+    sponge_tables_kernel<<<dim3((len + 127) / 128, tables), 128, 0, s>>>(shots, n_shots, NZ, nb, pitch, wz, nwz, wx);
 }
 
 // ---------------------------------------------------------------------------
