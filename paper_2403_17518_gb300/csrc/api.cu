@@ -1003,6 +1003,7 @@ int tune_depth(dhfwi_ctx *ctx, cudaStream_t st, const float *one_step_ms, int re
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
     int rc = DHFWI_OK;
+    const long long cells = ctx->stats.cell_updates;  // the trials' updates are not the call's
     float hist_ms = 0.f;  // Born from the history, one step per launch
     // which: 0 forward, 1 adjoint, 2 Born, 3 one step of Born from the history, 4 two of them.
     for (int which = 0; which < 5 && !rc; which++) {
@@ -1069,6 +1070,7 @@ int tune_depth(dhfwi_ctx *ctx, cudaStream_t st, const float *one_step_ms, int re
         const float one = which == 4 ? hist_ms : one_step_ms[which == 0 ? 0 : which + 1] * (2.f * np / reps);
         ctx->depth[which == 4 ? 3 : which] = ms <= one ? 2 : 1;
     }
+    ctx->stats.cell_updates = cells;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (rc) {  // no two-step launch possible here: one step per launch

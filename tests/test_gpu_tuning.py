@@ -1,0 +1,39 @@
+"""What the autotuner of a first call at a geometry leaves behind: the statistics of
+the call itself, and trials that follow from the records alone."""
+import copy
+
+import numpy as np
+import pytest
+
+import synth
+from gpu_helpers import f32, f32_geom, gpu_ctx, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+def _case(monkeypatch, nt=40, nt_max=None):
+    for k in ("DHFWI_STEP_VARIANT", "DHFWI_TIME_BLOCK", "DHFWI_HISTORY_MB"):
+        monkeypatch.delenv(k, raising=False)
+    c = synth.tiny_case(nz=60, nx=90, nt=nt_max or nt, nb=20, n_shots=2, seed=3)
+    c.geom.nt = np.full_like(c.geom.nt, nt)
+    v = to_dev(f32(1800.0 + 400.0 * synth.rng(7).uniform(size=(60, 90))))
+    return c, f32_geom(copy.deepcopy(c.geom)), v
+
+
+def test_first_call_counts_its_own_updates(monkeypatch):
+    c, g, v = _case(monkeypatch)
+    for call in ("model", "gradient", "born"):
+        ctx = gpu_ctx(c)
+        cells = []
+        for _ in range(2):
+            if call == "model":
+                ctx.model_shots(v, g)
+            elif call == "gradient":
+                ctx.fwi_gradient(v, g, ctx.new_data(g).zero_())
+            else:
+                ctx.born_demig(v, g, 0.01 * v)
+            cells.append(ctx.stats()["cell_updates"])
+        ctx.close()
+        w = g.win_x1.astype(np.int64) - g.win_x0 + 2 * c.nb
+        once = int(np.sum(w * g.nt)) * (c.nz + 2 * c.nb)
+        assert cells == [(1 if call == "model" else 2) * once] * 2, call
