@@ -995,7 +995,7 @@ int tune_depth(dhfwi_ctx *ctx, cudaStream_t st, const float *one_step_ms, int re
     const Plan &P = ctx->plan;
     const long long pool = P.pool_floats;
     float *F = (float *)ctx->fields.p;
-    const int np = std::min(4, P.nt_max / 2);  // pairs timed
+    const int np = std::min(4, P.nt_sorted[0] / 2);  // pairs timed; nt_max may pass the longest record
     for (int &d : ctx->depth) d = 1;
     if (np == 0) return DHFWI_OK;
     const Group all{0, P.n_shots};

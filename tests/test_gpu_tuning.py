@@ -37,3 +37,19 @@ def test_first_call_counts_its_own_updates(monkeypatch):
         w = g.win_x1.astype(np.int64) - g.win_x0 + 2 * c.nb
         once = int(np.sum(w * g.nt)) * (c.nz + 2 * c.nb)
         assert cells == [(1 if call == "model" else 2) * once] * 2, call
+
+
+def test_trials_follow_the_records(monkeypatch):
+    """Records far shorter than the geometry's nt_max (its wavelets' length): the
+    trials are those of a geometry whose nt_max is the longest record."""
+    extra = []
+    for nt_max in (6, 60):
+        c, g, v = _case(monkeypatch, nt=6, nt_max=nt_max)
+        ctx = gpu_ctx(c)
+        launches = []
+        for _ in range(2):
+            ctx.model_shots(v, g)
+            launches.append(ctx.stats()["kernel_launches"])
+        extra.append(launches[0] - launches[1])
+        ctx.close()
+    assert extra[0] == extra[1]
