@@ -82,10 +82,12 @@ struct dhfwi_ctx {
     // Step-kernel launch choice per kind: forward, forward+segment store,
     // adjoint, Born.  Picked by autotune() for the current plan.
     StepLaunch launch[4];
+    float one_step_ms[4] = {};  // of the chosen kernels, per launch
     // Time steps per launch (1 or 2) of the forward and the adjoint sweeps, of
     // Born demigration and of Born from a stored history, chosen by the
-    // autotuner.
+    // autotuner (Born's by the plan's first Born call: born_tuned).
     int depth[4] = {2, 2, 2, 2};
+    bool born_tuned = true;
     // Reuse of the stored forward wavefield between calls (dhfwi_set_reuse):
     // the identity of the last complete backward-capable forward pass (plan
     // hash, model hash, history segments, checkpoint interval) whose a^n
@@ -699,13 +701,14 @@ void set_variant(dhfwi_ctx *ctx, int kind, int v) {
     cudaGetLastError();
 }
 
-int tune_depth(dhfwi_ctx *ctx, cudaStream_t st, const float *one_step_ms, int reps);
+enum { TRY_FWD = 0, TRY_ADJ = 1, TRY_BORN = 2, TRY_BORN_HIST = 3, TRY_HIST_ONE = 4 };  // see depth_trial
+int tune_depth(dhfwi_ctx *ctx, int first, int last, cudaStream_t st);
 
 // Autotuner: for the current plan, time every step-kernel variant of each
 // kind on the plan's full tile list (all shots active) using the scratch
-// field pools, and keep the fastest; then the time-blocking depth of each sweep (tune_depth).  The pools are zeroed again by the
-// call that follows, so tuning leaves no trace in the results.  Runs once per
-// geometry; DHFWI_STEP_VARIANT=<0..6> pins a variant instead (and the depth
+// field pools, and keep the fastest; then the time-blocking depth of the
+// sweeps (tune_depth).  The pools are zeroed again by the call that follows,
+// so tuning leaves no trace in the results.  Runs once per geometry; DHFWI_STEP_VARIANT=<0..6> pins a variant instead (and the depth
 // stays two unless DHFWI_TIME_BLOCK says otherwise).
 int autotune(dhfwi_ctx *ctx, cudaStream_t st) {
     const Plan &P = ctx->plan;
@@ -719,6 +722,7 @@ int autotune(dhfwi_ctx *ctx, cudaStream_t st) {
         const bool valid = v >= 0 && v < N_STEP_VARIANTS;
         for (int k = 0; k < 4; k++)
             set_variant(ctx, k, valid ? std::min(v, step_variants(kernel_kind[k]) - 1) : 1);
+        ctx->born_tuned = true;
         ctx->tuned_hash = P.hash;
         return DHFWI_OK;
     }
@@ -737,7 +741,6 @@ int autotune(dhfwi_ctx *ctx, cudaStream_t st) {
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
     long long timed = 0;
-    float best_ms[4] = {0.f, 0.f, 0.f, 0.f};
     for (int kind = 0; kind < 4; kind++) {
         float best = 1e30f;
         int best_v = 1;
@@ -804,12 +807,13 @@ int autotune(dhfwi_ctx *ctx, cudaStream_t st) {
             }
         }
         set_variant(ctx, kind, best_v);
-        best_ms[kind] = best;
+        ctx->one_step_ms[kind] = best / reps;
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     ctx->stats.kernel_launches += timed;
-    if ((rc = tune_depth(ctx, st, best_ms, reps))) return rc;
+    if ((rc = tune_depth(ctx, TRY_FWD, TRY_ADJ, st))) return rc;
+    ctx->born_tuned = false;
     ctx->tuned_hash = P.hash;
     CK(cudaGetLastError());
     return DHFWI_OK;
@@ -985,97 +989,105 @@ int born_flow(dhfwi_ctx *ctx, BornFlow b, const Group &g, int n1, bool from_hist
 // Groups of the slots for the two-step launches: all of them together.
 std::vector<Group> groups_of(const Plan &P) { return {Group{0, P.n_shots}}; }
 
-// Time-blocking depth of the forward and the adjoint sweeps, of Born and of
-// Born from the history: a two-step launch of a few pairs on the plan's full
-// tile list against the chosen one-step kernel's time for as many steps
-// (one_step_ms: the variant loop's best time of `reps` launches per kind:
-// forward, forward with store, adjoint, Born).  The faster depth is kept.
-int tune_depth(dhfwi_ctx *ctx, cudaStream_t st, const float *one_step_ms, int reps) {
-    if (!encode_tiled()) return DHFWI_OK;
+// Time-blocking depth: a two-step launch of a few pairs on the plan's full tile
+// list against the chosen one-step kernel's time for as many steps.  The faster
+// depth is kept.  The forward and the adjoint sweeps are tried by the first call
+// at a geometry, the two Born forms by its first Born call (their trials would
+// lengthen the tuning of a 101 x 101 plan, 4 shots, by a fifth for programs that
+// never call Born).
+//
+// A trial: `np` pairs, or (TRY_HIST_ONE) as many single steps of Born from the
+// history, whose one-step kernel the variant loop does not time.
+int depth_trial(dhfwi_ctx *ctx, int which, int np, cudaStream_t st) {
     const Plan &P = ctx->plan;
     const long long pool = P.pool_floats;
     float *F = (float *)ctx->fields.p;
-    const int np = std::min(4, P.nt_sorted[0] / 2);  // pairs timed; nt_max may pass the longest record
-    for (int &d : ctx->depth) d = 1;
-    if (np == 0) return DHFWI_OK;
     const Group all{0, P.n_shots};
+    int rc = DHFWI_OK;
+    if (which == TRY_FWD) {
+        FwdFlow a{};
+        a.c = common(ctx);
+        a.rec = (float *)ctx->dtmp.p;
+        float *u = F, *un = F + pool, *d = F + 2 * pool, *dn = F + 7 * pool;
+        return fwd_flow(ctx, a, all, 0, 2 * np, u, un, d, dn, st);
+    }
+    if (which == TRY_ADJ) {
+        AdjFlow b{};
+        b.c = common(ctx);
+        b.a.base = F + 3 * pool;
+        b.g = F + 4 * pool;
+        b.r = (const float *)ctx->rtmp.p;
+        float *u = F, *un = F + pool, *d = F + 2 * pool, *dn = F + 8 * pool;
+        return adj_flow(ctx, b, all, 2 * np, 0, u, un, d, dn, st);
+    }
+    if (which == TRY_HIST_ONE) {
+        BornArgs b{};
+        b.c = common(ctx);
+        b.p = F + 3 * pool;
+        b.pn = F + 4 * pool;
+        b.dp = F + 5 * pool;
+        b.dkap = (const float *)ctx->kap.p;
+        b.d = (float *)ctx->dtmp.p;
+        b.a = F + 8 * pool;
+        TileMaps M;
+        for (int i = 0; i < 2 * np && !rc; i++)
+            if (!(rc = born_hist_maps(ctx, b, &M))) launch_born_hist_step(b, active_tiles(P, 0), M, st);
+        ctx->stats.kernel_launches += 2 * np;
+        return rc;
+    }
+    BornFlow b{};
+    b.c = common(ctx);
+    b.dkap = (const float *)ctx->kap.p;
+    b.rec = (float *)ctx->dtmp.p;
+    b.a.base = F + 8 * pool;
+    b.u[0] = F;
+    b.u[1] = F + pool;
+    b.du[0] = F + 2 * pool;
+    b.du[1] = F + 7 * pool;
+    b.p[0] = F + 3 * pool;
+    b.p[1] = F + 4 * pool;
+    b.dp[0] = F + 5 * pool;
+    b.dp[1] = F + 6 * pool;
+    return born_flow(ctx, b, all, 2 * np, which == TRY_BORN_HIST, st);
+}
+
+// Time of a trial after one for warm-up.
+int time_trial(dhfwi_ctx *ctx, int which, int np, cudaEvent_t e0, cudaEvent_t e1, float *ms, cudaStream_t st) {
+    int rc = depth_trial(ctx, which, np, st);
+    if (rc) return rc;
+    CK(cudaEventRecord(e0, st));
+    if ((rc = depth_trial(ctx, which, np, st))) return rc;
+    CK(cudaEventRecord(e1, st));
+    CK(cudaEventSynchronize(e1));
+    CK(cudaEventElapsedTime(ms, e0, e1));
+    return DHFWI_OK;
+}
+
+// Depth of the sweeps [first, last] (TRY_*).  A two-step launch that is not
+// possible here leaves them at one step per launch.
+int tune_depth(dhfwi_ctx *ctx, int first, int last, cudaStream_t st) {
+    const int np = std::min(4, ctx->plan.nt_sorted[0] / 2);  // nt_max may pass the longest record
+    for (int which = first; which <= last; which++) ctx->depth[which] = 1;
+    if (!encode_tiled() || np == 0) return DHFWI_OK;
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
-    int rc = DHFWI_OK;
     const long long cells = ctx->stats.cell_updates;  // the trials' updates are not the call's
-    float hist_ms = 0.f;  // Born from the history, one step per launch
-    // which: 0 forward, 1 adjoint, 2 Born, 3 one step of Born from the history, 4 two of them.
-    for (int which = 0; which < 5 && !rc; which++) {
-        float ms = 0.f;
-        for (int rep = 0; rep < 2 && !rc; rep++) {  // one warm-up
-            if (rep == 1) cudaEventRecord(e0, st);
-            if (which == 0) {
-                FwdFlow a{};
-                a.c = common(ctx);
-                a.rec = (float *)ctx->dtmp.p;
-                float *u = F, *un = F + pool, *d = F + 2 * pool, *dn = F + 7 * pool;
-                rc = fwd_flow(ctx, a, all, 0, 2 * np, u, un, d, dn, st);
-            } else if (which == 1) {
-                AdjFlow b{};
-                b.c = common(ctx);
-                b.a.base = F + 3 * pool;
-                b.g = F + 4 * pool;
-                b.r = (const float *)ctx->rtmp.p;
-                float *u = F, *un = F + pool, *d = F + 2 * pool, *dn = F + 8 * pool;
-                rc = adj_flow(ctx, b, all, 2 * np, 0, u, un, d, dn, st);
-            } else if (which == 3) {
-                BornArgs b{};
-                b.c = common(ctx);
-                b.p = F + 3 * pool;
-                b.pn = F + 4 * pool;
-                b.dp = F + 5 * pool;
-                b.dkap = (const float *)ctx->kap.p;
-                b.d = (float *)ctx->dtmp.p;
-                b.a = F + 8 * pool;
-                TileMaps M;
-                for (int i = 0; i < 2 * np && !rc; i++)
-                    if (!(rc = born_hist_maps(ctx, b, &M))) launch_born_hist_step(b, active_tiles(P, 0), M, st);
-                ctx->stats.kernel_launches += 2 * np;
-            } else {
-                BornFlow b{};
-                b.c = common(ctx);
-                b.dkap = (const float *)ctx->kap.p;
-                b.rec = (float *)ctx->dtmp.p;
-                b.a.base = F + 8 * pool;
-                b.u[0] = F;
-                b.u[1] = F + pool;
-                b.du[0] = F + 2 * pool;
-                b.du[1] = F + 7 * pool;
-                b.p[0] = F + 3 * pool;
-                b.p[1] = F + 4 * pool;
-                b.dp[0] = F + 5 * pool;
-                b.dp[1] = F + 6 * pool;
-                rc = born_flow(ctx, b, all, 2 * np, which == 4, st);
-            }
-        }
-        cudaEventRecord(e1, st);
-        cudaError_t e = cudaEventSynchronize(e1);
-        if (e != cudaSuccess) {
-            cudaEventDestroy(e0);
-            cudaEventDestroy(e1);
-            return cuda_fail(ctx, e, "autotune (time-blocking depth)");
-        }
-        if (rc) break;
-        cudaEventElapsedTime(&ms, e0, e1);
-        if (which == 3) {
-            hist_ms = ms;
-            continue;
-        }
-        const float one = which == 4 ? hist_ms : one_step_ms[which == 0 ? 0 : which + 1] * (2.f * np / reps);
-        ctx->depth[which == 4 ? 3 : which] = ms <= one ? 2 : 1;
+    int rc = DHFWI_OK;
+    for (int which = first; which <= last && !rc; which++) {
+        static const int kind[3] = {0, 2, 3};  // of the one-step kernels (dhfwi_ctx::launch)
+        float two = 0.f, one = 0.f;
+        rc = time_trial(ctx, which, np, e0, e1, &two, st);
+        if (which == TRY_BORN_HIST) rc = rc ? rc : time_trial(ctx, TRY_HIST_ONE, np, e0, e1, &one, st);
+        else one = ctx->one_step_ms[kind[which]] * 2 * np;
+        if (!rc) ctx->depth[which] = two <= one ? 2 : 1;
     }
     ctx->stats.cell_updates = cells;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    if (rc) {  // no two-step launch possible here: one step per launch
+    if (rc) {
         ctx->err.clear();
-        for (int &d : ctx->depth) d = 1;
+        for (int which = first; which <= last; which++) ctx->depth[which] = 1;
     }
     return DHFWI_OK;
 }
@@ -1585,6 +1597,10 @@ int born_demig(dhfwi_ctx *ctx, const float *v0_dev, const dhfwi_geom *geom, cons
     const long long pool = P.pool_floats;
     if ((rc = ensure(ctx, ctx->fields, NPOOLS * sizeof(float) * (size_t)pool, "wavefield pools"))) return rc;
     float *F = (float *)ctx->fields.p;
+    if (!ctx->born_tuned) {
+        if ((rc = tune_depth(ctx, TRY_BORN, TRY_BORN_HIST, st))) return rc;
+        ctx->born_tuned = true;
+    }
     CK(cudaMemsetAsync(F, 0, sizeof(float) * 8 * (size_t)pool, st));
     BornArgs a{};
     a.c = common(ctx);

@@ -53,3 +53,27 @@ def test_trials_follow_the_records(monkeypatch):
         extra.append(launches[0] - launches[1])
         ctx.close()
     assert extra[0] == extra[1]
+
+
+def test_born_is_tried_by_the_first_born_call(monkeypatch):
+    """Programs that never call Born don't pay for its trials; those that do pay once,
+    whichever call came first."""
+    c, g, v = _case(monkeypatch)
+
+    def launches(calls):
+        ctx = gpu_ctx(c)
+        out = []
+        for call in calls:
+            if call == "model":
+                ctx.model_shots(v, g)
+            else:
+                ctx.born_demig(v, g, 0.01 * v)
+            out.append(ctx.stats()["kernel_launches"])
+        ctx.close()
+        return out
+
+    m0, m1, b0, b1 = launches(["model", "model", "born", "born"])
+    c0, c1, n0, n1 = launches(["born", "born", "model", "model"])
+    assert m0 > m1 and b0 > b1
+    assert c0 - c1 == (m0 - m1) + (b0 - b1)
+    assert n0 == n1
