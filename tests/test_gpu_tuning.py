@@ -77,3 +77,18 @@ def test_born_is_tried_by_the_first_born_call(monkeypatch):
     assert m0 > m1 and b0 > b1
     assert c0 - c1 == (m0 - m1) + (b0 - b1)
     assert n0 == n1
+
+
+def test_a_depth_is_not_fixed_by_one_sample(monkeypatch):
+    """Every depth trial runs once for warm-up and is timed twice: for Born on a plan
+    of one pair per launch three times four launches of both fields, four of the
+    scattered field from the history and eight single steps of it."""
+    c, g, v = _case(monkeypatch)
+    ctx = gpu_ctx(c)
+    ctx.model_shots(v, g)
+    launches = []
+    for _ in range(2):
+        ctx.born_demig(v, g, 0.01 * v)
+        launches.append(ctx.stats()["kernel_launches"])
+    ctx.close()
+    assert launches[0] - launches[1] == 3 * (4 + 4 + 8)
