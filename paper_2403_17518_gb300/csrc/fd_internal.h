@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 namespace dhfwi {
 
 // Stencil tile handled by one CTA: TZ rows x TX columns of one shot window.
@@ -105,6 +107,19 @@ __host__ __device__ inline long long model_row(int z, int NZ, int pf) {
     const int i = z < 0 ? 0 : z < NZ ? z : NZ - 1;
     return (long long)i * pf;
 }
+// A count per device (resident CTAs), taken by the first use on each: a kernel's
+// attributes and its occupancy belong to a device, and contexts may live on several.
+// Threads that come first together take the same count twice.
+struct PerDevice {
+    std::atomic<int> n[64] = {};
+    template <class Count>
+    int get(int dev, Count count) {
+        if (dev < 0 || dev >= 64) return count();
+        int v = n[dev].load(std::memory_order_acquire);
+        if (v == 0) n[dev].store(v = count(), std::memory_order_release);
+        return v;
+    }
+};
 // Most grown-region receiver entries the two-step adjoint's shared-memory
 // list holds (tiles with more read them from global memory when they open).
 constexpr int kInjCap = 256;

@@ -500,13 +500,14 @@ void launch_born_step_tma(const BornArgs &a, int ntiles, int variant, int grid, 
 
 void launch_born_hist_step(const BornArgs &a, int ntiles, const TileMaps &maps, cudaStream_t s) {
     if (ntiles <= 0) return;
-    static int cap = 0;
-    if (!cap) {
-        int dev = 0, nsm = 1;
-        cudaGetDevice(&dev);
+    static PerDevice ctas;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const int cap = ctas.get(dev, [&] {
+        int nsm = 1;
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        cap = occupancy((const void *)born_hist_tma_kernel<4>, 32 * (TZ / 4), kBornHistSmem) * nsm;
-    }
+        return occupancy((const void *)born_hist_tma_kernel<4>, 32 * (TZ / 4), kBornHistSmem) * nsm;
+    });
     launch_pdl(born_hist_tma_kernel<4>, ntiles < cap ? ntiles : cap, 4, kBornHistSmem, s, a, maps, ntiles);
 }
 

@@ -1179,33 +1179,28 @@ void launch_flow(K kernel, size_t smem, int threads, int cap, const Args &a, con
 }
 
 // CTAs of a kernel that are resident at once on the current device.
-int resident(const void *fn, size_t smem, int threads) {
-    int n = 0, dev = 0, sms = 1;
+template <auto KERNEL, size_t SMEM, int THREADS>
+int resident() {
+    static PerDevice ctas;
+    int dev = 0;
     cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, threads, smem);
-    return std::max(n, 1) * sms;
+    return ctas.get(dev, [&] {
+        int n = 0, sms = 1;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        cudaFuncSetAttribute((const void *)KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, (const void *)KERNEL, THREADS, SMEM);
+        return std::max(n, 1) * sms;
+    });
 }
 
 int cap_fwd(int store) {
-    static const int a = resident((const void *)fwd_pair_kernel<ST_A>, kPair2Smem, NT2),
-                     c = resident((const void *)fwd_pair_kernel<ST_CK>, kPair2Smem, NT2),
-                     n = resident((const void *)fwd_pair_kernel<ST_NONE>, kPair2Smem, NT2);
-    return store == ST_A ? a : store == ST_CK ? c : n;
+    return store == ST_A    ? resident<fwd_pair_kernel<ST_A>, kPair2Smem, NT2>()
+           : store == ST_CK ? resident<fwd_pair_kernel<ST_CK>, kPair2Smem, NT2>()
+                            : resident<fwd_pair_kernel<ST_NONE>, kPair2Smem, NT2>();
 }
-int cap_adj() {
-    static const int n = resident((const void *)adj_pair_kernel, kAdj2Smem, NT2);
-    return n;
-}
-int cap_born() {
-    static const int n = resident((const void *)born_pair_kernel, kBorn2Smem, NT2);
-    return n;
-}
-int cap_joint() {
-    static const int n = resident((const void *)born_joint_kernel, sizeof(JointSmem), NTJ);
-    return n;
-}
+int cap_adj() { return resident<adj_pair_kernel, kAdj2Smem, NT2>(); }
+int cap_born() { return resident<born_pair_kernel, kBorn2Smem, NT2>(); }
+int cap_joint() { return resident<born_joint_kernel, sizeof(JointSmem), NTJ>(); }
 
 }  // namespace
 

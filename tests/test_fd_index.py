@@ -1,5 +1,5 @@
-"""CPU checks of index arithmetic that the kernels share with the host
-(csrc/fd_internal.h), compiled as plain C++ and run at sizes past 2^31 cells."""
+"""CPU checks of what the kernels' header (csrc/fd_internal.h) shares with the host,
+compiled as plain C++: row offsets past 2^31 cells, launch limits per device."""
 import os
 import shutil
 import subprocess
@@ -31,3 +31,14 @@ def test_model_rows_of_large_models(tmp_path):
     got = [int(x) for x in run_host(tmp_path, body)]
     assert got == [min(max(z, 0), NZ - 1) * pf for z, NZ, pf in cases]
     assert max(got) >= 2**31
+
+
+def test_launch_limits_belong_to_a_device(tmp_path):
+    """Each device takes its own count, once; a device past the table takes it every time."""
+    body = """
+    static PerDevice p;
+    int taken = 0;
+    const int dev[] = {0, 1, 0, 63, 1, 64, 64};
+    for (int d : dev) std::printf("%d ", p.get(d, [&] { taken++; return 100 + d; }));
+    std::printf("%d", taken);"""
+    assert [int(x) for x in run_host(tmp_path, body)] == [100, 101, 100, 163, 101, 164, 164, 5]
