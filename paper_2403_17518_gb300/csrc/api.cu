@@ -841,26 +841,11 @@ int born_hist_maps(dhfwi_ctx *ctx, const BornArgs &b, TileMaps *M) {
 }
 
 // ---------------------------------------------------------------------------
-// Two-step launches (fd_tma2.cu).  A launch takes at most FLOW_PAIRS step pairs,
-// so that it ends within a fraction of a second at any size; one pair when all
-// its tiles are resident at once (see flow_pairs).
+// Two-step launches (fd_tma2.cu).  A launch takes at most FLOW_PAIRS step pairs
+// (64 shots of 400 x 1200: 12 ms of the forward sweep), or one when all its tiles
+// are resident at once (see flow_pairs).
 // ---------------------------------------------------------------------------
 constexpr int FLOW_PAIRS = 256;
-
-// The slots [s0, s1) that a sequence of two-step launches advances through all
-// its steps before the next ones.
-struct Group {
-    int s0, s1;
-};
-
-int group_nt(const Plan &P, const Group &g) { return P.nt_sorted[g.s0]; }  // its longest record
-
-// Cells of the group's shots active at step n.
-long long group_cells(const Plan &P, const Group &g, int n, int NZ) {
-    long long c = 0;
-    for (int k = g.s0; k < g.s1 && P.nt_sorted[k] > n; k++) c += (long long)P.shots[k].nxw * NZ;
-    return c;
-}
 
 // Step pairs per launch.  With at most one tile per resident CTA every tile
 // waits for its neighbours' stores of the pair before either way, and the end of
@@ -868,20 +853,17 @@ long long group_cells(const Plan &P, const Group &g, int n, int NZ) {
 // the per-tile flags: 101 x 101, 4 shots (36 tiles), 4.6 us per pair against
 // 6.2; from the second tile per CTA on the flags win (150 x 500, 25 shots, 525
 // tiles, migration: 14.5 ms against 16.5).
-int flow_pairs(const Plan &P, const Group &g, int kind) {
-    return P.tiles_prefix[g.s1] - P.tiles_prefix[g.s0] <= flow_ctas(kind) ? 1 : FLOW_PAIRS;
-}
+int flow_pairs(const Plan &P, int kind) { return (int)P.infos.size() <= flow_ctas(kind) ? 1 : FLOW_PAIRS; }
 
-// Common part of a launch over the group's tiles that are active at step n_any,
-// the step of the launch at which most of them are; zeroes their progress.
-int flow_args(dhfwi_ctx *ctx, const Group &g, int n_any, int npairs, FlowArgs *f, cudaStream_t st) {
+// Common part of a launch over the tiles that are active at step n_any, the step
+// of the launch at which most of them are; zeroes their progress.
+int flow_args(dhfwi_ctx *ctx, int n_any, int npairs, FlowArgs *f, cudaStream_t st) {
     const Plan &P = ctx->plan;
-    f->t0 = P.tiles_prefix[g.s0];
-    f->nt = std::min(active_tiles(P, n_any), P.tiles_prefix[g.s1]) - f->t0;
+    f->nt = active_tiles(P, n_any);
     f->npairs = npairs;
     f->act = (const int *)P.d_act.p;
     f->done = (unsigned *)P.d_done.p;
-    if (npairs > 1) CK(cudaMemsetAsync(f->done + f->t0, 0, sizeof(unsigned) * f->nt, st));
+    if (npairs > 1) CK(cudaMemsetAsync(f->done, 0, sizeof(unsigned) * f->nt, st));
     return DHFWI_OK;
 }
 
@@ -895,17 +877,17 @@ int flow_maps(dhfwi_ctx *ctx, float *const u[2], float *const d[2], CUtensorMap 
     return DHFWI_OK;
 }
 
-// Steps [n0, n1) of the group's shots, n1 - n0 even or n1 past their longest
-// record: the forward state (u in *cur, D in *dcur; the others are scratch and
-// take turns).  a holds what the launch stores and samples.
-int fwd_flow(dhfwi_ctx *ctx, FwdFlow &a, const Group &g, int n0, int n1, float *&cur, float *&nxt, float *&dcur,
-             float *&dnxt, cudaStream_t st) {
-    n1 = std::min(n1, group_nt(ctx->plan, g));
-    const int most = flow_pairs(ctx->plan, g, FLOW_FWD);
+// Steps [n0, n1), n1 - n0 even or n1 past the longest record: the forward state
+// (u in *cur, D in *dcur; the others are scratch and take turns).  a holds what
+// the launch stores and samples.
+int fwd_flow(dhfwi_ctx *ctx, FwdFlow &a, int n0, int n1, float *&cur, float *&nxt, float *&dcur, float *&dnxt,
+             cudaStream_t st) {
+    n1 = std::min(n1, ctx->plan.nt_sorted[0]);
+    const int most = flow_pairs(ctx->plan, FLOW_FWD);
     for (int n = n0; n < n1; n += 2 * most) {
         const int np = std::min(most, (n1 - n + 1) / 2);
         int rc;
-        if ((rc = flow_args(ctx, g, n, np, &a.f, st))) return rc;
+        if ((rc = flow_args(ctx, n, np, &a.f, st))) return rc;
         a.n0 = n;
         a.u[0] = cur;
         a.u[1] = nxt;
@@ -915,7 +897,7 @@ int fwd_flow(dhfwi_ctx *ctx, FwdFlow &a, const Group &g, int n0, int n1, float *
         if ((rc = flow_maps(ctx, a.u, a.d, &M.m[0], &M.m[2]))) return rc;
         launch_fwd_flow(a, M, st);
         ctx->stats.kernel_launches++;
-        for (int i = n; i < n + 2 * np && i < n1; i++) ctx->stats.cell_updates += group_cells(ctx->plan, g, i, ctx->NZ);
+        for (int i = n; i < n + 2 * np && i < n1; i++) ctx->stats.cell_updates += active_cells(ctx->plan, i, ctx->NZ);
         if (np & 1) {
             std::swap(cur, nxt);
             std::swap(dcur, dnxt);
@@ -925,15 +907,15 @@ int fwd_flow(dhfwi_ctx *ctx, FwdFlow &a, const Group &g, int n0, int n1, float *
     return DHFWI_OK;
 }
 
-// Adjoint steps k1 .. n0 + 1 (an even number) of the group's shots, state as
-// above; those with shorter records join as k comes down to them.
-int adj_flow(dhfwi_ctx *ctx, AdjFlow &b, const Group &g, int k1, int n0, float *&cur, float *&nxt, float *&dcur,
-             float *&dnxt, cudaStream_t st) {
-    const int most = flow_pairs(ctx->plan, g, FLOW_ADJ);
+// Adjoint steps k1 .. n0 + 1 (an even number), state as above; shots with shorter
+// records join as k comes down to them.
+int adj_flow(dhfwi_ctx *ctx, AdjFlow &b, int k1, int n0, float *&cur, float *&nxt, float *&dcur, float *&dnxt,
+             cudaStream_t st) {
+    const int most = flow_pairs(ctx->plan, FLOW_ADJ);
     for (int k = k1; k > n0; k -= 2 * most) {
         const int np = std::min(most, (k - n0) / 2);
         int rc;
-        if ((rc = flow_args(ctx, g, k - 2 * np, np, &b.f, st))) return rc;
+        if ((rc = flow_args(ctx, k - 2 * np, np, &b.f, st))) return rc;
         b.k1 = k;
         b.nu[0] = cur;
         b.nu[1] = nxt;
@@ -943,7 +925,7 @@ int adj_flow(dhfwi_ctx *ctx, AdjFlow &b, const Group &g, int k1, int n0, float *
         if ((rc = flow_maps(ctx, b.nu, b.d, &M.m[0], &M.m[2]))) return rc;
         launch_adj_flow(b, M, st);
         ctx->stats.kernel_launches++;
-        for (int i = k - 2 * np; i < k; i++) ctx->stats.cell_updates += group_cells(ctx->plan, g, i, ctx->NZ);
+        for (int i = k - 2 * np; i < k; i++) ctx->stats.cell_updates += active_cells(ctx->plan, i, ctx->NZ);
         if (np & 1) {
             std::swap(cur, nxt);
             std::swap(dcur, dnxt);
@@ -953,15 +935,15 @@ int adj_flow(dhfwi_ctx *ctx, AdjFlow &b, const Group &g, int k1, int n0, float *
     return DHFWI_OK;
 }
 
-// Born steps [0, n1) of the group's shots from zero state: both fields, or
-// (from_history) the scattered one with a^n from b.a.
-int born_flow(dhfwi_ctx *ctx, BornFlow b, const Group &g, int n1, bool from_history, cudaStream_t st) {
-    n1 = std::min(n1, group_nt(ctx->plan, g));
-    const int most = flow_pairs(ctx->plan, g, from_history ? FLOW_BORN_HIST : FLOW_BORN);
+// Born steps [0, n1) from zero state: both fields, or (from_history) the scattered
+// one with a^n from b.a.
+int born_flow(dhfwi_ctx *ctx, BornFlow b, int n1, bool from_history, cudaStream_t st) {
+    n1 = std::min(n1, ctx->plan.nt_sorted[0]);
+    const int most = flow_pairs(ctx->plan, from_history ? FLOW_BORN_HIST : FLOW_BORN);
     for (int n = 0; n < n1; n += 2 * most) {
         const int np = std::min(most, (n1 - n + 1) / 2);
         int rc;
-        if ((rc = flow_args(ctx, g, n, np, &b.f, st))) return rc;
+        if ((rc = flow_args(ctx, n, np, &b.f, st))) return rc;
         b.n0 = n;
         TileMaps M;
         if (from_history) {
@@ -974,7 +956,7 @@ int born_flow(dhfwi_ctx *ctx, BornFlow b, const Group &g, int n1, bool from_hist
         }
         ctx->stats.kernel_launches++;
         for (int i = n; i < n + 2 * np && i < n1; i++)
-            ctx->stats.cell_updates += (from_history ? 1 : 2) * group_cells(ctx->plan, g, i, ctx->NZ);
+            ctx->stats.cell_updates += (from_history ? 1 : 2) * active_cells(ctx->plan, i, ctx->NZ);
         if (np & 1) {
             std::swap(b.u[0], b.u[1]);
             std::swap(b.du[0], b.du[1]);
@@ -985,9 +967,6 @@ int born_flow(dhfwi_ctx *ctx, BornFlow b, const Group &g, int n1, bool from_hist
     CK(cudaGetLastError());
     return DHFWI_OK;
 }
-
-// Groups of the slots for the two-step launches: all of them together.
-std::vector<Group> groups_of(const Plan &P) { return {Group{0, P.n_shots}}; }
 
 // Time-blocking depth: a two-step launch of a few pairs on the plan's full tile
 // list against the chosen one-step kernel's time for as many steps.  The faster
@@ -1002,14 +981,13 @@ int depth_trial(dhfwi_ctx *ctx, int which, int np, cudaStream_t st) {
     const Plan &P = ctx->plan;
     const long long pool = P.pool_floats;
     float *F = (float *)ctx->fields.p;
-    const Group all{0, P.n_shots};
     int rc = DHFWI_OK;
     if (which == TRY_FWD) {
         FwdFlow a{};
         a.c = common(ctx);
         a.rec = (float *)ctx->dtmp.p;
         float *u = F, *un = F + pool, *d = F + 2 * pool, *dn = F + 7 * pool;
-        return fwd_flow(ctx, a, all, 0, 2 * np, u, un, d, dn, st);
+        return fwd_flow(ctx, a, 0, 2 * np, u, un, d, dn, st);
     }
     if (which == TRY_ADJ) {
         AdjFlow b{};
@@ -1018,7 +996,7 @@ int depth_trial(dhfwi_ctx *ctx, int which, int np, cudaStream_t st) {
         b.g = F + 4 * pool;
         b.r = (const float *)ctx->rtmp.p;
         float *u = F, *un = F + pool, *d = F + 2 * pool, *dn = F + 8 * pool;
-        return adj_flow(ctx, b, all, 2 * np, 0, u, un, d, dn, st);
+        return adj_flow(ctx, b, 2 * np, 0, u, un, d, dn, st);
     }
     if (which == TRY_HIST_ONE) {
         BornArgs b{};
@@ -1048,7 +1026,7 @@ int depth_trial(dhfwi_ctx *ctx, int which, int np, cudaStream_t st) {
     b.p[1] = F + 4 * pool;
     b.dp[0] = F + 5 * pool;
     b.dp[1] = F + 6 * pool;
-    return born_flow(ctx, b, all, 2 * np, which == TRY_BORN_HIST, st);
+    return born_flow(ctx, b, 2 * np, which == TRY_BORN_HIST, st);
 }
 
 // Time of a trial: the better of two after one for warm-up, so that one disturbed
@@ -1135,30 +1113,28 @@ int run_forward(dhfwi_ctx *ctx, float *uA, float *uB, float *dd, float *dd2, flo
     if (time_blocking(ctx, 0)) {
         // K and H are even (or H is the last step): a pair never straddles a
         // segment or the end of the history.
-        for (const Group &g : groups_of(P)) {
-            float *cur = uA, *nxt = uB, *dcur = dd, *dnxt = dd2;
-            const long long cn = ctx->stats.cell_updates;
-            if (H > 0) {
-                FwdFlow a{};
-                a.c = common(ctx);
-                a.rec = d;
-                a.a.base = hist;
-                a.a.off = (const long long *)ctx->d_hoff.p;
-                a.a.last = H - 1;
-                if ((rc = fwd_flow(ctx, a, g, 0, H, cur, nxt, dcur, dnxt, st))) return rc;
-                ctx->stats.history_cells += ctx->stats.cell_updates - cn;
-            }
+        float *cur = uA, *nxt = uB, *dcur = dd, *dnxt = dd2;
+        const long long cn = ctx->stats.cell_updates;
+        if (H > 0) {
             FwdFlow a{};
             a.c = common(ctx);
             a.rec = d;
-            if (backward && H < P.nt_max) {
-                a.ck = ck;
-                a.ck_every = K;
-                a.ck_first = S;
-                a.pool = pool;
-            }
-            if ((rc = fwd_flow(ctx, a, g, H, P.nt_max, cur, nxt, dcur, dnxt, st))) return rc;
+            a.a.base = hist;
+            a.a.off = (const long long *)ctx->d_hoff.p;
+            a.a.last = H - 1;
+            if ((rc = fwd_flow(ctx, a, 0, H, cur, nxt, dcur, dnxt, st))) return rc;
+            ctx->stats.history_cells += ctx->stats.cell_updates - cn;
         }
+        FwdFlow a{};
+        a.c = common(ctx);
+        a.rec = d;
+        if (backward && H < P.nt_max) {
+            a.ck = ck;
+            a.ck_every = K;
+            a.ck_first = S;
+            a.pool = pool;
+        }
+        if ((rc = fwd_flow(ctx, a, H, P.nt_max, cur, nxt, dcur, dnxt, st))) return rc;
     } else {
         FwdArgs a{};
         a.c = common(ctx);
@@ -1220,84 +1196,74 @@ int run_backward(dhfwi_ctx *ctx, float *w, float *w2, float *w3, float *w4, floa
     const long long l0 = ctx->stats.kernel_launches, c0 = ctx->stats.cell_updates;
     int rc;
     phase_begin(ctx, 1, st);
-    // Groups share no state, so each goes back through all its steps by itself
-    // (one group when a part of the sweep takes one step per launch).
-    const std::vector<Group> groups = blocking && blocking_adj ? groups_of(P) : std::vector<Group>{{0, P.n_shots}};
-    for (const Group &g : groups) {
-        const int nt = group_nt(P, g);
-        const int t0 = P.tiles_prefix[g.s0];
-        const size_t goff = P.shots[g.s0].foff, glen = (size_t)(g.s1 - g.s0) * ctx->NZ * P.pitch;
-        float *ncur = nuA, *nnxt = nuB, *dcur_nu = nud, *dnxt_nu = nud2;
-        // The adjoint over the steps n1 .. n0 + 1, a^n from sa.
-        auto adjoint = [&](int n0, int n1, const ASteps &sa, auto slot) -> int {
-            AdjArgs b{};
-            b.c = common(ctx);
-            b.c.infos += t0;
-            b.c.tiles += t0;
-            b.r = r;
-            b.g = gpool;
-            int k = n1;
-            for (; k > n0 && (!blocking_adj || (k - n0) % 2); k--) {  // one step per launch
-                b.nu = ncur;
-                b.nun = nnxt;
-                b.dd = dcur_nu;
-                b.a = slot(k - 1);
-                b.k = k;
-                const int tiles = std::min(active_tiles(P, k - 1), P.tiles_prefix[g.s1]) - t0;
-                if ((rc = adj_step(ctx, b, tiles, ctx->launch[2], st))) return rc;
-                ctx->stats.kernel_launches++;
-                ctx->stats.cell_updates += group_cells(P, g, k - 1, ctx->NZ);
-                std::swap(ncur, nnxt);
-            }
-            if (k == n0) return DHFWI_OK;
-            AdjFlow f{};
+    const int nt = P.nt_sorted[0];  // the longest record
+    float *ncur = nuA, *nnxt = nuB, *dcur_nu = nud, *dnxt_nu = nud2;
+    // The adjoint over the steps n1 .. n0 + 1, a^n from sa.
+    auto adjoint = [&](int n0, int n1, const ASteps &sa, auto slot) -> int {
+        AdjArgs b{};
+        b.c = common(ctx);
+        b.r = r;
+        b.g = gpool;
+        int k = n1;
+        for (; k > n0 && (!blocking_adj || (k - n0) % 2); k--) {  // one step per launch
+            b.nu = ncur;
+            b.nun = nnxt;
+            b.dd = dcur_nu;
+            b.a = slot(k - 1);
+            b.k = k;
+            if ((rc = adj_step(ctx, b, active_tiles(P, k - 1), ctx->launch[2], st))) return rc;
+            ctx->stats.kernel_launches++;
+            ctx->stats.cell_updates += active_cells(P, k - 1, ctx->NZ);
+            std::swap(ncur, nnxt);
+        }
+        if (k == n0) return DHFWI_OK;
+        AdjFlow f{};
+        f.c = common(ctx);
+        f.r = r;
+        f.g = gpool;
+        f.a = sa;
+        return adj_flow(ctx, f, k, n0, ncur, nnxt, dcur_nu, dnxt_nu, st);
+    };
+    // Segments whose a^n is recomputed from checkpoints, the last first.
+    for (int js = (nt + K - 1) / K - 1; js >= S; js--) {
+        const int n0 = js * K, n1 = std::min(n0 + K, nt);
+        float *cur = ck + (2 * (long long)(js - S)) * pool, *nxt = w;
+        float *dcur = ck + (2 * (long long)(js - S) + 1) * pool, *dnxt = w2;
+        if (ctx->reuse) {
+            CK(cudaMemcpyAsync(w3, cur, sizeof(float) * (size_t)pool, cudaMemcpyDeviceToDevice, st));
+            CK(cudaMemcpyAsync(w4, dcur, sizeof(float) * (size_t)pool, cudaMemcpyDeviceToDevice, st));
+            cur = w3;
+            dcur = w4;
+        } else {
+            ctx->fws.valid = false;
+        }
+        ASteps sa;
+        sa.base = abuf;
+        sa.first = n0;
+        sa.stride = pool;
+        auto slot = [&](int n) -> float * { return abuf + (long long)(n - n0) * pool; };
+        if (blocking) {
+            FwdFlow f{};
             f.c = common(ctx);
-            f.r = r;
-            f.g = gpool;
             f.a = sa;
-            return adj_flow(ctx, f, g, k, n0, ncur, nnxt, dcur_nu, dnxt_nu, st);
-        };
-        // Segments whose a^n is recomputed from checkpoints, the last first.
-        for (int js = (nt + K - 1) / K - 1; js >= S; js--) {
-            const int n0 = js * K, n1 = std::min(n0 + K, nt);
-            float *cur = ck + (2 * (long long)(js - S)) * pool, *nxt = w;
-            float *dcur = ck + (2 * (long long)(js - S) + 1) * pool, *dnxt = w2;
-            if (ctx->reuse) {
-                CK(cudaMemcpyAsync(w3 + goff, cur + goff, sizeof(float) * glen, cudaMemcpyDeviceToDevice, st));
-                CK(cudaMemcpyAsync(w4 + goff, dcur + goff, sizeof(float) * glen, cudaMemcpyDeviceToDevice, st));
-                cur = w3;
-                dcur = w4;
-            } else {
-                ctx->fws.valid = false;
-            }
-            ASteps sa;
-            sa.base = abuf;
-            sa.first = n0;
-            sa.stride = pool;
-            auto slot = [&](int n) -> float * { return abuf + (long long)(n - n0) * pool; };
-            if (blocking) {
-                FwdFlow f{};
-                f.c = common(ctx);
-                f.a = sa;
-                if ((rc = fwd_flow(ctx, f, g, n0, n1, cur, nxt, dcur, dnxt, st))) return rc;
-            } else {
-                FwdArgs f{};
-                f.c = common(ctx);
-                for (int n = n0; n < n1; n++)
-                    if ((rc = forward_step(ctx, f, n, cur, nxt, dcur, ctx->launch[1], slot, st))) return rc;
-            }
-            if ((rc = adjoint(n0, n1, sa, slot))) return rc;
+            if ((rc = fwd_flow(ctx, f, n0, n1, cur, nxt, dcur, dnxt, st))) return rc;
+        } else {
+            FwdArgs f{};
+            f.c = common(ctx);
+            for (int n = n0; n < n1; n++)
+                if ((rc = forward_step(ctx, f, n, cur, nxt, dcur, ctx->launch[1], slot, st))) return rc;
         }
-        if (H > 0) {  // the stored steps
-            ASteps sa;
-            sa.base = hist;
-            sa.off = (const long long *)ctx->d_hoff.p;
-            sa.last = H - 1;
-            auto slot = [&](int n) -> float * { return hist + ctx->hoff[n]; };
-            if ((rc = adjoint(0, std::min(H, nt), sa, slot))) return rc;
-        }
-        CK(cudaGetLastError());
+        if ((rc = adjoint(n0, n1, sa, slot))) return rc;
     }
+    if (H > 0) {  // the stored steps
+        ASteps sa;
+        sa.base = hist;
+        sa.off = (const long long *)ctx->d_hoff.p;
+        sa.last = H - 1;
+        auto slot = [&](int n) -> float * { return hist + ctx->hoff[n]; };
+        if ((rc = adjoint(0, std::min(H, nt), sa, slot))) return rc;
+    }
+    CK(cudaGetLastError());
     phase_end(ctx, 1, st, ctx->stats.kernel_launches - l0, ctx->stats.cell_updates - c0);
     return DHFWI_OK;
 }
@@ -1638,8 +1604,7 @@ int born_demig(dhfwi_ctx *ctx, const float *v0_dev, const dhfwi_geom *geom, cons
             b.a.last = P.nt_max - 1;
             ctx->stats.reused |= 2;
         }
-        for (const Group &g : groups_of(P))
-            if ((rc = born_flow(ctx, b, g, P.nt_max, from_history, st))) return rc;
+        if ((rc = born_flow(ctx, b, P.nt_max, from_history, st))) return rc;
         phase_end(ctx, 2, st, ctx->stats.kernel_launches - l0, ctx->stats.cell_updates - c0);
         return end_call(ctx);
     }

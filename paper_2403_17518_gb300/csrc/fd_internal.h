@@ -201,14 +201,14 @@ int step_variants(int kind);
 // Resident CTAs per SM of a step kernel; kind 0 forward, 1 adjoint, 2 Born.
 int step_occupancy(int kind, int variant, int store_a);
 
-// Two-step (time-blocked) launches (fd_tma2.cu): npairs step pairs of the nt
-// tiles from t0 on, in one cooperative launch.
+// Two-step (time-blocked) launches (fd_tma2.cu): npairs step pairs of the
+// plan's first nt tiles in one cooperative launch.
 constexpr int HALO2 = 2 * HALO;
 constexpr int U2PITCH = TX + 2 * HALO2 + 4;  // columns of its u^n box (shared-memory row pitch)
 struct FlowArgs {
     unsigned *done;  // per tile of the plan: pairs done by this launch (zeroed before a launch of several)
     const int *act;  // act[n]: tiles of the plan with nt > n (a prefix)
-    int t0, nt, npairs;
+    int nt, npairs;
 };
 // a^n per step: base + off[n] (a stored history; off has last + 1 entries), or,
 // without off, base + (n - first) * stride.

@@ -219,8 +219,8 @@ struct PairSmem {
 
 // ---------------------------------------------------------------------------
 // The item loop.  CTA b takes the items b, b + gridDim.x, ... of the sequence
-// of pairs m = 0, 1, ... with count(m) tiles each (from the launch's first tile
-// on: shots by record length, so the active ones are a prefix).  The launch is
+// of pairs m = 0, 1, ... with count(m) tiles each (shots by record length, so
+// the active ones are a prefix).  The launch is
 // cooperative, so all CTAs are resident; items are taken in order, so the
 // first unfinished one never waits for a later one, and every wait ends.
 //
@@ -331,16 +331,15 @@ __device__ __forceinline__ void run_flow(const FlowArgs &F, const StepCommon &c,
             __syncwarp();
             return;
         }
-        const int tile = F.t0 + i;
         if (lane < 5)
-            reinterpret_cast<int4 *>(&it.T)[lane] = __ldg(reinterpret_cast<const int4 *>(&c.infos[tile]) + lane);
+            reinterpret_cast<int4 *>(&it.T)[lane] = __ldg(reinterpret_cast<const int4 *>(&c.infos[i]) + lane);
         __syncwarp();
         const TileInfo &T = it.T;
         if (lane < 6) it.p[lane] = k.ptr(lane, m, T);
         if (lane == 6) {
             const int n = k.step(m);
             it.m = m;
-            it.tile = tile;
+            it.tile = i;
             it.n = n;
             it.need = k.need(m, T);
             it.row = k.row(m, T);
@@ -565,7 +564,7 @@ __device__ __forceinline__ void pair_tile(const FwdFlow &A, const Pair2Stage &S,
 // (pairs n0 + 2 m) and the arrays' addresses.
 __device__ __forceinline__ long long cell0(const TileInfo &T) { return T.foff + (long long)T.z0 * T.pitch + T.x0; }
 __device__ __forceinline__ int active_count(const FlowArgs &F, int n) {
-    return min(max(__ldg(F.act + n) - F.t0, 0), F.nt);
+    return min(__ldg(F.act + n), F.nt);
 }
 // a^n of a launch: a stored history's step, or a slot of a segment buffer.
 __device__ __forceinline__ float *a_at(const ASteps &a, int n) {
