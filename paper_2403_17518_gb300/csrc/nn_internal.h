@@ -87,26 +87,23 @@ int wgrad_splits(long long kpix, int M, int N);
 // Weight gradient into dw (parameter layout) and bias gradient into db.
 // Returns the number of kernels launched.
 int launch_wgrad(const WgradArgs &a, int splits, float *dw, float *db, cudaStream_t s);
+// Pooling and the d(cat) split take C, strides and offsets that are multiples of 8
+// and 16-byte aligned buffers (every network width, workspace arena); the split an
+// even H and W (a level above another one).
 void launch_avgpool_fwd(const __nv_bfloat16 *x, int xs, int xo, int nimg, int H, int W, int C, __nv_bfloat16 *y,
                         cudaStream_t s);
-void launch_avgpool_bwd(const float *dy, int nimg, int H, int W, int C, float *dx, int accumulate, cudaStream_t s);
-void launch_leaky_bwd(const float *dA, const __nv_bfloat16 *a, int as, int ao, long long P, int C, float slope,
-                      __nv_bfloat16 *g, cudaStream_t s);
-void launch_f32_to_bf16_slice(const float *x, int xs, int xo, long long P, int C, __nv_bfloat16 *y, cudaStream_t s);
-// Fused forms (false: not launched, shapes or alignment not met): d(cat)
-// [P][2C] on an H x W grid into its skip half (f32, [P][C]) and upsampled
-// half (bf16, space-to-depth onto the H/2 x W/2 grid, see WgradArgs::g_s2d); the average
-// pool's backward plus a skip gradient times the LeakyReLU derivative of
-// act, in bf16 (avgpool_bwd, add_slice and leaky_bwd in one pass).
-bool launch_split_cat(const float *src, int nimg, int H, int W, int C, float *skip, __nv_bfloat16 *up,
+// The average pool's backward plus a skip gradient times the LeakyReLU derivative
+// of act, in bf16.
+void launch_avgpool_bwd_leaky(const float *dy, int nimg, int H, int W, int C, const float *skip,
+                              const __nv_bfloat16 *act, int as, int ao, float slope, __nv_bfloat16 *g,
+                              cudaStream_t s);
+// d(cat) [P][2C] on an H x W grid into its skip half (f32, [P][C]) and upsampled
+// half (bf16, space-to-depth onto the H/2 x W/2 grid, see WgradArgs::g_s2d).
+void launch_split_cat(const float *src, int nimg, int H, int W, int C, float *skip, __nv_bfloat16 *up,
                       cudaStream_t s);
 // f32 output gradient of a transposed conv on the fine grid (nimg x 2H x 2W x
 // C) into bf16 space-to-depth layout [nimg][H][W][2a+b][C].
 void launch_to_bf16_s2d(const float *x, int nimg, int H, int W, int C, __nv_bfloat16 *y, cudaStream_t s);
-bool launch_avgpool_bwd_leaky(const float *dy, int nimg, int H, int W, int C, const float *skip,
-                              const __nv_bfloat16 *act, int as, int ao, float slope, __nv_bfloat16 *g,
-                              cudaStream_t s);
-void launch_add_slice(const float *src, int ss, int so, long long P, int C, float *dst, cudaStream_t s);
 void launch_conv1x1_fwd(const __nv_bfloat16 *a, int C, long long P, const __nv_bfloat16 *w, const float *b, float *out,
                         cudaStream_t s);
 void launch_mse(const float *out, const float *y, long long P, __nv_bfloat16 *g, double *partial, int nblocks,

@@ -659,153 +659,6 @@ __global__ void bias_grad_final_kernel(const float *__restrict__ part, int nblk,
 // ---------------------------------------------------------------------------
 // Elementwise and small kernels
 // ---------------------------------------------------------------------------
-// Average pool 3x3, stride 2, zero padding 1 counted (divide by 9); output bf16.
-__global__ void avgpool_fwd_kernel(const __nv_bfloat16 *__restrict__ x, int xs, int xo, int nimg, int H, int W, int C,
-                                   __nv_bfloat16 *__restrict__ y) {
-    const int Ho = (H - 1) / 2 + 1, Wo = (W - 1) / 2 + 1;
-    const long long n = (long long)nimg * Ho * Wo * C;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(i % C);
-        long long r = i / C;
-        const int wo = (int)(r % Wo);
-        r /= Wo;
-        const int ho = (int)(r % Ho);
-        const int img = (int)(r / Ho);
-        float s = 0.f;
-        for (int a = 0; a < 3; a++) {
-            const int h = 2 * ho + a - 1;
-            if (h < 0 || h >= H) continue;
-            for (int b = 0; b < 3; b++) {
-                const int w = 2 * wo + b - 1;
-                if (w < 0 || w >= W) continue;
-                s += __bfloat162float(x[(((long long)img * H + h) * W + w) * xs + xo + c]);
-            }
-        }
-        y[i] = __float2bfloat16_rn(s * (1.0f / 9.0f));
-    }
-}
-
-// dx[h][w] (+)= sum of dy/9 over the pooling windows containing (h, w).
-// Four channels per thread (C a multiple of 4, 16-byte aligned rows): the
-// same sums in the same order as avgpool_bwd_kernel.
-__global__ void avgpool_bwd4_kernel(const float *__restrict__ dy, int nimg, int H, int W, int C4,
-                                    float *__restrict__ dx, int accumulate) {
-    const int Ho = (H - 1) / 2 + 1, Wo = (W - 1) / 2 + 1;
-    const long long n = (long long)nimg * H * W * C4;
-    const float4 *dy4 = reinterpret_cast<const float4 *>(dy);
-    float4 *dx4 = reinterpret_cast<float4 *>(dx);
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(i % C4);
-        const long long r0 = i / C4;
-        const int w = (int)(r0 % W);
-        const long long r1 = r0 / W;
-        const int h = (int)(r1 % H);
-        const long long img = r1 / H;
-        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int ho = (h > 0 ? h / 2 : 0); ho <= (h + 1) / 2 && ho < Ho; ho++) {
-            if (2 * ho - 1 > h || 2 * ho + 1 < h) continue;
-            for (int wo = (w > 0 ? w / 2 : 0); wo <= (w + 1) / 2 && wo < Wo; wo++) {
-                if (2 * wo - 1 > w || 2 * wo + 1 < w) continue;
-                const float4 v = dy4[((img * Ho + ho) * Wo + wo) * C4 + c];
-                s.x += v.x;
-                s.y += v.y;
-                s.z += v.z;
-                s.w += v.w;
-            }
-        }
-        const float k = 1.0f / 9.0f;
-        s.x *= k;
-        s.y *= k;
-        s.z *= k;
-        s.w *= k;
-        if (accumulate) {
-            const float4 o = dx4[i];
-            s.x = o.x + s.x;
-            s.y = o.y + s.y;
-            s.z = o.z + s.z;
-            s.w = o.w + s.w;
-        }
-        dx4[i] = s;
-    }
-}
-
-__global__ void avgpool_bwd_kernel(const float *__restrict__ dy, int nimg, int H, int W, int C, float *__restrict__ dx,
-                                   int accumulate) {
-    const int Ho = (H - 1) / 2 + 1, Wo = (W - 1) / 2 + 1;
-    const long long n = (long long)nimg * H * W * C;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(i % C);
-        long long r = i / C;
-        const int w = (int)(r % W);
-        r /= W;
-        const int h = (int)(r % H);
-        const int img = (int)(r / H);
-        float s = 0.f;
-        // Windows (ho, wo) with 2ho-1 <= h <= 2ho+1.
-        for (int ho = (h > 0 ? (h) / 2 : 0); ho <= (h + 1) / 2 && ho < Ho; ho++) {
-            if (2 * ho - 1 > h || 2 * ho + 1 < h) continue;
-            for (int wo = (w > 0 ? (w) / 2 : 0); wo <= (w + 1) / 2 && wo < Wo; wo++) {
-                if (2 * wo - 1 > w || 2 * wo + 1 < w) continue;
-                s += dy[(((long long)img * Ho + ho) * Wo + wo) * C + c];
-            }
-        }
-        s *= (1.0f / 9.0f);
-        dx[i] = accumulate ? dx[i] + s : s;
-    }
-}
-
-// g = bf16(dA * (a > 0 ? 1 : slope)) for a LeakyReLU output a (bf16, with
-// channel stride/offset), dA float32 dense [P][C].
-__global__ void leaky_bwd_kernel(const float *__restrict__ dA, const __nv_bfloat16 *__restrict__ a, int as, int ao,
-                                 long long P, int C, float slope, __nv_bfloat16 *__restrict__ g) {
-    const long long n = P * C;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const long long p = i / C;
-        const int c = (int)(i - p * C);
-        const float av = __bfloat162float(a[p * as + ao + c]);
-        g[i] = __float2bfloat16_rn(dA[i] * (av > 0.f ? 1.0f : slope));
-    }
-}
-
-__global__ void leaky_bwd4_kernel(const float4 *__restrict__ dA, const __nv_bfloat16 *__restrict__ a, int as, int ao,
-                                  long long P, int C4, float slope, Bf16x4 *__restrict__ g) {
-    const long long n = P * C4;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const long long p = i / C4;
-        const int c = (int)(i - p * C4) * 4;
-        const float4 av = bf4_to_f4(*reinterpret_cast<const Bf16x4 *>(a + p * as + ao + c));
-        const float4 d = dA[i];
-        g[i] = f4_to_bf4(make_float4(d.x * (av.x > 0.f ? 1.0f : slope), d.y * (av.y > 0.f ? 1.0f : slope),
-                                     d.z * (av.z > 0.f ? 1.0f : slope), d.w * (av.w > 0.f ? 1.0f : slope)));
-    }
-}
-
-__global__ void f32_to_bf16_slice4_kernel(const float *__restrict__ x, int xs, int xo, long long P, int C4,
-                                          Bf16x4 *__restrict__ y) {
-    const long long n = P * C4;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const long long p = i / C4;
-        const int c = (int)(i - p * C4) * 4;
-        y[i] = f4_to_bf4(*reinterpret_cast<const float4 *>(x + p * xs + xo + c));
-    }
-}
-
-__global__ void add_slice4_kernel(const float *__restrict__ src, int ss, int so, long long P, int C4,
-                                  float4 *__restrict__ dst) {
-    const long long n = P * C4;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const long long p = i / C4;
-        const int c = (int)(i - p * C4) * 4;
-        const float4 v = *reinterpret_cast<const float4 *>(src + p * ss + so + c);
-        float4 d = dst[i];
-        d.x += v.x;
-        d.y += v.y;
-        d.z += v.z;
-        d.w += v.w;
-        dst[i] = d;
-    }
-}
-
 // d(cat) [P][2C] of a decoder level (H x W grid) split into its halves: the
 // skip half copied (f32, [P][C]) for the encoder's backward, the upsampled
 // half rounded to bf16 in space-to-depth layout [img][H/2][W/2][2a+b][C]
@@ -842,8 +695,9 @@ __global__ void to_bf16_s2d_kernel(const float *__restrict__ x, int nimg, int H,
     }
 }
 
-// The 3x3 / stride-2 average pool with eight channels per thread (16-byte bf16
-// accesses; C, strides and offsets multiples of 8, which every network width is).
+// The 3x3 / stride-2 average pool (zero padding 1 counted: divided by 9) with eight
+// channels per thread (16-byte bf16 accesses; C, strides and offsets multiples of 8,
+// which every network width is).
 // Bound by HBM at the top level and by load latency below, so all loads of an output
 // are issued before its sum (in the window's order).  Its four launches on 32 patches
 // of 128 x 128 at base 32 take 50 us, what four channels per thread took too: the
@@ -883,8 +737,7 @@ __global__ void avgpool_fwd8_kernel(const __nv_bfloat16 *__restrict__ x, int xs,
 
 // Backward of the pool, plus the skip gradient of the same activation, times the
 // LeakyReLU derivative of that activation (bf16 act, stride as, offset ao): the next
-// block's output gradient g in bf16, as avgpool_bwd, add_slice and leaky_bwd in turn
-// would give it.  Eight channels per thread and the up to four windows' loads first:
+// block's output gradient g in bf16, every step rounded to float32.  Eight channels per thread and the up to four windows' loads first:
 // 108.4 -> 80.0 us for the four launches of the size above (four channels, one
 // window at a time).
 __global__ void avgpool_bwd_leaky8_kernel(const float4 *__restrict__ dy, int nimg, int H, int W, int C8,
@@ -927,28 +780,6 @@ __global__ void avgpool_bwd_leaky8_kernel(const float4 *__restrict__ dy, int nim
             }
             g[i] = Bf16x8{out[0], out[1]};
         }
-    }
-}
-
-// Copy channels [off, off+C) of a float32 [P][Ct] tensor into bf16 [P][C].
-__global__ void f32_to_bf16_slice_kernel(const float *__restrict__ x, int xs, int xo, long long P, int C,
-                                         __nv_bfloat16 *__restrict__ y) {
-    const long long n = P * C;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const long long p = i / C;
-        const int c = (int)(i - p * C);
-        y[i] = __float2bfloat16_rn(x[p * xs + xo + c]);
-    }
-}
-
-// dst[P][C] += src[P][Cs] channels [off, off+C)  (float32)
-__global__ void add_slice_kernel(const float *__restrict__ src, int ss, int so, long long P, int C,
-                                 float *__restrict__ dst) {
-    const long long n = P * C;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const long long p = i / C;
-        const int c = (int)(i - p * C);
-        dst[i] += src[p * ss + so + c];
     }
 }
 
@@ -1703,64 +1534,23 @@ int launch_wgrad(const WgradArgs &a, int splits, float *dw, float *db, cudaStrea
 
 void launch_avgpool_fwd(const __nv_bfloat16 *x, int xs, int xo, int nimg, int H, int W, int C, __nv_bfloat16 *y,
                         cudaStream_t s) {
-    const long long n = (long long)nimg * ((H - 1) / 2 + 1) * ((W - 1) / 2 + 1) * C;
-    if (C % 8 == 0 && ((xs | xo) & 7) == 0 && (((uintptr_t)x | (uintptr_t)y) & 15) == 0)
-        avgpool_fwd8_kernel<<<row_grid(((W - 1) / 2 + 1) * (C / 8), nimg * ((H - 1) / 2 + 1)), 256, 0, s>>>(
-            x, xs, xo, nimg, H, W, C / 8, reinterpret_cast<Bf16x8 *>(y));
-    else
-        avgpool_fwd_kernel<<<grid_for(n), 256, 0, s>>>(x, xs, xo, nimg, H, W, C, y);
+    avgpool_fwd8_kernel<<<row_grid(((W - 1) / 2 + 1) * (C / 8), nimg * ((H - 1) / 2 + 1)), 256, 0, s>>>(
+        x, xs, xo, nimg, H, W, C / 8, reinterpret_cast<Bf16x8 *>(y));
 }
-void launch_avgpool_bwd(const float *dy, int nimg, int H, int W, int C, float *dx, int accumulate, cudaStream_t s) {
-    const long long n = (long long)nimg * H * W * C;
-    if (C % 4 == 0 && (((uintptr_t)dy | (uintptr_t)dx) & 15) == 0)
-        avgpool_bwd4_kernel<<<grid_for(n / 4), 256, 0, s>>>(dy, nimg, H, W, C / 4, dx, accumulate);
-    else
-        avgpool_bwd_kernel<<<grid_for(n), 256, 0, s>>>(dy, nimg, H, W, C, dx, accumulate);
-}
-bool launch_split_cat(const float *src, int nimg, int H, int W, int C, float *skip, __nv_bfloat16 *up,
+void launch_split_cat(const float *src, int nimg, int H, int W, int C, float *skip, __nv_bfloat16 *up,
                       cudaStream_t s) {
-    if (C % 4 != 0 || (H | W) & 1 || (((uintptr_t)src | (uintptr_t)skip) & 15) != 0 || ((uintptr_t)up & 7) != 0)
-        return false;
-    const long long P = (long long)nimg * H * W;
-    split_cat4_kernel<<<row_grid(W * (C / 4), nimg * H), 256, 0, s>>>(src, nimg, H, W, C / 4,
-                                                                      reinterpret_cast<float4 *>(skip),
-                                                          reinterpret_cast<Bf16x4 *>(up));
-    return true;
+    split_cat4_kernel<<<row_grid(W * (C / 4), nimg * H), 256, 0, s>>>(
+        src, nimg, H, W, C / 4, reinterpret_cast<float4 *>(skip), reinterpret_cast<Bf16x4 *>(up));
 }
 void launch_to_bf16_s2d(const float *x, int nimg, int H, int W, int C, __nv_bfloat16 *y, cudaStream_t s) {
     to_bf16_s2d_kernel<<<grid_for((long long)nimg * 4 * H * W * C), 256, 0, s>>>(x, nimg, H, W, C, y);
 }
-bool launch_avgpool_bwd_leaky(const float *dy, int nimg, int H, int W, int C, const float *skip,
+void launch_avgpool_bwd_leaky(const float *dy, int nimg, int H, int W, int C, const float *skip,
                               const __nv_bfloat16 *act, int as, int ao, float slope, __nv_bfloat16 *g,
                               cudaStream_t s) {
-    if (C % 8 != 0 || ((as | ao) & 7) != 0 ||
-        (((uintptr_t)dy | (uintptr_t)skip | (uintptr_t)act | (uintptr_t)g) & 15) != 0)
-        return false;
     avgpool_bwd_leaky8_kernel<<<row_grid(W * (C / 8), nimg * H), 256, 0, s>>>(
         reinterpret_cast<const float4 *>(dy), nimg, H, W, C / 8, reinterpret_cast<const float4 *>(skip), act, as, ao,
         slope, reinterpret_cast<Bf16x8 *>(g));
-    return true;
-}
-void launch_leaky_bwd(const float *dA, const __nv_bfloat16 *a, int as, int ao, long long P, int C, float slope,
-                      __nv_bfloat16 *g, cudaStream_t s) {
-    if (C % 4 == 0 && ((as | ao) & 3) == 0 && (((uintptr_t)a | (uintptr_t)g) & 7) == 0 && ((uintptr_t)dA & 15) == 0)
-        leaky_bwd4_kernel<<<grid_for(P * C / 4), 256, 0, s>>>(reinterpret_cast<const float4 *>(dA), a, as, ao, P,
-                                                              C / 4, slope, reinterpret_cast<Bf16x4 *>(g));
-    else
-        leaky_bwd_kernel<<<grid_for(P * C), 256, 0, s>>>(dA, a, as, ao, P, C, slope, g);
-}
-void launch_f32_to_bf16_slice(const float *x, int xs, int xo, long long P, int C, __nv_bfloat16 *y, cudaStream_t s) {
-    if (C % 4 == 0 && ((xs | xo) & 3) == 0 && ((uintptr_t)x & 15) == 0 && ((uintptr_t)y & 7) == 0)
-        f32_to_bf16_slice4_kernel<<<grid_for(P * C / 4), 256, 0, s>>>(x, xs, xo, P, C / 4,
-                                                                      reinterpret_cast<Bf16x4 *>(y));
-    else
-        f32_to_bf16_slice_kernel<<<grid_for(P * C), 256, 0, s>>>(x, xs, xo, P, C, y);
-}
-void launch_add_slice(const float *src, int ss, int so, long long P, int C, float *dst, cudaStream_t s) {
-    if (C % 4 == 0 && ((ss | so) & 3) == 0 && (((uintptr_t)src | (uintptr_t)dst) & 15) == 0)
-        add_slice4_kernel<<<grid_for(P * C / 4), 256, 0, s>>>(src, ss, so, P, C / 4, reinterpret_cast<float4 *>(dst));
-    else
-        add_slice_kernel<<<grid_for(P * C), 256, 0, s>>>(src, ss, so, P, C, dst);
 }
 void launch_conv1x1_fwd(const __nv_bfloat16 *a, int C, long long P, const __nv_bfloat16 *w, const float *b, float *out,
                         cudaStream_t s) {

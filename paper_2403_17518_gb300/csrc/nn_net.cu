@@ -595,15 +595,12 @@ void after_wgrad(NetState &N, const void *g) {
     }
 }
 
-// Backward of one conv + LeakyReLU block: dA (float, dense [P][co]) is the
-// gradient of its output a; x its (bf16) input.  Writes the weight and bias
-// gradients and, when dx != nullptr, the input gradient (float [P][ci]).
-// The layer's output gradient g (bf16) is either computed here from dA
-// (f32) and the layer's activation a, or given as g_in (already computed by
-// the previous block's fused epilogue).  The input gradient goes to dx (f32),
-// or, when next_g is set, straight into the next block's g: times the
-// LeakyReLU derivative of next_act, the input x's activation (the two give
-// the same bits as storing dx and running the activation backward after).
+// Backward of one conv + LeakyReLU block from its output gradient g (bf16, the
+// activation's derivative applied); x is its (bf16) input.  Writes the weight and
+// bias gradients and, when dx != nullptr, the input gradient (float [P][ci]), or,
+// when next.g is set, puts it straight into the next block's g: times the LeakyReLU
+// derivative of next.act, the input x's activation (the same bits as storing dx and
+// running the activation backward after).
 struct FuseNext {
     const __nv_bfloat16 *act = nullptr;
     int stride = 0, off = 0;
@@ -619,19 +616,11 @@ struct SplitCat {
     bool *done = nullptr;
 };
 
-void block_bwd(NetState &N, int li, const float *dA, const __nv_bfloat16 *a, int as, int ao, const __nv_bfloat16 *x,
-               int xs, int xo, int ci, int nimg, int H, int W, float *dx, cudaStream_t s,
-               const __nv_bfloat16 *g_in = nullptr, const FuseNext &next = FuseNext(),
+void block_bwd(NetState &N, int li, const __nv_bfloat16 *g, const __nv_bfloat16 *x, int xs, int xo, int ci, int nimg,
+               int H, int W, float *dx, cudaStream_t s, const FuseNext &next = FuseNext(),
                const SplitCat &cat = SplitCat()) {
     const LayerDesc &d = N.L[li];
     const long long P = (long long)nimg * H * W;
-    const __nv_bfloat16 *g = g_in;
-    if (!g) {
-        before_gbuf_write(N, N.V.gbuf, s);
-        launch_leaky_bwd(dA, a, as, ao, P, d.co, 0.2f, N.V.gbuf, s);
-        g = N.V.gbuf;
-        N.launches++;
-    }
     fork_wgrad(N, s);
     const cudaStream_t ws = wgrad_stream(N, s);
     WgradArgs w{};
@@ -764,14 +753,13 @@ void backward_impl(NetState &N, int n, int H, int W, cudaStream_t s) {
     launch_conv1x1_bwd_leaky(gout, V.dec1[0], P0, C(0), N.w16 + dout.off, 0.2f, V.gbuf, N.red_part, RED_BLOCKS,
                              N.grad + dout.off, s);
     N.launches += 2;
-    float *dA = V.dA, *dB = V.dB;
+    float *dA = V.dA;
     // The two gradient buffers take turns: g holds the output gradient of the
     // block at hand, other receives the next one's.
     __nv_bfloat16 *g = V.gbuf, *other = V.gbuf2;
     for (int l = Lv; l >= 1; l--) {
         const int r = Lv - l;
         const int Hr = H >> r, Wr = W >> r;
-        const long long Pr = (long long)n * Hr * Wr;
         // up_l.1: output dec1, input dec0, its output gradient in g (from the
         // output layer's or the transposed conv's backward); its input gradient
         // goes straight into up_l.0's (dec0's activation backward fused).
@@ -779,9 +767,8 @@ void backward_impl(NetState &N, int n, int H, int W, cudaStream_t s) {
         fu.act = V.dec0[r];
         fu.stride = C(r);
         fu.g = other;
-        block_bwd(N, layer_index_up(N, l, 2), nullptr, nullptr, 0, 0, V.dec0[r], C(r), 0, C(r), n, Hr, Wr, nullptr, s,
-                  g, fu);
-        // up_l.0: output dec0, input cat (2C).  d(cat) [Pr][2C] is split into the
+        block_bwd(N, layer_index_up(N, l, 2), g, V.dec0[r], C(r), 0, C(r), n, Hr, Wr, nullptr, s, fu);
+        // up_l.0: output dec0, input cat (2C).  d(cat) is split into the
         // skip half, kept, and the upsampled half in bf16 and space-to-depth
         // layout on the coarse grid (the transposed conv's gradients are then
         // one-tap GEMMs): by the GEMM's epilogue, or in a pass over d(cat).
@@ -790,17 +777,12 @@ void backward_impl(NetState &N, int n, int H, int W, cudaStream_t s) {
         cat.skip = V.dskip[r];
         cat.up = g;
         cat.done = &split;
-        block_bwd(N, layer_index_up(N, l, 1), nullptr, nullptr, 0, 0, V.cat[r], 2 * C(r), 0, 2 * C(r), n, Hr, Wr, dA,
-                  s, other, FuseNext(), cat);
-        before_gbuf_write(N, g, s);
-        const bool s2d = split || launch_split_cat(dA, n, Hr, Wr, C(r), V.dskip[r], g, s);
-        if (s2d) {
-            N.launches += split ? 0 : 1;
-        } else {
-            cudaMemsetAsync(V.dskip[r], 0, sizeof(float) * Pr * C(r), s);
-            launch_add_slice(dA, 2 * C(r), 0, Pr, C(r), V.dskip[r], s);
-            launch_f32_to_bf16_slice(dA, 2 * C(r), C(r), Pr, C(r), g, s);
-            N.launches += 2;
+        block_bwd(N, layer_index_up(N, l, 1), other, V.cat[r], 2 * C(r), 0, 2 * C(r), n, Hr, Wr, dA, s, FuseNext(),
+                  cat);
+        if (!split) {
+            before_gbuf_write(N, g, s);
+            launch_split_cat(dA, n, Hr, Wr, C(r), V.dskip[r], g, s);
+            N.launches++;
         }
         // Transposed conv: input is the level-(r+1) activation.
         const int li = layer_index_up(N, l, 0);
@@ -810,8 +792,8 @@ void backward_impl(NetState &N, int n, int H, int W, cudaStream_t s) {
         WgradArgs w{};
         w.mode = WG_CONVT;
         w.g = g;
-        w.g_stride = s2d ? 4 * C(r) : C(r);
-        w.g_s2d = s2d;
+        w.g_stride = 4 * C(r);
+        w.g_s2d = true;
         w.x = xin;
         w.x_stride = C(r + 1);
         w.x_off = 0;
@@ -833,26 +815,14 @@ void backward_impl(NetState &N, int n, int H, int W, cudaStream_t s) {
         FpropArgs a{};
         a.src = g;
         a.src_off = 0;
-        if (s2d) {  // input gradient: the one-tap GEMM over the 4 C(r) space-to-depth channels
-            a.src_stride = 4 * C(r);
-            a.Hs = Hc;
-            a.Ws = Wc;
-            a.C = 4 * C(r);
-            a.ntaps = 1;
-            a.scale = 1;
-            a.dh[0] = a.dw[0] = 0;
-        } else {
-            a.src_stride = C(r);
-            a.Hs = Hr;
-            a.Ws = Wr;
-            a.C = C(r);
-            a.ntaps = 4;
-            a.scale = 2;
-            for (int t = 0; t < 4; t++) {
-                a.dh[t] = t >> 1;
-                a.dw[t] = t & 1;
-            }
-        }
+        // Input gradient: the one-tap GEMM over the 4 C(r) space-to-depth channels.
+        a.src_stride = 4 * C(r);
+        a.Hs = Hc;
+        a.Ws = Wc;
+        a.C = 4 * C(r);
+        a.ntaps = 1;
+        a.scale = 1;
+        a.dh[0] = a.dw[0] = 0;
         a.Ho = Hc;
         a.Wo = Wc;
         a.M = n * Hc * Wc;
@@ -876,52 +846,30 @@ void backward_impl(NetState &N, int n, int H, int W, cudaStream_t s) {
         N.launches += 5;
         std::swap(g, other);
     }
-    // gin: the next block's output gradient (bf16, in g) when the pass before
-    // already produced it, as the last transposed conv did.
-    const __nv_bfloat16 *gin = g;
+    // The encoder: g holds the output gradient of the block at hand, which the
+    // last transposed conv's or the pool's backward produced.
     for (int r = Lv; r >= 1; r--) {
         const int Hr = H >> r, Wr = W >> r;
-        const long long Pr = (long long)n * Hr * Wr;
-        if (r < Lv && !gin) {
-            launch_add_slice(V.dskip[r], C(r), 0, Pr, C(r), dA, s);
-            N.launches++;
-        }
-        const __nv_bfloat16 *ar = r < Lv ? V.cat[r] : V.bottom;
-        const int ars = r < Lv ? 2 * C(r) : C(r);
         FuseNext fd;
         fd.act = V.tmp[r];
         fd.stride = C(r);
         fd.g = other;
-        block_bwd(N, layer_index_down(N, r, 1), gin ? nullptr : dA, ar, ars, 0, V.tmp[r], C(r), 0, C(r), n, Hr, Wr,
-                  nullptr, s, gin, fd);
-        block_bwd(N, layer_index_down(N, r, 0), nullptr, nullptr, 0, 0, V.pool[r], C(r - 1), 0, C(r - 1), n, Hr, Wr,
-                  dA, s, other);
+        block_bwd(N, layer_index_down(N, r, 1), g, V.tmp[r], C(r), 0, C(r), n, Hr, Wr, nullptr, s, fd);
+        block_bwd(N, layer_index_down(N, r, 0), other, V.pool[r], C(r - 1), 0, C(r - 1), n, Hr, Wr, dA, s);
         // Level r-1's output gradient: the pool's backward of dA plus the skip
         // gradient, times the LeakyReLU derivative of that output (cat[r-1]'s
         // first half), straight to bf16 for the next block.
         before_gbuf_write(N, g, s);
-        if (launch_avgpool_bwd_leaky(dA, n, H >> (r - 1), W >> (r - 1), C(r - 1), V.dskip[r - 1], V.cat[r - 1],
-                                     2 * C(r - 1), 0, 0.2f, g, s)) {
-            gin = g;
-        } else {
-            launch_avgpool_bwd(dA, n, H >> (r - 1), W >> (r - 1), C(r - 1), dB, 0, s);
-            std::swap(dA, dB);
-            gin = nullptr;
-            g = V.gbuf;  // (where block_bwd puts an output gradient it computes itself)
-            other = V.gbuf2;
-        }
-        N.launches++;
-    }
-    if (!gin) {
-        launch_add_slice(V.dskip[0], C(0), 0, P0, C(0), dA, s);
+        launch_avgpool_bwd_leaky(dA, n, H >> (r - 1), W >> (r - 1), C(r - 1), V.dskip[r - 1], V.cat[r - 1],
+                                 2 * C(r - 1), 0, 0.2f, g, s);
         N.launches++;
     }
     FuseNext f0;
     f0.act = V.a_inc0;
     f0.stride = C(0);
     f0.g = other;
-    block_bwd(N, 1, gin ? nullptr : dA, V.cat[0], 2 * C(0), 0, V.a_inc0, C(0), 0, C(0), n, H, W, nullptr, s, gin, f0);
-    block_bwd(N, 0, nullptr, nullptr, 0, 0, V.xin, CPAD, 0, CPAD, n, H, W, nullptr, s, other);
+    block_bwd(N, 1, g, V.a_inc0, C(0), 0, C(0), n, H, W, nullptr, s, f0);
+    block_bwd(N, 0, other, V.xin, CPAD, 0, CPAD, n, H, W, nullptr, s);
 }
 
 // Loss of the current batch: MSE against yf; writes g_out (bf16) to the
