@@ -75,3 +75,37 @@ def test_launches_take_many_pairs(monkeypatch):
     ctx.model_shots(to_dev(v), f32_geom(c.geom))
     assert ctx.stats()["kernel_launches"] == 3
     ctx.close()
+
+
+def test_two_contexts_at_once():
+    """Two threads, each with its own context and stream: the launches of one neither
+    wait for nor disturb the other's."""
+    import threading
+
+    import torch
+
+    c, v, _ = _case(56)
+    g = f32_geom(c.geom)
+    out = {}
+
+    def work(k, rounds):
+        ctx = gpu_ctx(c)
+        with torch.cuda.stream(torch.cuda.Stream()):
+            vd = to_dev(v)
+            for _ in range(rounds):
+                d = ctx.model_shots(vd, g)
+                J, grad = ctx.fwi_gradient(vd, g, 0.5 * d)
+                b = ctx.born_demig(vd, g, 0.01 * vd)
+            torch.cuda.current_stream().synchronize()
+            out[k] = [x.cpu().numpy() for x in (d, grad, b)] + [J]
+        ctx.close()
+
+    work("alone", 1)
+    threads = [threading.Thread(target=work, args=(k, 3)) for k in ("a", "b")]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for k in ("a", "b"):
+        for x, y in zip(out["alone"], out[k]):
+            np.testing.assert_array_equal(x, y)
