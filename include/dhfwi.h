@@ -124,11 +124,14 @@ typedef struct {
      * either way. */
     int history_steps;
     long long history_cells;   /* phase-0 cell updates that also stored a^n */
-    /* Time steps (1 or 2) by which a tile of the forward and the adjoint
-     * sweeps advances at a time: the autotuner times both depths per geometry
-     * (of Born the form that reads the history; both fields together take 2);
-     * DHFWI_TIME_BLOCK=0 (environment) forces 1, any other value 2.  A launch of the two-step kernels covers many such pairs
-     * (kernel_launches and phase_launches count launches, not steps). */
+    /* Time steps (1 or 2) by which a tile of the forward [0] and the adjoint
+     * sweeps [1] advances at a time: the autotuner times both depths per
+     * geometry, and chooses those of Born (both fields, or the scattered one
+     * with the background from the history; not reported here) in the
+     * geometry's first Born call.  DHFWI_TIME_BLOCK=0 (environment) forces 1,
+     * any other value 2.  A two-step launch covers many pairs of steps where
+     * the plan has more tiles than are resident at once (kernel_launches and
+     * phase_launches count launches, not steps). */
     int time_block[2];
     /* What the last call took from the stored forward pass of an earlier
      * call (dhfwi_set_reuse): bit 0, rtm_mig skipped its forward pass; bit 1,

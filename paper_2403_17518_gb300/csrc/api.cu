@@ -708,8 +708,9 @@ int tune_depth(dhfwi_ctx *ctx, int first, int last, cudaStream_t st);
 // kind on the plan's full tile list (all shots active) using the scratch
 // field pools, and keep the fastest; then the time-blocking depth of the
 // sweeps (tune_depth).  The pools are zeroed again by the call that follows,
-// so tuning leaves no trace in the results.  Runs once per geometry; DHFWI_STEP_VARIANT=<0..6> pins a variant instead (and the depth
-// stays two unless DHFWI_TIME_BLOCK says otherwise).
+// so tuning leaves no trace in the results.  Runs once per geometry;
+// DHFWI_STEP_VARIANT=<0..6> pins a variant instead (and the depth stays two
+// unless DHFWI_TIME_BLOCK says otherwise).
 int autotune(dhfwi_ctx *ctx, cudaStream_t st) {
     const Plan &P = ctx->plan;
     if (ctx->tuned_hash == P.hash) return DHFWI_OK;

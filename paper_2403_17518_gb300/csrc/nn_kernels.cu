@@ -737,9 +737,9 @@ __global__ void avgpool_fwd8_kernel(const __nv_bfloat16 *__restrict__ x, int xs,
 
 // Backward of the pool, plus the skip gradient of the same activation, times the
 // LeakyReLU derivative of that activation (bf16 act, stride as, offset ao): the next
-// block's output gradient g in bf16, every step rounded to float32.  Eight channels per thread and the up to four windows' loads first:
-// 108.4 -> 80.0 us for the four launches of the size above (four channels, one
-// window at a time).
+// block's output gradient g in bf16, every step rounded to float32.  Eight channels
+// per thread and the up to four windows' loads first: 108.4 -> 80.0 us for the four
+// launches of the size above (four channels, one window at a time).
 __global__ void avgpool_bwd_leaky8_kernel(const float4 *__restrict__ dy, int nimg, int H, int W, int C8,
                                           const float4 *__restrict__ skip, const __nv_bfloat16 *__restrict__ act,
                                           int as, int ao, float slope, Bf16x8 *__restrict__ g) {
